@@ -38,7 +38,7 @@ struct Caps {
     int hcap;      // slots of the J -> position hash (power of two >= 2*pcap), 0 = none
     int small_p;   // largest |J| solved by the register-resident warp QR (0: never)
     int stage_bytes;  // shared memory for staging QR panels (global-memory bins), 0 = none
-    int append;       // CTA bins: keep the factor between loops and append to it (Section 3)
+    int append;       // CTA bins: room for the kept factor's positions (Section 3)
     int dcap;         // max number of distinct columns dropped from J (they are not charged again on re-entry)
     int spai;         // SPAI selection: a score per candidate column (scap of them)
 };
@@ -136,7 +136,8 @@ template <typename T> struct Work {
     }
 };
 
-enum ColStatus { COL_DONE = 0, COL_OVERFLOW = 1 };
+// COL_OVERFLOW_J: |J| outgrew the bin (a bin with the same |J| limit cannot take the column either)
+enum ColStatus { COL_DONE = 0, COL_OVERFLOW = 1, COL_OVERFLOW_J = 2 };
 
 // Entries of a CSR row loaded together in the row-driven loops
 constexpr int kRowGroup = 4;
@@ -264,45 +265,6 @@ __device__ __noinline__ int qr_factor_team(Team team, T *B, int q, int p, T *rhs
     int rank_flag = 0;
     for (int j = j_start; j < p; ++j) householder_step(team, B, q, p, rhs, vhead, taus, j, j + 1, small, rank_flag);
     return rank_flag;
-}
-
-// Compact-WY pieces shared by the panel factorization and the QR update.
-// V: nb explicit reflectors (zeros above the diagonal, heads on it) of
-// length qq in shared memory, ld qq; taus: their 2 / v^T v.  wy_form_T forms
-// T from V alone; the staged factorization forms it alongside instead
-// (panel_factor_fused), so wy_form_T has no caller at present.
-// T (kPanel x kPanel in tm) of H_0 ... H_{nb-1} = I - V T V^T:
-// y(s,t) = v_s^T v_t (s < t), then column by column
-// T(t,t) = tau_t, T(0:t, t) = -tau_t T(0:t, 0:t) y(0:t, t).
-template <class Team, typename T>
-__device__ __forceinline__ void wy_form_T(const Team &team, const T *V, int qq, int nb, const T *taus, T *tm) {
-    const int me = team.rank();
-    const int lane = me & 31, wid = me >> 5;
-    constexpr int NW = (Team::SIZE + 31) / 32;
-    for (int pair = wid; pair < nb * nb; pair += NW) {
-        const int s_ = pair / nb, t_ = pair - s_ * nb;
-        if (s_ >= t_) continue;
-        const T *vs = V + (int64_t)s_ * qq, *vt = V + (int64_t)t_ * qq;
-        T d = 0;
-        for (int r = t_ + lane; r < qq; r += 32) d += vs[r] * vt[r];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
-        if (lane == 0) tm[s_ * kPanel + t_] = d;
-    }
-    team.sync();
-    for (int t = 0; t < nb; ++t) {
-        const T tau = taus[t];
-        T val = T(0);
-        if (me < t) {
-            T acc = 0;
-            for (int s2 = me; s2 < t; ++s2) acc += tm[me * kPanel + s2] * tm[s2 * kPanel + t];
-            val = -tau * acc;
-        }
-        team.sync();
-        if (me < t) tm[me * kPanel + t] = val;
-        if (me == t) tm[t * kPanel + t] = tau;
-        team.sync();
-    }
 }
 
 // Columns c in [c_lo, c_hi] of B (ld q; c == p stands for rhs), rows
@@ -779,12 +741,12 @@ __device__ __noinline__ void apply_qt_panels(Team team, const T *B, int q, int p
 // does not fit four columns falls back to single Householder steps (panels of
 // one).  The reflectors, R and rhs are those of the unblocked version up to
 // rounding.  j_start > 0 factors only columns j_start..p-1 (the columns
-// appended to a factor whose first j_start columns are done, Section 3);
-// backsub = false leaves Q^T rhs in rhs.
+// appended to a factor whose first j_start columns are done, Section 3).
+// Leaves Q^T rhs in rhs.
 template <class Team, typename T>
 __device__ __noinline__ int qr_solve_staged(Team team, T *B, int q, int p, T *rhs, T *vhead, T *taus, T small,
                                             T *stage, int stage_bytes, T *Tst, int32_t *pnb,
-                                            int j_start = 0, bool backsub = true) {
+                                            int j_start) {
     const int me = team.rank();
     constexpr int NW = Team::SIZE / 32;
     T *tm = stage;                                  // kPanel x kPanel
@@ -837,7 +799,6 @@ __device__ __noinline__ int qr_solve_staged(Team team, T *B, int q, int p, T *rh
         wy_apply(team, V, qq, nb, tm, B, q, p, rhs, j0, j0 + nb, p);
         j0 += nb;
     }
-    if (backsub) back_substitute_blocked(team, B, q, p, rhs, small);
     return rank_flag;
 }
 
@@ -864,47 +825,55 @@ __device__ __noinline__ void apply_qt_team(Team team, const T *B, int q, int p, 
     else back_substitute_blocked(team, B, q, p, rhs, small);
 }
 
-// The QR update of Section 3, first half: the reflectors 0..p0-1 of a
-// finished factor (built on q0 rows; every row below is zero in them) applied
-// to the appended columns p0..p-1 of B (ld q), rows j..q0-1.  In the
-// global-memory bins (pnb != nullptr) the reflectors go panel by panel as
-// they were factored, each panel in compact-WY form with its stored T, split
-// into sub-panels when its explicit V outgrows the staging area (q has grown
-// since it was factored).  Sub-panels of fewer than four reflectors, and the
-// shared-memory bins, take one reflector per pass, one warp per column.
+// Reflector j (built on q0 rows) applied to the columns p0..p-1 of B (ld q),
+// one warp per column; ends with a team synchronisation.
 template <class Team, typename T>
-__device__ __noinline__ void qr_update_apply(Team team, T *B, int q, int p, int q0, int p0, const T *vhead,
-                                             const T *taus, T *stage, int stage_bytes, const T *Tst,
-                                             const int32_t *pnb) {
+__device__ __forceinline__ void update_one_reflector(const Team &team, T *B, int q, int p, int q0, int p0,
+                                                     const T *vhead, const T *taus, int j) {
     const int me = team.rank();
     const int lane = me & 31, wid = me >> 5;
     constexpr int NW = (Team::SIZE + 31) / 32;
+    const T *col = B + (int64_t)j * q;
+    const T v0 = vhead[j], two_over = taus[j];
+    if (two_over > T(0)) {
+        for (int c = p0 + wid; c < p; c += NW) {
+            T *t = B + (int64_t)c * q;
+            T d = 0;
+            for (int i = j + lane; i < q0; i += 32) d += ((i == j) ? v0 : col[i]) * t[i];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+            const T f = d * two_over;
+            for (int i = j + lane; i < q0; i += 32) t[i] -= f * ((i == j) ? v0 : col[i]);
+        }
+    }
+    team.sync();
+}
+
+// The QR update of Section 3, first half: the reflectors 0..p0-1 of a
+// finished factor (built on q0 rows; every row below is zero in them) applied
+// to the appended columns p0..p-1 of B (ld q), rows j..q0-1, panel by panel as
+// they were factored, each panel in compact-WY form with its stored T, split
+// into sub-panels when its explicit V outgrows the staging area (q has grown
+// since it was factored).  Sub-panels of fewer than four reflectors take one
+// reflector at a time.
+template <class Team, typename T>
+__device__ __noinline__ void qr_update_apply_staged(Team team, T *B, int q, int p, int q0, int p0, const T *vhead,
+                                                    const T *taus, T *stage, int stage_bytes, const T *Tst,
+                                                    const int32_t *pnb) {
+    const int me = team.rank();
     T *tm = stage;
     T *V = stage + kStageHead<Team>;
-    const int64_t velems = stage_bytes > 0 ? (int64_t)stage_bytes / (int64_t)sizeof(T) - kStageHead<Team> : 0;
+    const int64_t velems = (int64_t)stage_bytes / (int64_t)sizeof(T) - kStageHead<Team>;
     int j0 = 0;
     while (j0 < p0) {
-        const int nb = pnb ? pnb[j0] : 1;
+        const int nb = pnb[j0];
         // the panel in sub-panels of as many reflectors as the staging area holds:
         // the diagonal blocks of a panel's T are the T's of its sub-panels
         for (int js = 0; js < nb;) {
             const int j1 = j0 + js, qq = q0 - j1;
             const int ns = (int)min((int64_t)(nb - js), qq > 0 ? velems / (int64_t)qq : (int64_t)0);
-            if (ns < 4) {  // one reflector, one warp per column
-                const T *col = B + (int64_t)j1 * q;
-                const T v0 = vhead[j1], two_over = taus[j1];
-                if (two_over > T(0)) {
-                    for (int c = p0 + wid; c < p; c += NW) {
-                        T *t = B + (int64_t)c * q;
-                        T d = 0;
-                        for (int i = j1 + lane; i < q0; i += 32) d += ((i == j1) ? v0 : col[i]) * t[i];
-#pragma unroll
-                        for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
-                        const T f = d * two_over;
-                        for (int i = j1 + lane; i < q0; i += 32) t[i] -= f * ((i == j1) ? v0 : col[i]);
-                    }
-                }
-                team.sync();
+            if (ns < 4) {
+                update_one_reflector(team, B, q, p, q0, p0, vhead, taus, j1);
                 ++js;
                 continue;
             }
@@ -1202,28 +1171,29 @@ template <class Team, typename T> struct Column {
             }
         }
         if constexpr (!is_lane_team<Team>::value) {
-            const bool keep = cap.append != 0;  // keep Q^T e_k for later updates
-            if (cap.stage_bytes > 0 && p >= 2 * kPanel)
-                rank_flag = qr_solve_staged<Team, T>(team, w.B, q, p, w.rhs, w.vhead, w.tau, small, (T *)w.stage,
-                                                     cap.stage_bytes, w.Tst, w.pnb, 0, !keep);
-            else if (keep) {
+            // the CTA bins keep the factor, with Q^T e_k, for later updates
+            bool staged = false;
+            if constexpr (Team::STAGED) {
+                if (p >= 2 * kPanel) {
+                    staged = true;
+                    rank_flag = qr_solve_staged<Team, T>(team, w.B, q, p, w.rhs, w.vhead, w.tau, small, (T *)w.stage,
+                                                         cap.stage_bytes, w.Tst, w.pnb, 0);
+                }
+            }
+            if (!staged) {
                 rank_flag = qr_factor_team<Team, T>(team, w.B, q, p, w.rhs, w.vhead, w.tau, small, 0);
                 single_panels(0);
-            } else {
-                rank_flag = qr_solve_team<Team, T>(team, w.B, q, p, w.rhs, w.vhead, w.tau, small);
             }
-            if (keep) {
-                // a factor from scratch: factor order = sorted order
-                const int me = team.rank();
-                for (int i = me; i < q; i += Team::SIZE) {
-                    w.qte[i] = w.rhs[i];
-                    w.Ip[i] = i;
-                }
-                for (int c = me; c < p; c += Team::SIZE) w.Jp[c] = c;
-                team.sync();
-                back_substitute_blocked(team, w.B, q, p, w.rhs, small);
-                fact_valid = true;
+            // a factor from scratch: factor order = sorted order
+            const int me = team.rank();
+            for (int i = me; i < q; i += Team::SIZE) {
+                w.qte[i] = w.rhs[i];
+                w.Ip[i] = i;
             }
+            for (int c = me; c < p; c += Team::SIZE) w.Jp[c] = c;
+            team.sync();
+            back_substitute_blocked(team, w.B, q, p, w.rhs, small);
+            fact_valid = true;
             return;
         }
         rank_flag = qr_solve_team<Team, T>(team, w.B, q, p, w.rhs, w.vhead, w.tau, small);
@@ -1231,12 +1201,13 @@ template <class Team, typename T> struct Column {
 
     // Reflectors j0..p-1 factored one at a time: panels of one (global-memory bins)
     __device__ void single_panels(int j0) {
-        if (w.pnb == nullptr) return;
-        for (int j = j0 + team.rank(); j < p; j += Team::SIZE) {
-            w.pnb[j] = 1;
-            w.Tst[(int64_t)j * kPanel] = w.tau[j];
+        if constexpr (Team::STAGED) {
+            for (int j = j0 + team.rank(); j < p; j += Team::SIZE) {
+                w.pnb[j] = 1;
+                w.Tst[(int64_t)j * kPanel] = w.tau[j];
+            }
+            team.sync();
         }
-        team.sync();
     }
 
     // factor row of sorted I position i / factor column of sorted J position c
@@ -1257,13 +1228,10 @@ template <class Team, typename T> struct Column {
                 return;
             }
         }
-        if constexpr (!is_lane_team<Team>::value) {
-            if (w.pnb != nullptr) {
-                apply_qt_panels<Team, T>(team, w.B, q, p, w.rhs, w.vhead, w.Tst, w.pnb, (T *)w.stage,
-                                         cap.stage_bytes);
-                back_substitute_blocked(team, w.B, q, p, w.rhs, small);
-                return;
-            }
+        if constexpr (Team::STAGED) {
+            apply_qt_panels<Team, T>(team, w.B, q, p, w.rhs, w.vhead, w.Tst, w.pnb, (T *)w.stage, cap.stage_bytes);
+            back_substitute_blocked(team, w.B, q, p, w.rhs, small);
+            return;
         }
         apply_qt_team<Team, T>(team, w.B, q, p, w.rhs, w.vhead, w.tau, small);
     }
@@ -1290,30 +1258,43 @@ template <class Team, typename T> struct Column {
             // I can hold hundreds), summed by a fixed butterfly.  The global-memory
             // bins search a copy of J in the staging area (shared memory).
             const int32_t *Js = w.J;
-            if (cap.stage_bytes > 0 && (size_t)p * sizeof(int32_t) <= (size_t)cap.stage_bytes) {
-                int32_t *jc = reinterpret_cast<int32_t *>(w.stage);
-                for (int c = me; c < p; c += Team::SIZE) jc[c] = w.J[c];
-                Js = jc;
+            if constexpr (Team::STAGED) {
+                if ((size_t)p * sizeof(int32_t) <= (size_t)cap.stage_bytes) {
+                    int32_t *jc = reinterpret_cast<int32_t *>(w.stage);
+                    for (int c = me; c < p; c += Team::SIZE) jc[c] = w.J[c];
+                    Js = jc;
+                }
             }
             team.sync();
             const int lane = me & 31;
-            constexpr int NWR = Team::SIZE / 32;
-            for (int i = me >> 5; i < s; i += NWR) {
-                const int32_t row = w.S[i];
-                const int64_t e0 = A.row_ptr[row], e1 = A.row_ptr[row + 1];
-                double acc = 0.0;
-                for (int64_t e = e0 + lane; e < e1; e += 32) {
-                    const int pos = find_i32(Js, p, A.col_idx[e]);
-                    if (pos >= 0) { acc = fma(A.val[e], w.m[pos], acc); ++cnt; }
-                }
+            constexpr int NWR = Team::SIZE / 32, VK = Team::VK;
+            // squares of the rows of virtual warp (me >> 5) + NWR * v in ssv[v]: the same sums for every CTA size
+            double ssv[VK];
 #pragma unroll
-                for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-                if (row == k) acc -= 1.0;
-                if (lane == 0) {
-                    w.r[i] = acc;
-                    if (!refine) ss = fma(acc, acc, ss);
+            for (int v = 0; v < VK; ++v) ssv[v] = 0.0;
+            for (int i0 = me >> 5; i0 < s; i0 += NWR * VK) {
+#pragma unroll
+                for (int v = 0; v < VK; ++v) {
+                    const int i = i0 + NWR * v;
+                    if (i < s) {
+                        const int32_t row = w.S[i];
+                        const int64_t e0 = A.row_ptr[row], e1 = A.row_ptr[row + 1];
+                        double acc = 0.0;
+                        for (int64_t e = e0 + lane; e < e1; e += 32) {
+                            const int pos = find_i32(Js, p, A.col_idx[e]);
+                            if (pos >= 0) { acc = fma(A.val[e], w.m[pos], acc); ++cnt; }
+                        }
+#pragma unroll
+                        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+                        if (row == k) acc -= 1.0;
+                        if (lane == 0) {
+                            w.r[i] = acc;
+                            if (!refine) ssv[v] = fma(acc, acc, ssv[v]);
+                        }
+                    }
                 }
             }
+            if (!refine) rho = sqrt(team.sum_lane0(ssv));
         } else {
             team.sync();
             for (int i = me; i < s; i += Team::SIZE) {
@@ -1340,7 +1321,9 @@ template <class Team, typename T> struct Column {
             }
         }
         // the refinement step reads r only; its norm is not formed
-        if (!refine) rho = sqrt(team.sum(ss));
+        if constexpr (is_lane_team<Team>::value) {
+            if (!refine) rho = sqrt(team.sum(ss));
+        }
         long long nnzJ = team.sum(cnt);
         if (refine) c_ref64 += 2 * nnzJ + 2 * (long long)s;
         else c_res += 2 * nnzJ + 2 * (long long)s;
@@ -1543,12 +1526,19 @@ template <class Team, typename T> struct Column {
             if (ik < q && w.I[ik] == k && w.Ip[ik] >= qo) w.qte[w.Ip[ik]] = T(1);
         }
         team.sync();
-        qr_update_apply<Team, T>(team, w.B, q, p, qo, po, w.vhead, w.tau, (T *)w.stage, cap.stage_bytes, w.Tst,
-                                 w.pnb);
-        if (cap.stage_bytes > 0 && p >= 2 * kPanel) {
-            qr_solve_staged<Team, T>(team, w.B, q, p, w.qte, w.vhead, w.tau, small, (T *)w.stage, cap.stage_bytes,
-                                     w.Tst, w.pnb, po, false);
+        bool staged = false;
+        if constexpr (Team::STAGED) {
+            qr_update_apply_staged<Team, T>(team, w.B, q, p, qo, po, w.vhead, w.tau, (T *)w.stage, cap.stage_bytes,
+                                            w.Tst, w.pnb);
+            if (p >= 2 * kPanel) {
+                staged = true;
+                qr_solve_staged<Team, T>(team, w.B, q, p, w.qte, w.vhead, w.tau, small, (T *)w.stage,
+                                         cap.stage_bytes, w.Tst, w.pnb, po);
+            }
         } else {
+            for (int j = 0; j < po; ++j) update_one_reflector(team, w.B, q, p, qo, po, w.vhead, w.tau, j);
+        }
+        if (!staged) {
             qr_factor_team<Team, T>(team, w.B, q, p, w.qte, w.vhead, w.tau, small, po);
             single_panels(po);
         }
@@ -1965,7 +1955,7 @@ template <class Team, typename T> struct Column {
             // general path below
             long long b = 0;
             const int len = pattern_of_column(team, A.col_ptr, A.row_idx, k, cap.pcap, w.J, &b);
-            if (len < 0) return COL_OVERFLOW;
+            if (len < 0) return COL_OVERFLOW_J;
             p = len;
             c_bytes += b;
         } else {
@@ -2004,7 +1994,7 @@ template <class Team, typename T> struct Column {
                     if (na == 0) break;  // no candidate: nothing can be added later either
                     ++l;
                     note_bytes_columns(0, na, w.buf);
-                    if (!merge_J(na)) return COL_OVERFLOW;
+                    if (!merge_J(na)) return COL_OVERFLOW_J;
                     grown = true;
                     continue;
                 }
@@ -2021,7 +2011,7 @@ template <class Team, typename T> struct Column {
                 ++l;
                 if (nj == 0) continue;  // empty Jhat: back to the loop test (Algorithm 1)
                 note_bytes_columns(0, nj, w.buf);
-                if (!merge_J(nj)) return COL_OVERFLOW;
+                if (!merge_J(nj)) return COL_OVERFLOW_J;
                 grown = true;
             }
             if (!grown) break;

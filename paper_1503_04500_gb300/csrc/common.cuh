@@ -97,6 +97,8 @@ struct ColQueue {
     int32_t *ovf_cols;        // where columns that outgrow the bin go
     uint32_t *ovf_count;
     int64_t ovf_cap;
+    int32_t *wide_cols;       // columns whose |J| outgrows the bin (NULL: ovf_cols)
+    uint32_t *wide_count;
 };
 
 // ----------------------------------------------------------------------------
@@ -141,6 +143,7 @@ __device__ __forceinline__ bool dom_before(long long a, int i, long long b, int 
 struct HalfTeam {
     static constexpr int SIZE = 16;
     static constexpr int LANES = 16;
+    static constexpr bool STAGED = false;
     unsigned mask;  // this half's lanes
     __device__ __forceinline__ HalfTeam() : mask(0xffffu << (threadIdx.x & 16)) {}
     __device__ __forceinline__ int rank() const { return threadIdx.x & 15; }
@@ -186,6 +189,7 @@ struct HalfTeam {
 struct WarpTeam {
     static constexpr int SIZE = 32;
     static constexpr int LANES = 32;
+    static constexpr bool STAGED = false;
     static constexpr unsigned mask = 0xffffffffu;
     __device__ __forceinline__ int rank() const { return threadIdx.x & 31; }
     __device__ __forceinline__ void sync() const { __syncwarp(); }
@@ -229,12 +233,21 @@ struct WarpTeam {
     }
 };
 
-// A whole CTA of NT threads; `red` is NT/32+1 words of shared scratch (8 bytes
-// each, holding any reduced type), `redi` as many ints.
-template <int NT> struct BlockTeam {
+// A whole CTA of NT threads; `red` is kVirtualWarps+1 words of shared scratch
+// (8 bytes each, holding any reduced type), `redi` as many ints.  STAGED: the
+// bin stages panels in shared memory (its workspace is in global memory).
+//
+// Every CTA size gives the same bits: a float reduction over rows or columns
+// takes one element per thread (the smaller CTAs hold problems of at most NT
+// rows and columns), so it is the same per-warp butterflies, added over the
+// warps in order; the absent warps of a smaller CTA would add zeros.
+constexpr int kVirtualWarps = 16;
+template <int NT, bool STAGED_ = false> struct BlockTeam {
     static constexpr int SIZE = NT;
     static constexpr int LANES = 32;
     static constexpr int NW = NT / 32;
+    static constexpr bool STAGED = STAGED_;
+    static_assert(NW <= kVirtualWarps && kVirtualWarps % NW == 0, "warps per CTA");
     unsigned long long *red;
     int *redi;
     __device__ __forceinline__ int rank() const { return threadIdx.x; }
@@ -255,6 +268,21 @@ template <int NT> struct BlockTeam {
         V s = slot<V>(0);
 #pragma unroll
         for (int w = 1; w < NW; ++w) s += slot<V>(w);
+        return s;
+    }
+    // sum of the values that lane 0 of each of kVirtualWarps warps would hold:
+    // this warp holds those of warps wid, wid + NW, ...; added in warp order
+    static constexpr int VK = kVirtualWarps / NW;
+    template <typename V> __device__ __forceinline__ V sum_lane0(const V (&x)[VK]) const {
+        __syncthreads();
+        if ((threadIdx.x & 31) == 0) {
+#pragma unroll
+            for (int v = 0; v < VK; ++v) slot<V>((threadIdx.x >> 5) + NW * v) = x[v];
+        }
+        __syncthreads();
+        V s = slot<V>(0);
+#pragma unroll
+        for (int w = 1; w < kVirtualWarps; ++w) s += slot<V>(w);
         return s;
     }
     template <typename V> __device__ __forceinline__ V maxv(V x) const {

@@ -6,6 +6,10 @@
 namespace rsai {
 
 constexpr int kBlockThreads = 512;  // CTA team size of bins C and G (measured: 1.3x faster than 256)
+// Bin S: |I| <= 128 (one row per thread), several CTAs per SM
+constexpr int kSmallThreads = 128;
+template <typename T> constexpr int kSmallCtas = sizeof(T) == 8 ? 3 : 5;
+enum { CTA_BIN_SMALL = 0, CTA_BIN_SHARED = 1, CTA_BIN_GLOBAL = 2 };
 constexpr int kWarpsPerCta = 4;     // warps per CTA in bin W
 constexpr int kStatBlocks = 256;    // blocks of the per-column statistics reduction
 // Column counts per bin in the global counters (after the CTR_COUNT work
@@ -61,9 +65,26 @@ cudaError_t launch_bin_warp(int mode, bool fp32, int grid, int warps, const DevA
 cudaError_t launch_bin_half(int mode, bool fp32, int grid, int warps, const DevA &A, const DevParams &P,
                             const Caps &cap, const ColQueue &Q, const ColOut &O, const Frozen &F,
                             unsigned long long *gctr, bool last, cudaStream_t st);
-cudaError_t launch_bin_block(int mode, bool fp32, int grid, const DevA &A, const DevParams &P, const Caps &cap,
-                             const ColQueue &Q, const ColOut &O, const Frozen &F, unsigned long long *gctr,
-                             bool last, char *gwork, size_t gstride, int bin, cudaStream_t st);
+cudaError_t launch_bin_block(int mode, bool fp32, int kind, int grid, const DevA &A, const DevParams &P,
+                             const Caps &cap, const ColQueue &Q, const ColOut &O, const Frozen &F,
+                             unsigned long long *gctr, bool last, char *gwork, size_t gstride, int bin,
+                             cudaStream_t st);
+// per precision (warp_bins_f32.cu, warp_bins_f64.cu, cta_bins_f32.cu, cta_bins_f64.cu)
+template <typename T>
+cudaError_t launch_warp_t(int mode, int grid, int warps, const DevA &A, const DevParams &P, const Caps &cap,
+                          const ColQueue &Q, const ColOut &O, const Frozen &F, unsigned long long *gctr, bool last,
+                          cudaStream_t st);
+template <typename T>
+cudaError_t launch_half_t(int mode, int grid, int warps, const DevA &A, const DevParams &P, const Caps &cap,
+                          const ColQueue &Q, const ColOut &O, const Frozen &F, unsigned long long *gctr, bool last,
+                          cudaStream_t st);
+template <typename T>
+cudaError_t launch_block_t(int mode, int kind, int grid, const DevA &A, const DevParams &P, const Caps &cap,
+                           const ColQueue &Q, const ColOut &O, const Frozen &F, unsigned long long *gctr, bool last,
+                           char *gwork, size_t gstride, int bin, cudaStream_t st);
+template <typename T> int occupancy_warp_t(int warps, const Caps &cap);
+template <typename T> int occupancy_half_t(int warps, const Caps &cap);
+template <typename T> int occupancy_block_t(int kind, const Caps &cap);
 cudaError_t launch_adjoint_gather(int64_t n, int64_t nnzM, const int64_t *row_ptr, const int32_t *col_idx,
                                   const int64_t *Mrowptr, const int32_t *Mcols, const int64_t *Mcsc_to_csr,
                                   int64_t *Mcsr_to_csc, const int64_t *qoff, const int32_t *poolI,
@@ -71,7 +92,7 @@ cudaError_t launch_adjoint_gather(int64_t n, int64_t nnzM, const int64_t *row_pt
                                   const double *xM, double *grad, cudaStream_t st);
 int occupancy_bin_warp(bool fp32, int warps, const Caps &cap);
 int occupancy_bin_half(bool fp32, int warps, const Caps &cap);
-int occupancy_bin_block(bool fp32, const Caps &cap, bool global_work);
+int occupancy_bin_block(bool fp32, int kind, const Caps &cap);
 
 // apply / solver kernels (apply_kernels.cu)
 cudaError_t launch_spmv(int64_t n, const int64_t *row_ptr, const int32_t *col_idx, const double *val,

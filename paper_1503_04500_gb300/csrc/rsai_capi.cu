@@ -65,10 +65,11 @@ struct rsai_handle {
     long long *bnc = nullptr, *bnnz = nullptr;
     int32_t *err = nullptr;
     // [0..3] queue counters of bins W, W2, C, G; [4..6] overflow counts W->W2,
-    // W2->C, C->G; [7] columns of a pool-overflow rerun; [8] queue counter of
-    // bin H, [9] overflow count H->W
+    // S->C, C->G; [7] columns of a pool-overflow rerun; [8] queue counter of
+    // bin H, [9] overflow count H->W; [10] queue counter of bin S, [11]
+    // columns forwarded to it (W and W2)
     uint32_t *qnext = nullptr;
-    int32_t *ovf0 = nullptr, *ovf1 = nullptr, *ovf2 = nullptr, *ovf3 = nullptr;
+    int32_t *ovf0 = nullptr, *ovf1 = nullptr, *ovf2 = nullptr, *ovf3 = nullptr, *ovf_s = nullptr;
     int32_t *ovf3_sorted = nullptr;  // the global bin's queue, largest column first
     uint8_t *cost_bucket = nullptr;
     uint32_t *cost_hist = nullptr;   // [kCostBuckets]
@@ -93,8 +94,8 @@ struct rsai_handle {
     size_t gstride = 0;
     int grid_g = 0;
     // bins
-    Caps capH{}, capW{}, capW2{}, capC{}, capG{};
-    int grid_h = 0, grid_w = 0, grid_w2 = 0, warps_w2 = 0, grid_c = 0;
+    Caps capH{}, capW{}, capW2{}, capS{}, capC{}, capG{};
+    int grid_h = 0, grid_w = 0, grid_w2 = 0, warps_w2 = 0, grid_s = 0, grid_c = 0;
     rsai_tuning tuning{8, 0, kSmallP, 0, 0};
     // refit / backward scratch (allocated on first use)
     double *fval = nullptr, *fcval = nullptr;
@@ -245,19 +246,22 @@ cudaError_t enqueue_bins(rsai_handle *h, int mode, const DevA &A, const Frozen &
                          const int32_t *wlist = nullptr, const uint32_t *wcount = nullptr) {
     const int64_t n = h->n;
     cudaMemsetAsync(h->qnext, 0, sizeof(uint32_t) * 7, st);  // queue and overflow counters; [7] = retry count
-    cudaMemsetAsync(h->qnext + 8, 0, sizeof(uint32_t) * 2, st);
+    cudaMemsetAsync(h->qnext + 8, 0, sizeof(uint32_t) * 4, st);
     const DevParams P = dev_params(h);
     const bool fp32 = h->params.precision == RSAI_FP32_REFINE;
     ColOut O{h->col_off, h->col_len, h->col_q, h->rho, h->loops, h->flags, h->pool_rows, h->pool_vals,
              h->pool_cap, h->pool_top, h->err};
     // the first bin (H or W) takes the given list (or every column)
     const bool use_h = h->tuning.half_bin != 0;
-    ColQueue QH{wlist, wcount, n, h->qnext + 8, h->ovf0, h->qnext + 9, h->ovf_cap};
-    ColQueue QW = use_h ? ColQueue{h->ovf0, h->qnext + 9, n, h->qnext + 0, h->ovf1, h->qnext + 4, h->ovf_cap}
-                        : ColQueue{wlist, wcount, n, h->qnext + 0, h->ovf1, h->qnext + 4, h->ovf_cap};
-    ColQueue QW2{h->ovf1, h->qnext + 4, n, h->qnext + 1, h->ovf2, h->qnext + 5, h->ovf_cap};
-    ColQueue QC{h->ovf2, h->qnext + 5, n, h->qnext + 2, h->ovf3, h->qnext + 6, h->ovf_cap};
-    ColQueue QG{h->ovf3_sorted, h->qnext + 6, n, h->qnext + 3, nullptr, nullptr, 0};
+    ColQueue QH{wlist, wcount, n, h->qnext + 8, h->ovf0, h->qnext + 9, h->ovf_cap, nullptr, nullptr};
+    // a column whose |J| outgrows W skips W2, which has the same limit on |J|
+    // and would run it to the same point
+    ColQueue QW{use_h ? h->ovf0 : wlist, use_h ? h->qnext + 9 : wcount, n, h->qnext + 0, h->ovf1, h->qnext + 4,
+                h->ovf_cap, h->ovf_s, h->qnext + 11};
+    ColQueue QW2{h->ovf1, h->qnext + 4, n, h->qnext + 1, h->ovf_s, h->qnext + 11, h->ovf_cap, nullptr, nullptr};
+    ColQueue QS{h->ovf_s, h->qnext + 11, n, h->qnext + 10, h->ovf2, h->qnext + 5, h->ovf_cap, nullptr, nullptr};
+    ColQueue QC{h->ovf2, h->qnext + 5, n, h->qnext + 2, h->ovf3, h->qnext + 6, h->ovf_cap, nullptr, nullptr};
+    ColQueue QG{h->ovf3_sorted, h->qnext + 6, n, h->qnext + 3, nullptr, nullptr, 0, nullptr, nullptr};
     if (ev) cudaEventRecord(ev[1], st);
     cudaError_t e = cudaSuccess;
     if (use_h) {
@@ -269,7 +273,11 @@ cudaError_t enqueue_bins(rsai_handle *h, int mode, const DevA &A, const Frozen &
     e = launch_bin_warp(mode, fp32, h->grid_w2, h->warps_w2, A, P, h->capW2, QW2, O, F, gctr, false, st);
     if (e != cudaSuccess) return e;
     if (ev) cudaEventRecord(ev[2], st);
-    e = launch_bin_block(mode, fp32, h->grid_c, A, P, h->capC, QC, O, F, gctr, false, nullptr, 0, 1, st);
+    e = launch_bin_block(mode, fp32, CTA_BIN_SMALL, h->grid_s, A, P, h->capS, QS, O, F, gctr, false, nullptr, 0, 1,
+                         st);
+    if (e != cudaSuccess) return e;
+    e = launch_bin_block(mode, fp32, CTA_BIN_SHARED, h->grid_c, A, P, h->capC, QC, O, F, gctr, false, nullptr, 0, 1,
+                         st);
     if (e != cudaSuccess) return e;
     if (before_global) {
         const int hr = before_global(h, st);
@@ -284,7 +292,7 @@ cudaError_t enqueue_bins(rsai_handle *h, int mode, const DevA &A, const Frozen &
     k_cost_scatter<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(h->ovf3, h->qnext + 6, h->cost_bucket, h->cost_hist,
                                                                  h->ovf3_sorted);
     if (ev) cudaEventRecord(ev[3], st);
-    e = launch_bin_block(mode, fp32, h->grid_g, A, P, h->capG, QG, O, F, gctr, true, h->gwork, h->gstride, 2, st);
+    e = launch_bin_block(mode, fp32, CTA_BIN_GLOBAL, h->grid_g, A, P, h->capG, QG, O, F, gctr, true, h->gwork, h->gstride, 2, st);
     return e;
 }
 
@@ -297,7 +305,7 @@ cudaError_t enqueue_build(rsai_handle *h, cudaStream_t st, cudaEvent_t *ev = nul
     if (ev) cudaEventRecord(ev[0], st);
     cudaMemsetAsync(h->dscal, 0, sizeof(unsigned long long) * kScalars, st);
     cudaMemsetAsync(h->err, 0, sizeof(int32_t), st);
-    cudaMemsetAsync(h->qnext, 0, sizeof(uint32_t) * 10, st);
+    cudaMemsetAsync(h->qnext, 0, sizeof(uint32_t) * 12, st);
     cudaMemsetAsync(h->pool_top, 0, sizeof(unsigned long long), st);
     cudaMemsetAsync(h->row_count, 0, sizeof(int32_t) * (size_t)n, st);
     cudaMemsetAsync(h->cursor, 0, sizeof(int32_t) * (size_t)n, st);
@@ -386,7 +394,7 @@ int plan_h(rsai_handle *h, bool fp32) {
         if (rc_ != RSAI_OK) return rc_;    \
     } while (0)
 
-// choose the capacities of the five bins from the device limits
+// choose the capacities of the six bins from the device limits
 int plan_bins(rsai_handle *h) {
     const bool fp32 = h->params.precision == RSAI_FP32_REFINE;
     int dev = h->device, max_optin = 0;
@@ -406,6 +414,13 @@ int plan_bins(rsai_handle *h) {
     // bin W2: the warp bin's algorithm for |I| <= 128 (B 128 x 32), fewer warps per SM
     h->capW2 = Caps{128, 32, 512, 64, 128 * 32, 64, h->tuning.small_qr_max_p, 0, 0, 128, spai};
     if (plan_w2(h, fp32) != RSAI_OK) return RSAI_ERR_CUDA;
+    // bin S: 128 threads per column, |I| <= 128, |J| <= 64, four or five columns
+    // per SM (FP32; three in FP64) instead of bin C's one: the small end of bin
+    // C, on the same arithmetic bit for bit
+    h->capS = Caps{128, 64, 512, std::min(std::max(64, rneed), 512), 128 * 64, 0, 0, 0, 1, 256, spai};
+    occ = occupancy_bin_block(fp32, CTA_BIN_SMALL, h->capS);
+    if (occ < 1) return RSAI_ERR_CUDA;
+    h->grid_s = h->sms * occ;
     // bin C: shared-memory workspace as large as the opt-in limit allows
     Caps c{1024, 256, 4096, std::min(rneed * 2, 2048), 0, 0, 0, 0, 1, 1024, spai};
     size_t base = fp32 ? work_bytes<float>(c) : work_bytes<double>(c);
@@ -413,7 +428,7 @@ int plan_bins(rsai_handle *h) {
     if (base >= avail) return RSAI_ERR_CUDA;
     c.bcap = (int64_t)((avail - base) / (fp32 ? sizeof(float) : sizeof(double))) - 64;
     h->capC = c;
-    occ = occupancy_bin_block(fp32, h->capC, false);
+    occ = occupancy_bin_block(fp32, CTA_BIN_SHARED, h->capC);
     if (occ < 1) return RSAI_ERR_CUDA;
     h->grid_c = h->sms * occ;
     // bin G: a global-memory slab per CTA, one CTA per SM
@@ -546,11 +561,12 @@ int build_common(rsai_handle *h, cudaStream_t st) {
     if (h->params.precision == RSAI_FP32_REFINE) TRY(dalloc(h, &h->cval32, nnz, st));
     // ---- buffers of the build sequence ----
     h->ovf_cap = n;
-    TRY(dalloc(h, &h->qnext, 10, st));
+    TRY(dalloc(h, &h->qnext, 12, st));
     TRY(dalloc(h, &h->ovf0, n, st));
     TRY(dalloc(h, &h->ovf1, n, st));
     TRY(dalloc(h, &h->ovf2, n, st));
     TRY(dalloc(h, &h->ovf3, n, st));
+    TRY(dalloc(h, &h->ovf_s, n, st));
     TRY(dalloc(h, &h->ovf3_sorted, n, st));
     TRY(dalloc(h, &h->cost_bucket, n, st));
     TRY(dalloc(h, &h->cost_hist, kCostBuckets, st));
