@@ -24,7 +24,8 @@
 
 #include <type_traits>
 
-#include "common.cuh"
+#include "panel.cuh"
+#include "stage_map.cuh"
 #include "warp_small.cuh"
 
 namespace rsai {
@@ -42,9 +43,6 @@ struct Caps {
     int dcap;         // max number of distinct columns dropped from J (they are not charged again on re-entry)
     int spai;         // SPAI selection: a score per candidate column (scap of them)
 };
-
-// Columns of one compact-WY panel (global-memory bins)
-constexpr int kPanel = 16;
 
 template <typename T> struct Work {
     T *B, *vhead, *tau, *rhs;
@@ -178,724 +176,6 @@ __device__ __forceinline__ long long solve_flops(long long q0, long long p0, lon
     long long s2 = mm * (mm + 1) * (2 * mm + 1) / 6;
     f += (q - p) * (2 * mm + 2 * mm * (mm + 1)) + mm * (mm + 1) + 4 * s2;
     return f + p * p;
-}
-
-// rhs[0..p) <- R^{-1} rhs[0..p) (column-oriented, in place)
-template <class Team, typename T>
-__device__ void back_substitute_team(const Team &team, const T *B, int q, int p, T *rhs, T small) {
-    const int me = team.rank();
-    for (int i = p - 1; i >= 0; --i) {
-        T d = B[(int64_t)i * q + i];
-        T xi = (fabs(d) <= small) ? T(0) : rhs[i] / d;
-        team.sync();
-        for (int c = me; c < i; c += Team::SIZE) rhs[c] -= B[(int64_t)i * q + c] * xi;
-        if (me == 0) rhs[i] = xi;
-        team.sync();
-    }
-}
-
-// Householder QR of B (q x p, column-major, ld q) applied to rhs, then back
-// substitution into rhs[0..p).  Keeps the reflectors (v_j below the diagonal
-// of B, heads in vhead, tau = 2 / v^T v in tau) for the refinement solve.  Returns the
-// rank flag.  Team-generic: the norm of the pivot column is one team
-// reduction; the trailing columns (and rhs) are dealt out to the team's warps,
-// each warp forming its column's dot product with the reflector (lanes over
-// rows, one warp reduction) and applying the update itself, so a step costs
-// one team synchronisation instead of one per column.  Not inlined.
-// One Householder step j on B (q x p, ld q) and rhs: the reflector of column j
-// over rows >= j, applied to the columns c in [c_begin, p) and to rhs.  The
-// norm is one team reduction; the columns are dealt out to the team's warps,
-// each warp forming its column's dot product (lanes over rows, one warp
-// reduction) and applying the update itself.  Stores R_jj, v_j(j), v_j^T v_j.
-template <class Team, typename T>
-__device__ __forceinline__ void householder_step(const Team &team, T *B, int q, int p, T *rhs, T *vhead, T *taus,
-                                                 int j, int c_begin, T small, int &rank_flag) {
-    const int me = team.rank();
-    constexpr int LN = Team::LANES;  // lanes of one group: the team itself, or one warp of a CTA
-    constexpr int NW = Team::SIZE / LN;
-    const int lane = me % LN, wid = me / LN;
-    T *col = B + (int64_t)j * q;
-    T part = 0;
-    for (int i = j + me; i < q; i += Team::SIZE) part += col[i] * col[i];
-    const T sigma = team.sum(part);
-    const T x0 = col[j];
-    const T nrm = sqrt(sigma);
-    const T alpha = (x0 >= T(0)) ? -nrm : nrm;
-    const T v0 = x0 - alpha;
-    const T vtv = sigma - x0 * x0 + v0 * v0;
-    const T two_over = (vtv > T(0)) ? T(2) / vtv : T(0);
-    if (two_over > T(0)) {
-        for (int c = c_begin + wid; c <= p; c += NW) {
-            T *t = (c < p) ? B + (int64_t)c * q : rhs;
-            T d = 0;
-            for (int i = j + lane; i < q; i += LN) d += ((i == j) ? v0 : col[i]) * t[i];
-            d = team.lanes_sum(d);
-            const T f = d * two_over;
-            for (int i = j + lane; i < q; i += LN) t[i] -= f * ((i == j) ? v0 : col[i]);
-        }
-    }
-    team.sync();
-    if (me == 0) {
-        col[j] = alpha;
-        vhead[j] = v0;
-        taus[j] = two_over;
-    }
-    rank_flag |= (fabs(alpha) <= small) ? 1 : 0;
-    team.sync();
-}
-
-// Householder QR of B (q x p, column-major, ld q) applied to rhs, then back
-// substitution into rhs[0..p).  Keeps the reflectors (v_j below the diagonal
-// of B, heads in vhead, tau = 2 / v^T v in tau) for the refinement solve.  Returns the
-// rank flag.  Team-generic, one team synchronisation per step; not inlined.
-template <class Team, typename T>
-__device__ __noinline__ int qr_solve_team(Team team, T *B, int q, int p, T *rhs, T *vhead, T *taus, T small) {
-    int rank_flag = 0;
-    for (int j = 0; j < p; ++j) householder_step(team, B, q, p, rhs, vhead, taus, j, j + 1, small, rank_flag);
-    back_substitute_team(team, B, q, p, rhs, small);
-    return rank_flag;
-}
-
-// Householder steps j_start..p-1 on B and rhs, no back substitution (rhs is
-// left holding Q^T rhs): a factor from scratch (j_start = 0) that is kept for
-// later updates, or the appended block of the QR update.  Not inlined.
-template <class Team, typename T>
-__device__ __noinline__ int qr_factor_team(Team team, T *B, int q, int p, T *rhs, T *vhead, T *taus, T small,
-                                           int j_start) {
-    int rank_flag = 0;
-    for (int j = j_start; j < p; ++j) householder_step(team, B, q, p, rhs, vhead, taus, j, j + 1, small, rank_flag);
-    return rank_flag;
-}
-
-// Columns c in [c_lo, c_hi] of B (ld q; c == p stands for rhs), rows
-// j0..j0+qq-1: C <- C - V (T^T (V^T C)).  Each warp takes kCols columns at a
-// time (four in FP32, two in FP64) so that every reflector value read from
-// shared memory serves kCols columns, kRows rows per lane and pass.  A pass
-// over kRows full rows of a full panel takes a path without per-element bounds
-// tests (a warp's missing columns read its first column again and store
-// nothing).  Ends with a team synchronisation.
-template <class Team, typename T>
-__device__ __forceinline__ void wy_apply(const Team &team, const T *V, int qq, int nb, const T *tm, T *B, int q,
-                                         int p, T *rhs, int j0, int c_lo, int c_hi) {
-    const int me = team.rank();
-    const int lane = me & 31, wid = me >> 5;
-    constexpr int NW = (Team::SIZE + 31) / 32;
-    constexpr int kCols = sizeof(T) == 8 ? 2 : 4;  // W of kCols x kPanel values stays in registers
-    constexpr int kRows = 4;
-    const bool full_panel = nb == kPanel;
-    for (int c0 = c_lo + wid * kCols; c0 <= c_hi; c0 += NW * kCols) {
-        T *tc[kCols];
-        bool has[kCols];
-#pragma unroll
-        for (int x = 0; x < kCols; ++x) {
-            const int c = c0 + x;
-            has[x] = c <= c_hi;
-            tc[x] = !has[x] ? nullptr : ((c < p) ? B + (int64_t)c * q + j0 : rhs + j0);
-        }
-        T *tf[kCols];  // the fast path's columns: a missing one reads column c0
-#pragma unroll
-        for (int x = 0; x < kCols; ++x) tf[x] = has[x] ? tc[x] : tc[0];
-        const bool all_cols = full_panel;  // every present column on the fast path
-        T wv[kCols][kPanel];
-#pragma unroll
-        for (int x = 0; x < kCols; ++x)
-#pragma unroll
-            for (int u = 0; u < kPanel; ++u) wv[x][u] = T(0);
-        // W = V^T C; kRows rows per pass (r, r + 32, ...), their loads issued before any use
-        for (int r = lane; r < qq; r += 32 * kRows) {
-            T cr[kRows][kCols];
-            if (all_cols && r + 32 * (kRows - 1) < qq) {
-#pragma unroll
-                for (int y = 0; y < kRows; ++y)
-#pragma unroll
-                    for (int x = 0; x < kCols; ++x) cr[y][x] = tf[x][r + 32 * y];
-#pragma unroll
-                for (int u = 0; u < kPanel; ++u) {
-                    const T *vu = V + (int64_t)u * qq + r;
-                    T v[kRows];
-#pragma unroll
-                    for (int y = 0; y < kRows; ++y) v[y] = vu[32 * y];
-#pragma unroll
-                    for (int x = 0; x < kCols; ++x)
-#pragma unroll
-                        for (int y = 0; y < kRows; ++y) wv[x][u] += v[y] * cr[y][x];
-                }
-                continue;
-            }
-#pragma unroll
-            for (int y = 0; y < kRows; ++y)
-#pragma unroll
-                for (int x = 0; x < kCols; ++x) cr[y][x] = (tc[x] && r + 32 * y < qq) ? tc[x][r + 32 * y] : T(0);
-#pragma unroll
-            for (int u = 0; u < kPanel; ++u) {
-                if (u < nb) {
-                    T v[kRows];
-#pragma unroll
-                    for (int y = 0; y < kRows; ++y) v[y] = (r + 32 * y < qq) ? V[(int64_t)u * qq + r + 32 * y] : T(0);
-#pragma unroll
-                    for (int x = 0; x < kCols; ++x)
-#pragma unroll
-                        for (int y = 0; y < kRows; ++y) wv[x][u] += v[y] * cr[y][x];
-                }
-            }
-        }
-#pragma unroll
-        for (int x = 0; x < kCols; ++x)
-#pragma unroll
-            for (int u = 0; u < kPanel; ++u)
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) wv[x][u] += __shfl_xor_sync(0xffffffffu, wv[x][u], o);
-        // w2 = T^T w (kept in wv, highest u first so that lower entries are still w)
-#pragma unroll
-        for (int x = 0; x < kCols; ++x) {
-#pragma unroll
-            for (int u = kPanel - 1; u >= 0; --u) {
-                T acc = 0;
-#pragma unroll
-                for (int s2 = 0; s2 <= u; ++s2)
-                    if (u < nb) acc += tm[s2 * kPanel + u] * wv[x][s2];
-                wv[x][u] = acc;
-            }
-        }
-        for (int r = lane; r < qq; r += 32 * kRows) {
-            T acc[kRows][kCols];
-            if (all_cols && r + 32 * (kRows - 1) < qq) {
-#pragma unroll
-                for (int y = 0; y < kRows; ++y)
-#pragma unroll
-                    for (int x = 0; x < kCols; ++x) acc[y][x] = tf[x][r + 32 * y];
-#pragma unroll
-                for (int u = 0; u < kPanel; ++u) {
-                    const T *vu = V + (int64_t)u * qq + r;
-#pragma unroll
-                    for (int y = 0; y < kRows; ++y) {
-                        const T v = vu[32 * y];
-#pragma unroll
-                        for (int x = 0; x < kCols; ++x) acc[y][x] -= v * wv[x][u];
-                    }
-                }
-#pragma unroll
-                for (int y = 0; y < kRows; ++y)
-#pragma unroll
-                    for (int x = 0; x < kCols; ++x)
-                        if (has[x]) tc[x][r + 32 * y] = acc[y][x];
-                continue;
-            }
-#pragma unroll
-            for (int y = 0; y < kRows; ++y)
-#pragma unroll
-                for (int x = 0; x < kCols; ++x) acc[y][x] = (tc[x] && r + 32 * y < qq) ? tc[x][r + 32 * y] : T(0);
-#pragma unroll
-            for (int u = 0; u < kPanel; ++u) {
-                if (u < nb) {
-#pragma unroll
-                    for (int y = 0; y < kRows; ++y) {
-                        const T v = (r + 32 * y < qq) ? V[(int64_t)u * qq + r + 32 * y] : T(0);
-#pragma unroll
-                        for (int x = 0; x < kCols; ++x) acc[y][x] -= v * wv[x][u];
-                    }
-                }
-            }
-#pragma unroll
-            for (int y = 0; y < kRows; ++y)
-#pragma unroll
-                for (int x = 0; x < kCols; ++x)
-                    if (tc[x] && r + 32 * y < qq) tc[x][r + 32 * y] = acc[y][x];
-        }
-    }
-    team.sync();
-}
-
-// Head of the panel staging area (global-memory bins), in elements of T: the
-// panel's T (kPanel x kPanel), the CTA reduction slots (kPanel per warp) and
-// two kPanel-vectors of results; the staged panel V follows.
-template <class Team> constexpr int kStageHead = kPanel * kPanel + (Team::SIZE / 32 + 2) * kPanel;
-
-// Sum of kPanel values over the 32 lanes of a warp by halving exchanges (a
-// lane keeps the half of its vector that its partner sends back summed): 16
-// shuffles instead of 16 x 5.  Lanes 2e and 2e+1 end up holding the sum of
-// entry rs_entry(lane) in v[0].
-__device__ __forceinline__ int rs_entry(int lane) {
-    return ((lane >> 4) & 1) * 8 + ((lane >> 3) & 1) * 4 + ((lane >> 2) & 1) * 2 + ((lane >> 1) & 1);
-}
-template <typename T> __device__ __forceinline__ T warp_reduce_scatter16(T (&v)[kPanel], int lane) {
-    static_assert(kPanel == 16, "the exchange pattern below is written for 16 values");
-#pragma unroll
-    for (int h = 8, o = 16; h >= 1; h >>= 1, o >>= 1) {
-        const bool up = (lane & o) != 0;
-#pragma unroll
-        for (int i = 0; i < h; ++i) {
-            const T send = up ? v[i] : v[i + h];
-            const T keep = up ? v[i + h] : v[i];
-            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-        }
-    }
-    return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
-}
-
-// out[0..kPanel) = the sums of v[0..kPanel) over the CTA, visible to every
-// thread on return (two synchronisations).  The warps' partial sums go through
-// red, kPanel per warp; warp 0 adds them, lane l taking entry l % kPanel over
-// every other warp and one shuffle joining the two halves.
-template <class Team, typename T>
-__device__ __forceinline__ void team_sum16(const Team &team, T (&v)[kPanel], T *red, T *out) {
-    constexpr int NW = Team::SIZE / 32;
-    const int me = team.rank(), lane = me & 31;
-    const T sv = warp_reduce_scatter16(v, lane);
-    if ((lane & 1) == 0) red[(me >> 5) * kPanel + rs_entry(lane)] = sv;
-    team.sync();
-    if (me < 32) {
-        const int e = lane & (kPanel - 1);
-        T a = T(0);
-#pragma unroll
-        for (int w = lane >> 4; w < NW; w += 2) a += red[w * kPanel + e];
-        a += __shfl_xor_sync(0xffffffffu, a, 16);
-        if (lane < kPanel) out[lane] = a;
-    }
-    team.sync();
-}
-
-// Asynchronous element copies global -> shared (cp.async, 4 or 8 bytes: no
-// alignment beyond the element's own); cp_async_wait waits for the calling
-// thread's copies.
-template <typename T> __device__ __forceinline__ void cp_async_elem(T *smem_dst, const T *gmem_src) {
-    static_assert(sizeof(T) == 4 || sizeof(T) == 8, "4- or 8-byte elements");
-    const unsigned sa = (unsigned)__cvta_generic_to_shared(smem_dst);
-    if constexpr (sizeof(T) == 4)
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(sa), "l"(gmem_src) : "memory");
-    else
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(sa), "l"(gmem_src) : "memory");
-}
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
-
-// rhs[0..p) <- R^{-1} rhs[0..p) for a CTA team, in blocks of kBS rows from
-// the bottom: one warp solves the block's triangle (lane l holds row b0 + l
-// and loads its row of the block into registers first), then every thread
-// subtracts the block's part from the rows above.  Each row receives its
-// terms in the same order (descending column) as the one-row-at-a-time
-// version, so the results are identical.
-template <class Team, typename T>
-__device__ void back_substitute_blocked(const Team &team, const T *B, int q, int p, T *rhs, T small) {
-    constexpr int kBS = sizeof(T) == 8 ? 16 : 32;
-    const int me = team.rank();
-    for (int b1 = p; b1 > 0;) {
-        const int b0 = max(0, b1 - kBS);
-        const int nbk = b1 - b0;
-        if (me < 32) {
-            const int i = b0 + me;
-            const bool row = me < nbk;
-            T rv[kBS];
-#pragma unroll
-            for (int u = 0; u < kBS; ++u) rv[u] = (row && u < nbk) ? B[(int64_t)(b0 + u) * q + i] : T(0);
-            const T dd = row ? B[(int64_t)i * q + i] : T(1);
-            T xi = row ? rhs[i] : T(0);
-#pragma unroll
-            for (int u = kBS - 1; u >= 0; --u) {
-                if (u < nbk) {
-                    const T rr = __shfl_sync(0xffffffffu, xi, u);
-                    const T d = __shfl_sync(0xffffffffu, dd, u);
-                    const T xr = (fabs(d) <= small) ? T(0) : rr / d;
-                    if (me == u) xi = xr;
-                    else if (me < u) xi -= rv[u] * xr;
-                }
-            }
-            if (row) rhs[i] = xi;
-        }
-        team.sync();
-        for (int c = me; c < b0; c += Team::SIZE) {
-            T bv[kBS];
-#pragma unroll
-            for (int u = 0; u < kBS; ++u) bv[u] = (u < nbk) ? B[(int64_t)(b0 + u) * q + c] : T(0);
-            T a = rhs[c];
-#pragma unroll
-            for (int u = kBS - 1; u >= 0; --u)
-                if (u < nbk) a -= bv[u] * rhs[b0 + u];
-            rhs[c] = a;
-        }
-        team.sync();
-        b1 = b0;
-    }
-}
-
-// Householder QR of the staged panel V (rows 0..qq-1, nb <= kPanel columns,
-// ld qq, shared memory) with the T of its compact-WY form.  Step t makes one
-// pass over rows r >= t for x.x (x = column t), c.x for the trailing panel
-// columns c and v_s.x for the earlier reflectors s, and one CTA reduction of
-// the kPanel sums.  Since v_t differs from x only in its head (v0 instead of
-// x0), v_t.c = c.x + (v0 - x0) c_t and Y(s,t) = v_s.v_t = v_s.x + (v0 - x0) v_s(t).
-// Y(s,t) is kept below the diagonal of tm (tm[t * kPanel + s]) and tau_t on it;
-// after the last step one warp forms T(t,t) = tau_t and
-// T(s,t) = -tau_t sum_{s <= s2 < t} T(s,s2) Y(s2,t) above it (tm[s * kPanel + t]).
-// Leaves R on and above the diagonal, the reflector tails below it, and
-// vhead[t] = v0, taus[t] = 2 / v^T v.
-template <class Team, typename T>
-__device__ __forceinline__ void panel_factor_fused(const Team &team, T *V, int qq, int nb, T *vhead, T *taus, T *tm,
-                                                   T *red, T *out, T *out2, T small, int &rank_flag) {
-    const int me = team.rank();
-    for (int t = 0; t < nb; ++t) {
-        T *x = V + (int64_t)t * qq;
-        T acc[kPanel];
-#pragma unroll
-        for (int u = 0; u < kPanel; ++u) acc[u] = T(0);
-        // two rows per thread and iteration: their loads are issued together
-        int r = t + me;
-        for (; r + Team::SIZE < qq; r += 2 * Team::SIZE) {
-            const T xa = x[r], xb = x[r + Team::SIZE];
-#pragma unroll
-            for (int u = 0; u < kPanel; ++u) {
-                if (u < nb) {
-                    const T *vu = V + (int64_t)u * qq + r;
-                    acc[u] += vu[0] * xa + vu[Team::SIZE] * xb;
-                }
-            }
-        }
-        if (r < qq) {
-            const T xr = x[r];
-#pragma unroll
-            for (int u = 0; u < kPanel; ++u)
-                if (u < nb) acc[u] += V[(int64_t)u * qq + r] * xr;
-        }
-        team_sum16(team, acc, red, out);
-        const T sigma = out[t];
-        const T x0 = x[t];
-        const T nrm = sqrt(sigma);
-        const T alpha = (x0 >= T(0)) ? -nrm : nrm;
-        const T v0 = x0 - alpha;
-        const T vtv = sigma - x0 * x0 + v0 * v0;
-        const T two_over = (vtv > T(0)) ? T(2) / vtv : T(0);
-        if (me < nb) {
-            if (me == t) {
-                tm[t * kPanel + t] = two_over;
-            } else {
-                const T d = out[me] + (v0 - x0) * V[(int64_t)me * qq + t];
-                if (me > t) out2[me] = d * two_over;  // f_c for the trailing column c = me
-                else tm[t * kPanel + me] = d;          // Y(s,t) for the earlier reflector s = me
-            }
-        }
-        team.sync();
-        if (two_over > T(0)) {
-            int r2 = t + me;
-            for (; r2 + Team::SIZE < qq; r2 += 2 * Team::SIZE) {
-                const T va = (r2 == t) ? v0 : x[r2], vb = x[r2 + Team::SIZE];
-#pragma unroll
-                for (int u = 0; u < kPanel; ++u) {
-                    if (u > t && u < nb) {
-                        T *cu = V + (int64_t)u * qq + r2;
-                        const T f = out2[u];
-                        const T ca = cu[0], cb = cu[Team::SIZE];
-                        cu[0] = ca - f * va;
-                        cu[Team::SIZE] = cb - f * vb;
-                    }
-                }
-            }
-            if (r2 < qq) {
-                const T vr = (r2 == t) ? v0 : x[r2];
-#pragma unroll
-                for (int u = 0; u < kPanel; ++u)
-                    if (u > t && u < nb) V[(int64_t)u * qq + r2] -= out2[u] * vr;
-            }
-        }
-        team.sync();
-        if (me == 0) {
-            x[t] = alpha;
-            vhead[t] = v0;
-            taus[t] = two_over;
-        }
-        rank_flag |= (fabs(alpha) <= small) ? 1 : 0;
-    }
-    // T from Y and tau: lane s of warp 0 holds row s of T
-    if (me < 32) {
-        const int sr = me;
-        T trow[kPanel];
-#pragma unroll
-        for (int t = 0; t < kPanel; ++t) {
-            trow[t] = T(0);
-            if (t < nb) {
-                const T tau = tm[t * kPanel + t];
-                T a = T(0);
-#pragma unroll
-                for (int s2 = 0; s2 < t; ++s2)
-                    if (s2 >= sr) a += trow[s2] * tm[t * kPanel + s2];
-                if (sr < t) trow[t] = -tau * a;
-                else if (sr == t) trow[t] = tau;
-            }
-        }
-        if (sr < nb) {
-#pragma unroll
-            for (int t = 0; t < kPanel; ++t)
-                if (t > sr && t < nb) tm[sr * kPanel + t] = trow[t];
-        }
-    }
-    team.sync();
-}
-
-// rhs <- Q^T rhs with the reflectors in the panels they were factored in
-// (pnb, Tst): per panel w = V^T rhs (one CTA reduction), y = T^T w, and
-// rhs <- rhs - V y, with V = the explicit reflectors (vhead on the diagonal,
-// the tails of B below it).  A panel is taken in sub-panels of as many
-// reflectors as the staging area holds (the diagonal blocks of its T); each is
-// copied there first (cp.async) and both passes read shared memory.  When
-// fewer than two reflectors fit, or one is left, the rest of the panel reads
-// its tails from the slab.
-template <class Team, typename T>
-__device__ __noinline__ void apply_qt_panels(Team team, const T *B, int q, int p, T *rhs, const T *vhead,
-                                             const T *Tst, const int32_t *pnb, T *stage, int stage_bytes) {
-    constexpr int NW = Team::SIZE / 32;
-    const int me = team.rank();
-    T *red = stage + kPanel * kPanel, *out = red + NW * kPanel, *out2 = out + kPanel;
-    T *V = stage + kStageHead<Team>;
-    const int64_t velems = (int64_t)stage_bytes / (int64_t)sizeof(T) - kStageHead<Team>;
-    for (int jp = 0; jp < p;) {
-        const int nbp = pnb[jp];
-        // sub-panels of as many reflectors as the staging area holds (the
-        // diagonal blocks of a panel's T are the T's of its sub-panels); a
-        // sub-panel that cannot be staged reads its reflectors from the slab
-        for (int js = 0; js < nbp;) {
-            const int j0 = jp + js;
-            const int qq = q - j0;
-            const int64_t fit = velems / (int64_t)max(qq, 1);
-            const bool staged = nbp - js > 1 && fit >= 2;
-            const int nb = staged ? (int)min((int64_t)(nbp - js), fit) : nbp - js;
-            if (staged) {
-                for (int t = 0; t < nb; ++t) {
-                    const T *src = B + (int64_t)(j0 + t) * q + j0;
-                    T *dst = V + (int64_t)t * qq;
-                    for (int r = me; r < qq; r += Team::SIZE) {
-                        if (r > t) cp_async_elem(dst + r, src + r);
-                        else dst[r] = (r == t) ? vhead[j0 + t] : T(0);
-                    }
-                }
-                cp_async_wait();
-                team.sync();
-            }
-            T acc[kPanel];
-#pragma unroll
-            for (int u = 0; u < kPanel; ++u) acc[u] = T(0);
-            if (staged) {
-                for (int r = me; r < qq; r += Team::SIZE) {
-                    const T x = rhs[j0 + r];
-#pragma unroll
-                    for (int u = 0; u < kPanel; ++u)
-                        if (u < nb) acc[u] += V[(int64_t)u * qq + r] * x;
-                }
-            } else {
-                for (int i = j0 + me; i < q; i += Team::SIZE) {
-                    const T x = rhs[i];
-#pragma unroll
-                    for (int u = 0; u < kPanel; ++u) {
-                        if (u < nb) {
-                            const int j = j0 + u;
-                            const T v = (i > j) ? B[(int64_t)j * q + i] : ((i == j) ? vhead[j] : T(0));
-                            acc[u] += v * x;
-                        }
-                    }
-                }
-            }
-            team_sum16(team, acc, red, out);
-            if (me < nb) {
-                T y = 0;
-                for (int s2 = 0; s2 <= me; ++s2) y += Tst[(int64_t)(j0 + me) * kPanel + js + s2] * out[s2];
-                out2[me] = y;
-            }
-            team.sync();
-            if (staged) {
-                for (int r = me; r < qq; r += Team::SIZE) {
-                    T a = rhs[j0 + r];
-#pragma unroll
-                    for (int u = 0; u < kPanel; ++u)
-                        if (u < nb) a -= V[(int64_t)u * qq + r] * out2[u];
-                    rhs[j0 + r] = a;
-                }
-            } else {
-                for (int i = j0 + me; i < q; i += Team::SIZE) {
-                    T a = rhs[i];
-#pragma unroll
-                    for (int u = 0; u < kPanel; ++u) {
-                        if (u < nb) {
-                            const int j = j0 + u;
-                            const T v = (i > j) ? B[(int64_t)j * q + i] : ((i == j) ? vhead[j] : T(0));
-                            a -= v * out2[u];
-                        }
-                    }
-                    rhs[i] = a;
-                }
-            }
-            team.sync();
-            js += nb;
-        }
-        jp += nbp;
-    }
-}
-
-// Blocked Householder QR (compact WY) for the bins whose workspace is in
-// global memory.  Panels of nb <= kPanel columns (nb chosen so that rows j0..q
-// of the panel fit the shared-memory staging area) are copied to shared
-// memory (cp.async), factored there with their T (panel_factor_fused), written
-// back, and turned into explicit reflectors V (zeros above the head, v(j) on
-// the diagonal); with T upper triangular, H_1...H_nb = I - V T V^T, every
-// trailing column and the right-hand side get
-//   C <- C - V (T^T (V^T C))
-// in one pass (one warp per four columns), so the trailing matrix in global memory
-// is streamed once per panel instead of once per reflector.  Each panel's size
-// and T are kept (pnb, Tst) for the QR update and the refinement.  A panel that
-// does not fit four columns falls back to single Householder steps (panels of
-// one).  The reflectors, R and rhs are those of the unblocked version up to
-// rounding.  j_start > 0 factors only columns j_start..p-1 (the columns
-// appended to a factor whose first j_start columns are done, Section 3).
-// Leaves Q^T rhs in rhs.
-template <class Team, typename T>
-__device__ __noinline__ int qr_solve_staged(Team team, T *B, int q, int p, T *rhs, T *vhead, T *taus, T small,
-                                            T *stage, int stage_bytes, T *Tst, int32_t *pnb,
-                                            int j_start) {
-    const int me = team.rank();
-    constexpr int NW = Team::SIZE / 32;
-    T *tm = stage;                                  // kPanel x kPanel
-    T *red = stage + kPanel * kPanel;               // reduction slots
-    T *out = red + NW * kPanel, *out2 = out + kPanel;
-    T *V = stage + kStageHead<Team>;                // panel, ld = q - j0
-    const int64_t velems = (int64_t)stage_bytes / (int64_t)sizeof(T) - kStageHead<Team>;
-    int rank_flag = 0;
-    int j0 = j_start;
-    while (j0 < p) {
-        const int qq = q - j0;
-        int nb = (int)min((int64_t)kPanel, velems / (int64_t)max(qq, 1));
-        nb = min(nb, p - j0);
-        if (nb < 4) {
-            householder_step(team, B, q, p, rhs, vhead, taus, j0, j0 + 1, small, rank_flag);
-            if (me == 0) {
-                pnb[j0] = 1;
-                Tst[(int64_t)j0 * kPanel] = taus[j0];
-            }
-            ++j0;
-            continue;
-        }
-        // 1. stage rows j0..q-1 of the panel columns (asynchronous copies)
-        for (int t = 0; t < nb; ++t) {
-            const T *src = B + (int64_t)(j0 + t) * q + j0;
-            for (int r = me; r < qq; r += Team::SIZE) cp_async_elem(V + (int64_t)t * qq + r, src + r);
-        }
-        cp_async_wait();
-        team.sync();
-        // 2. factor the panel in shared memory (local rows r = i - j0), T alongside
-        panel_factor_fused(team, V, qq, nb, vhead + j0, taus + j0, tm, red, out, out2, small, rank_flag);
-        // 3. panel back to B (R entries and reflector tails), 4. explicit V, T kept
-        for (int idx = me; idx < nb * qq; idx += Team::SIZE) {
-            const int t = idx / qq, r = idx - t * qq;
-            B[(int64_t)(j0 + t) * q + j0 + r] = V[idx];
-        }
-        team.sync();
-        for (int idx = me; idx < nb * qq; idx += Team::SIZE) {
-            const int t = idx / qq, r = idx - t * qq;
-            if (r < t) V[idx] = T(0);
-            else if (r == t) V[idx] = vhead[j0 + t];
-        }
-        for (int e = me; e < nb * kPanel; e += Team::SIZE) {
-            const int t = e / kPanel, s2 = e - t * kPanel;
-            Tst[(int64_t)(j0 + t) * kPanel + s2] = (s2 <= t) ? tm[s2 * kPanel + t] : T(0);
-        }
-        if (me == 0) pnb[j0] = nb;
-        team.sync();
-        // 5. trailing columns and rhs, rows j0..q-1
-        wy_apply(team, V, qq, nb, tm, B, q, p, rhs, j0, j0 + nb, p);
-        j0 += nb;
-    }
-    return rank_flag;
-}
-
-// rhs <- Q^T rhs with the stored reflectors, then R^{-1}; not inlined
-template <class Team, typename T>
-__device__ __noinline__ void apply_qt_team(Team team, const T *B, int q, int p, T *rhs, const T *vhead,
-                                           const T *taus, T small) {
-    const int me = team.rank();
-    for (int j = 0; j < p; ++j) {
-        const T *col = B + (int64_t)j * q;
-        const T v0 = vhead[j], tau = taus[j];
-        if (tau > T(0)) {
-            T d = 0;
-            for (int i = me; i < q; i += Team::SIZE)
-                if (i >= j) d += ((i == j) ? v0 : col[i]) * rhs[i];
-            T sdot = team.sum(d);
-            T f = sdot * tau;
-            for (int i = me; i < q; i += Team::SIZE)
-                if (i >= j) rhs[i] -= f * ((i == j) ? v0 : col[i]);
-        }
-        team.sync();
-    }
-    if constexpr (is_lane_team<Team>::value) back_substitute_team(team, B, q, p, rhs, small);
-    else back_substitute_blocked(team, B, q, p, rhs, small);
-}
-
-// Reflector j (built on q0 rows) applied to the columns p0..p-1 of B (ld q),
-// one warp per column; ends with a team synchronisation.
-template <class Team, typename T>
-__device__ __forceinline__ void update_one_reflector(const Team &team, T *B, int q, int p, int q0, int p0,
-                                                     const T *vhead, const T *taus, int j) {
-    const int me = team.rank();
-    const int lane = me & 31, wid = me >> 5;
-    constexpr int NW = (Team::SIZE + 31) / 32;
-    const T *col = B + (int64_t)j * q;
-    const T v0 = vhead[j], two_over = taus[j];
-    if (two_over > T(0)) {
-        for (int c = p0 + wid; c < p; c += NW) {
-            T *t = B + (int64_t)c * q;
-            T d = 0;
-            for (int i = j + lane; i < q0; i += 32) d += ((i == j) ? v0 : col[i]) * t[i];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
-            const T f = d * two_over;
-            for (int i = j + lane; i < q0; i += 32) t[i] -= f * ((i == j) ? v0 : col[i]);
-        }
-    }
-    team.sync();
-}
-
-// The QR update of Section 3, first half: the reflectors 0..p0-1 of a
-// finished factor (built on q0 rows; every row below is zero in them) applied
-// to the appended columns p0..p-1 of B (ld q), rows j..q0-1, panel by panel as
-// they were factored, each panel in compact-WY form with its stored T, split
-// into sub-panels when its explicit V outgrows the staging area (q has grown
-// since it was factored).  Sub-panels of fewer than four reflectors take one
-// reflector at a time.
-template <class Team, typename T>
-__device__ __noinline__ void qr_update_apply_staged(Team team, T *B, int q, int p, int q0, int p0, const T *vhead,
-                                                    const T *taus, T *stage, int stage_bytes, const T *Tst,
-                                                    const int32_t *pnb) {
-    const int me = team.rank();
-    T *tm = stage;
-    T *V = stage + kStageHead<Team>;
-    const int64_t velems = (int64_t)stage_bytes / (int64_t)sizeof(T) - kStageHead<Team>;
-    int j0 = 0;
-    while (j0 < p0) {
-        const int nb = pnb[j0];
-        // the panel in sub-panels of as many reflectors as the staging area holds:
-        // the diagonal blocks of a panel's T are the T's of its sub-panels
-        for (int js = 0; js < nb;) {
-            const int j1 = j0 + js, qq = q0 - j1;
-            const int ns = (int)min((int64_t)(nb - js), qq > 0 ? velems / (int64_t)qq : (int64_t)0);
-            if (ns < 4) {
-                update_one_reflector(team, B, q, p, q0, p0, vhead, taus, j1);
-                ++js;
-                continue;
-            }
-            for (int t = 0; t < ns; ++t) {
-                const T *src = B + (int64_t)(j1 + t) * q + j1;
-                T *dst = V + (int64_t)t * qq;
-                for (int r = me; r < qq; r += Team::SIZE) {
-                    if (r > t) cp_async_elem(dst + r, src + r);
-                    else dst[r] = (r == t) ? vhead[j1 + t] : T(0);
-                }
-            }
-            cp_async_wait();
-            for (int e = me; e < kPanel * kPanel; e += Team::SIZE) {
-                const int s2 = e / kPanel, t = e - s2 * kPanel;
-                tm[e] = (t < ns && s2 <= t) ? Tst[(int64_t)(j1 + t) * kPanel + js + s2] : T(0);
-            }
-            team.sync();
-            wy_apply(team, V, qq, ns, tm, B, q, p, (T *)nullptr, j1, p0, p - 1);
-            js += ns;
-        }
-        j0 += nb;
-    }
 }
 
 // J = rows of A(:,k), ascending as the CSC keeps them; returns |J|, or -1 if
@@ -1127,8 +407,38 @@ template <class Team, typename T> struct Column {
     }
     __device__ __forceinline__ int find_J(int32_t col) const { return jset().find(col); }
 
-    // I = sorted rows of A(:,J) (Section 2).  Returns false on overflow.
+    // The bitmap over indices 0..n-1 in the staging area (global-memory bins;
+    // off elsewhere and for n too large for it)
+    __device__ __forceinline__ StageMap stage_map() const { return StageMap(w.stage, cap.stage_bytes, A.n); }
+
+    // I = sorted rows of A(:,J) (Section 2).  Returns false on overflow.  In the
+    // global-memory bins the staging area keeps the map of I for the gathers.
     __device__ bool rows_of_J() {
+        if constexpr (Team::STAGED) {
+            const StageMap map = stage_map();
+            if (map.on()) {
+                map.clear(team);
+                int entries = 0;
+                for (int c = team.rank(); c < p; c += Team::SIZE) {
+                    const int64_t st = A.col_ptr[w.J[c]];
+                    const int len = (int)(A.col_ptr[w.J[c] + 1] - st);
+                    entries += len;
+                    for (int e = 0; e < len; e += 4) {
+                        int32_t v[4];
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) v[u] = (e + u < len) ? A.row_idx[st + e + u] : 0;
+#pragma unroll
+                        for (int u = 0; u < 4; ++u)
+                            if (e + u < len) map.mark(v[u]);
+                    }
+                }
+                entries = team.sum(entries);
+                const int nq = map.finish(team, w.I, cap.qcap);
+                if (next_pow2(entries) > cap.scap || nq > cap.qcap) return false;
+                q = nq;
+                return true;
+            }
+        }
         int base = 0;
         for (int c0 = 0; c0 < p; c0 += Team::SIZE) {
             int c = c0 + team.rank();
@@ -1236,6 +546,95 @@ template <class Team, typename T> struct Column {
         apply_qt_team<Team, T>(team, w.B, q, p, w.rhs, w.vhead, w.tau, small);
     }
 
+    // r on the rows of S and, unless `refine`, rho (CTA teams).  The sum of a row
+    // is defined on 32 lane chains (entries l, l + 32, ... of the row on lane l)
+    // joined by a butterfly over offsets 16, 8, 4, 2, 1, and ||r||^2 as the
+    // chains of the rows w, w + 16, ... for w < 16, added in order, for every CTA
+    // size.  FP64 additions are what bounds this (a warp instruction takes the
+    // SM's FP64 unit 16 cycles however many of its lanes are active), and most rows
+    // hold under 16 entries: so eight lanes work on a row, each keeping its
+    // four chains (lanes l, l + 8, l + 16, l + 24), the first two levels of the
+    // butterfly are additions within a lane, skipped where all four rows of the
+    // warp are short (they would add zeros), and the chains of squares run on
+    // 16 lanes of one warp, one each, at the end.
+    __device__ __forceinline__ void row_sums(bool refine, int &cnt) {
+        const int me = team.rank();
+        const int32_t *Js = w.J;
+        StageMap map(nullptr, 0, A.n);
+        if constexpr (Team::STAGED) {
+            map = stage_map();
+            if (map.on()) {
+                map.clear(team);
+                for (int c = me; c < p; c += Team::SIZE) map.mark(w.J[c]);
+                map.finish(team, nullptr, cap.pcap);
+            } else if ((size_t)p * sizeof(int32_t) <= (size_t)cap.stage_bytes) {
+                int32_t *jc = reinterpret_cast<int32_t *>(w.stage);
+                for (int c = me; c < p; c += Team::SIZE) jc[c] = w.J[c];
+                Js = jc;
+            }
+        }
+        team.sync();
+        const int sub = me & 7;
+        constexpr int RW = Team::SIZE / 8;  // rows per pass of the team
+        const int passes = (s + RW - 1) / RW;
+        for (int t = 0; t < passes; ++t) {
+            const int i = t * RW + (me >> 3);
+            int32_t row = -1;
+            int64_t e0 = 0;
+            int len = 0;
+            if (i < s) {
+                row = w.S[i];
+                e0 = A.row_ptr[row];
+                len = (int)(A.row_ptr[row + 1] - e0);
+            }
+            double acc[4] = {0.0, 0.0, 0.0, 0.0};
+            int most = len;
+#pragma unroll
+            for (int o = 16; o >= 8; o >>= 1) most = max(most, __shfl_xor_sync(0xffffffffu, most, o));
+            for (int b = 0; b < most; b += 32) {
+#pragma unroll
+                for (int h = 0; h < 4; ++h) {
+                    if (b + 8 * h >= most) break;  // the same for the whole warp
+                    const int e = b + 8 * h + sub;
+                    if (e < len) {
+                        const int32_t col = A.col_idx[e0 + e];
+                        int pos;
+                        if (Team::STAGED && map.on()) pos = map.find(col);
+                        else pos = find_i32(Js, p, col);
+                        if (pos >= 0) {
+                            acc[h] = fma(A.val[e0 + e], w.m[pos], acc[h]);
+                            ++cnt;
+                        }
+                    }
+                }
+            }
+            double x = acc[0];
+            if (most > 16) {
+                x += acc[2];
+                x += acc[1] + acc[3];
+            } else if (most > 8) {
+                x += acc[1];
+            }
+#pragma unroll
+            for (int o = 4; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+            if (row == k) x -= 1.0;
+            if (sub == 0 && i < s) w.r[i] = x;
+        }
+        team.sync();
+        if (!refine) {
+            double ss = 0.0;
+            if (me < 32) {
+                if (me < kVirtualWarps)
+                    for (int i = me; i < s; i += kVirtualWarps) ss = fma(w.r[i], w.r[i], ss);
+                double tot = __shfl_sync(0xffffffffu, ss, 0);
+#pragma unroll
+                for (int v = 1; v < kVirtualWarps; ++v) tot += __shfl_sync(0xffffffffu, ss, v);
+                ss = tot;
+            }
+            rho = sqrt(team.bcast(ss, 0));
+        }
+    }
+
     // S = I u {k}; r = A(:,J) m - e_k on S in double (Eq. 2.4), row by row
     // through the CSR of A: in ascending j on the warp bins (the oracle's
     // order), a fixed lane-strided order and butterfly on the CTA bins.
@@ -1253,48 +652,10 @@ template <class Team, typename T> struct Column {
         }
         double ss = 0.0;
         int cnt = 0;
+        (void)ss;
         if constexpr (!is_lane_team<Team>::value) {
-            // CTA teams: a warp per row, its lanes over the row's entries (rows of
-            // I can hold hundreds), summed by a fixed butterfly.  The global-memory
-            // bins search a copy of J in the staging area (shared memory).
-            const int32_t *Js = w.J;
-            if constexpr (Team::STAGED) {
-                if ((size_t)p * sizeof(int32_t) <= (size_t)cap.stage_bytes) {
-                    int32_t *jc = reinterpret_cast<int32_t *>(w.stage);
-                    for (int c = me; c < p; c += Team::SIZE) jc[c] = w.J[c];
-                    Js = jc;
-                }
-            }
-            team.sync();
-            const int lane = me & 31;
-            constexpr int NWR = Team::SIZE / 32, VK = Team::VK;
-            // squares of the rows of virtual warp (me >> 5) + NWR * v in ssv[v]: the same sums for every CTA size
-            double ssv[VK];
-#pragma unroll
-            for (int v = 0; v < VK; ++v) ssv[v] = 0.0;
-            for (int i0 = me >> 5; i0 < s; i0 += NWR * VK) {
-#pragma unroll
-                for (int v = 0; v < VK; ++v) {
-                    const int i = i0 + NWR * v;
-                    if (i < s) {
-                        const int32_t row = w.S[i];
-                        const int64_t e0 = A.row_ptr[row], e1 = A.row_ptr[row + 1];
-                        double acc = 0.0;
-                        for (int64_t e = e0 + lane; e < e1; e += 32) {
-                            const int pos = find_i32(Js, p, A.col_idx[e]);
-                            if (pos >= 0) { acc = fma(A.val[e], w.m[pos], acc); ++cnt; }
-                        }
-#pragma unroll
-                        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-                        if (row == k) acc -= 1.0;
-                        if (lane == 0) {
-                            w.r[i] = acc;
-                            if (!refine) ssv[v] = fma(acc, acc, ssv[v]);
-                        }
-                    }
-                }
-            }
-            if (!refine) rho = sqrt(team.sum_lane0(ssv));
+            // CTA teams: eight lanes per row, four rows per warp; see row_sums
+            row_sums(refine, cnt);
         } else {
             team.sync();
             for (int i = me; i < s; i += Team::SIZE) {
@@ -1357,6 +718,22 @@ template <class Team, typename T> struct Column {
         c_qmax = max(c_qmax, q);
     }
 
+    // x[0..len) = 0 (x 16-byte aligned), 16 bytes per store
+    __device__ __forceinline__ void fill_zero(T *x, int len) const {
+        constexpr int CW = 16 / (int)sizeof(T);
+        const int full = len / CW;
+        for (int i = team.rank(); i < full; i += Team::SIZE) reinterpret_cast<uint4 *>(x)[i] = make_uint4(0, 0, 0, 0);
+        for (int i = full * CW + team.rank(); i < len; i += Team::SIZE) x[i] = T(0);
+    }
+    // position of row i in I, right after rows_of_J (which left the map of I in the staging area)
+    __device__ __forceinline__ int find_I(int32_t i) const {
+        if constexpr (Team::STAGED) {
+            const StageMap map = stage_map();
+            if (map.on()) return map.find(i);
+        }
+        return find_i32(w.I, q, i);
+    }
+
     // Solve the LS problem on the current J (Eq. 2.3).  `append`: J extends
     // the previously solved J by Jhat (the paper's QR update; counted as
     // such).  The CTA bins (Caps::append) then update the kept factor instead
@@ -1379,8 +756,7 @@ template <class Team, typename T> struct Column {
         if (!rows_of_J()) return false;
         if ((int64_t)q * p > cap.bcap) return false;
         // B = A(I,J), zero-filled
-        int64_t qp = (int64_t)q * p;
-        for (int64_t i = me; i < qp; i += Team::SIZE) w.B[i] = T(0);
+        fill_zero(w.B, q * p);
         for (int i = me; i < q; i += Team::SIZE) w.rhs[i] = (w.I[i] == k) ? T(1) : T(0);
         team.sync();
         T fro2 = 0;
@@ -1402,7 +778,7 @@ template <class Team, typename T> struct Column {
                 for (int u = 0; u < 4; ++u) {
                     if (ri[u] >= 0) {
                         const T a = av[u];
-                        Bc[find_i32(w.I, q, ri[u])] = a;
+                        Bc[find_I(ri[u])] = a;
                         fro2 += a * a;
                     }
                 }
@@ -1492,14 +868,17 @@ template <class Team, typename T> struct Column {
 #pragma unroll
                 for (int u = 0; u < K; ++u) {
                     const int64_t o = lo + me + (int64_t)u * Team::SIZE;
-                    if (o < hi) w.B[(o / qo) * q + o % qo] = v[u];
+                    if (o < hi) {  // at most bcap elements: 32-bit quotients
+                        const unsigned col = (unsigned)o / (unsigned)qo;
+                        w.B[(int64_t)col * q + ((unsigned)o - col * (unsigned)qo)] = v[u];
+                    }
                 }
             }
             team.sync();
-            const int nr = q - qo;
-            for (int64_t idx = me; idx < (int64_t)po * nr; idx += Team::SIZE) {
-                const int c = (int)(idx / nr);
-                w.B[(int64_t)c * q + qo + (idx - (int64_t)c * nr)] = T(0);
+            const unsigned nr = (unsigned)(q - qo);
+            for (unsigned idx = me; idx < (unsigned)po * nr; idx += Team::SIZE) {
+                const unsigned c = idx / nr;
+                w.B[(int64_t)c * q + qo + (idx - c * nr)] = T(0);
             }
         }
         for (int64_t idx = (int64_t)po * q + me; idx < (int64_t)p * q; idx += Team::SIZE) w.B[idx] = T(0);
@@ -1512,7 +891,7 @@ template <class Team, typename T> struct Column {
             T *Bc = w.B + (int64_t)(po + b) * q;
             for (int64_t e = A.col_ptr[j]; e < A.col_ptr[j + 1]; ++e) {
                 const T a = csc_value<T>(A, e);
-                const int ii = find_i32(w.I, q, A.row_idx[e]);
+                const int ii = find_I(A.row_idx[e]);
                 if (ii >= 0) Bc[w.Ip[ii]] = a;
                 fro2 += a * a;
             }
@@ -1725,9 +1104,27 @@ template <class Team, typename T> struct Column {
 
     // Jhat = cols(A(Rhat,:)) \ J into w.buf; returns |Jhat| or -1 on overflow.
     // The rows of Rhat are dealt out to the team's ranks, as many passes as
-    // |Rhat| (<= c <= 32) needs on a team of 16.
+    // |Rhat| (<= c <= 32) needs on a team of 16.  In the global-memory bins a
+    // warp takes a row and the columns are collected in the staging area's map.
     __device__ int new_columns(int nh) {
         const int me = team.rank();
+        if constexpr (Team::STAGED) {
+            const StageMap map = stage_map();
+            if (map.on()) {
+                map.clear(team);
+                int entries = 0;
+                for (int t = me >> 5; t < nh; t += Team::SIZE / 32) {
+                    const int64_t st = A.row_ptr[w.Rhat[t]], en = A.row_ptr[w.Rhat[t] + 1];
+                    if ((me & 31) == 0) entries += (int)(en - st);
+                    for (int64_t e = st + (me & 31); e < en; e += 32) map.mark(A.col_idx[e]);
+                }
+                entries = team.sum(entries);
+                if (next_pow2(entries) > cap.scap) return -1;
+                for (int c = me; c < p; c += Team::SIZE) map.unmark(w.J[c]);
+                // at most `entries` <= scap columns: buf holds them
+                return map.finish(team, w.buf, cap.scap);
+            }
+        }
         int tot = 0;
         for (int t0 = 0; t0 < nh; t0 += Team::SIZE) {
             const int t = t0 + me;

@@ -270,21 +270,6 @@ template <int NT, bool STAGED_ = false> struct BlockTeam {
         for (int w = 1; w < NW; ++w) s += slot<V>(w);
         return s;
     }
-    // sum of the values that lane 0 of each of kVirtualWarps warps would hold:
-    // this warp holds those of warps wid, wid + NW, ...; added in warp order
-    static constexpr int VK = kVirtualWarps / NW;
-    template <typename V> __device__ __forceinline__ V sum_lane0(const V (&x)[VK]) const {
-        __syncthreads();
-        if ((threadIdx.x & 31) == 0) {
-#pragma unroll
-            for (int v = 0; v < VK; ++v) slot<V>((threadIdx.x >> 5) + NW * v) = x[v];
-        }
-        __syncthreads();
-        V s = slot<V>(0);
-#pragma unroll
-        for (int w = 1; w < kVirtualWarps; ++w) s += slot<V>(w);
-        return s;
-    }
     template <typename V> __device__ __forceinline__ V maxv(V x) const {
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {

@@ -33,3 +33,28 @@ def test_columns_between_the_warp_and_the_large_cta_bin(precision, N, eps, drop)
     tol = 1e-9 if precision == "fp64" else 1e-6
     np.testing.assert_allclose(mv.cpu().numpy(), res[2], rtol=tol, atol=tol * np.abs(res[2]).max())
     np.testing.assert_allclose(np.sqrt(rho2.cpu().numpy()), rho, rtol=tol, atol=1e-12)
+
+
+def embedded(block, n):
+    """diag(block, I): the block's columns are built as in the block alone."""
+    m = block.n
+    rows = np.concatenate([np.repeat(np.arange(m), np.diff(block.row_ptr)), np.arange(m, n)])
+    cols = np.concatenate([block.col_idx, np.arange(m, n)])
+    return gen.from_coo(n, rows, cols, np.concatenate([block.val, np.ones(n - m)]))
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32_refine"])
+@pytest.mark.parametrize("n", [1_200_000, 1_300_000])
+def test_index_sets_of_large_problems(precision, n):
+    """The global bin keeps index sets as bitmaps of n bits while they fit its shared memory
+    (n up to about 1.2 million) and sorts and searches beyond; both give the small problem's
+    columns bit for bit."""
+    block = gen.powerlaw(900, seed=5, dmax=100)
+    kw = dict(c=5, l_max=8, eps=0.4, tol=1e-3, drop="fixed")
+    _, _, small, rho_s, loops_s, _, st = gpu_M(block, precision=precision, **kw)
+    assert st["cols_bin"][2] > 0
+    _, _, large, rho, loops, _, _ = gpu_M(embedded(block, n), precision=precision, **kw)
+    m, nnz = block.n, small[0][-1]
+    assert np.array_equal(large[0][: m + 1], small[0])
+    assert np.array_equal(large[1][:nnz], small[1]) and np.array_equal(large[2][:nnz], small[2])
+    assert np.array_equal(rho[:m], rho_s) and np.array_equal(loops[:m], loops_s)
