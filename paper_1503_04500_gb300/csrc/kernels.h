@@ -100,25 +100,12 @@ cudaError_t launch_spmv(int64_t n, const int64_t *row_ptr, const int32_t *col_id
 // gval[e] = gy[row(e)] * x[col(e)] over the stored entries of a CSR matrix
 cudaError_t launch_spmv_grad_values(int64_t n, const int64_t *row_ptr, const int32_t *col_idx, const double *gy,
                                     const double *x, double *gval, cudaStream_t st);
-cudaError_t launch_dot(int64_t n, const double *x, const double *y, double *partials, double *out, cudaStream_t st);
+// right-preconditioned BiCGStab (bicgstab.cu)
 int bicgstab_run(int64_t n, const int64_t *Arp, const int32_t *Aci, const double *Av, const int64_t *Mrp,
                  const int32_t *Mci, const double *Mv, const double *b, double *x, double rtol, int maxit,
                  int *iters, double *relres, cudaStream_t st, double *work = nullptr);
 // device bytes bicgstab_run needs as its workspace for size n
 size_t bicgstab_workspace_bytes(int64_t n);
-
-// BiCGStab vector steps (apply_kernels.cu); scalars on the device
-__global__ void k_bicg_p(int64_t n, const double *sc, const double *r, const double *v, double *p);
-__global__ void k_bicg_alpha(double *sc);
-__global__ void k_bicg_s(int64_t n, const double *sc, const double *r, const double *v, double *s);
-__global__ void k_bicg_half(int64_t n, const double *sc, const double *p, double *y);
-__global__ void k_bicg_omega(double *sc);
-__global__ void k_bicg_update(int64_t n, const double *sc, const double *p, const double *s, const double *t,
-                              double *y, double *r);
-__global__ void k_bicg_shift(double *sc);
-__global__ void k_bicg_init(int64_t n, const double *b, double *r, double *rhat, double *p, double *v, double *y,
-                            double *sc);
-__global__ void k_axpy_sub(int64_t n, const double *b, const double *ax, double *out);
 
 // FMA-chain peak (peak_kernels.cu)
 cudaError_t run_peak_fma(bool fp64, cudaStream_t st, double *flops_per_s);

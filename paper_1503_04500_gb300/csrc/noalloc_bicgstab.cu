@@ -36,7 +36,7 @@
 namespace rsai {
 
 constexpr int64_t kNoAllocMaxN = 65536;
-constexpr int64_t kNoAllocPartials = 512;  // >= the dot kernels' partial sums
+constexpr int64_t kNoAllocPartials = 2048;  // >= the dot products' partial sums and the control block
 constexpr int64_t kNoAllocWords = 9 * kNoAllocMaxN + kNoAllocPartials + 16;
 
 static __device__ __align__(256) double g_noalloc_scratch[kNoAllocWords];

@@ -1,0 +1,78 @@
+"""rsai_spmv and rsai_bicgstab at the edges of their work splits (groups of four rows, blocks
+of 256 rows, rounds of 304 blocks), against NumPy."""
+import numpy as np
+import pytest
+
+from paper_1503_04500_gb300 import inputs as gen
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+rsai = pytest.importorskip("paper_1503_04500_gb300.rsai")
+
+
+def matvec(A, x):
+    rows = np.repeat(np.arange(A.n), np.diff(A.row_ptr))
+    return np.bincount(rows, weights=A.val * x[A.col_idx], minlength=A.n)
+
+
+def reference(A, apply_M, b, rtol, maxit):
+    """Right-preconditioned BiCGStab as Section 5 runs it; returns (x, iterations)."""
+    r = b.copy()
+    y, p, v = np.zeros_like(b), np.zeros_like(b), np.zeros_like(b)
+    rho_old = alpha = omega = 1.0
+    nb = np.linalg.norm(b)
+    for it in range(1, maxit + 1):
+        rho = b @ r
+        p = r + (rho / rho_old) * (alpha / omega) * (p - omega * v)
+        v = matvec(A, apply_M(p))
+        alpha = rho / (b @ v)
+        s = r - alpha * v
+        if np.linalg.norm(s) / nb < rtol:
+            return apply_M(y + alpha * p), it
+        t = matvec(A, apply_M(s))
+        omega = (t @ s) / (t @ t)
+        y = y + alpha * p + omega * s
+        r = s - omega * t
+        if np.linalg.norm(r) / nb < rtol:
+            return apply_M(y), it
+        rho_old = rho
+    return apply_M(y), maxit
+
+
+@pytest.mark.parametrize("preconditioned", [False, True])
+@pytest.mark.parametrize("n", [1, 3, 255, 256, 257, 1000, 77824, 77825])
+def test_products_and_iterations(n, preconditioned):
+    A = gen.from_dense(np.array([[2.0]])) if n == 1 else gen.powerlaw(n, seed=n, dmax=30)
+    dA = rsai.DeviceMatrix.from_host(A)
+    rng = np.random.default_rng(n)
+    b = rng.standard_normal(n)
+    h, apply_M = None, lambda z: z
+    if preconditioned:
+        h = rsai.build(dA, c=1, l_max=1, eps=0.9, tol=1e-3)
+        M = gen.SparseMatrix(n, *(t.cpu().numpy() for t in h.M()), None, None, None, None)
+        apply_M = lambda z: matvec(M, z)  # noqa: E731
+        z = rng.standard_normal(n)
+        y = h.apply(torch.as_tensor(z, device="cuda")).cpu().numpy()
+        np.testing.assert_allclose(y, matvec(M, z), rtol=1e-13, atol=1e-13 * np.abs(y).max())
+    # three iterations are a smooth function of the data on both sides (these matrices, with diagonals
+    # of both signs, need hundreds of iterations without a preconditioner, whose count is decided by
+    # rounding); at n = 1 and 3 the solve is exact before that
+    x, iters, relres, status = rsai.bicgstab(dA, h, torch.as_tensor(b, device="cuda"), rtol=1e-8, maxit=3)
+    ref, ref_iters = reference(A, apply_M, b, 1e-8, 3)
+    assert iters == ref_iters and status == (0 if n <= 3 else 11)
+    x = x.cpu().numpy()
+    np.testing.assert_allclose(x, ref, rtol=1e-9, atol=1e-9 * np.abs(ref).max())
+    np.testing.assert_allclose(relres, np.linalg.norm(b - matvec(A, x)) / np.linalg.norm(b), rtol=1e-9, atol=1e-13)
+
+
+@pytest.mark.parametrize("maxit", [0, 1])
+def test_iteration_limit(maxit):
+    A = gen.powerlaw(500, seed=4, dmax=30)
+    b = np.ones(500)
+    x, iters, relres, status = rsai.bicgstab(rsai.DeviceMatrix.from_host(A), None, torch.as_tensor(b, device="cuda"),
+                                             rtol=1e-14, maxit=maxit)
+    ref, _ = reference(A, lambda z: z, b, 1e-14, maxit)
+    assert status == 11 and iters == maxit
+    np.testing.assert_allclose(x.cpu().numpy(), ref, rtol=1e-10, atol=1e-12)
+    np.testing.assert_allclose(relres, np.linalg.norm(b - matvec(A, x.cpu().numpy())) / np.linalg.norm(b), rtol=1e-10)
