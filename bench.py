@@ -150,7 +150,7 @@ class ClockSampler:
 
 # the sources the bin kernels (k_bin_warp, k_bin_block) are compiled from
 BIN_KERNEL_SOURCES = ("build_kernels.cu", "bin_queue.cuh", "warp_bins.cuh", "cta_bins.cuh", "column.cuh", "team_qr.cuh",
-                      "panel.cuh", "stage_map.cuh", "common.cuh", "warp_small.cuh")
+                      "panel.cuh", "help.cuh", "stage_map.cuh", "common.cuh", "warp_small.cuh")
 
 
 def strip_comments(src: str) -> str:

@@ -152,6 +152,9 @@ __device__ void run_queue(const Team &team, Work<T> &w, const DevA &A, const Dev
             }
         }
         if constexpr (paired) __syncwarp();
+        if constexpr (Team::STAGED) {
+            if (have && me == 0) atomicAdd(w.ho->board.cols_done, 1u);
+        }
     }
     team.sync();
     if (me == 0) {

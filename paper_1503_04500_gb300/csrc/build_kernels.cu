@@ -44,10 +44,12 @@ cudaError_t launch_bin_half(int mode, bool fp32, int grid, int warps, const DevA
 
 cudaError_t launch_bin_block(int mode, bool fp32, int kind, int grid, const DevA &A, const DevParams &P,
                              const Caps &cap, const ColQueue &Q, const ColOut &O, const Frozen &F,
-                             unsigned long long *gctr, bool last, char *gwork, size_t gstride, int bin,
-                             cudaStream_t st) {
-    return fp32 ? launch_block_t<float>(mode, kind, grid, A, P, cap, Q, O, F, gctr, last, gwork, gstride, bin, st)
-                : launch_block_t<double>(mode, kind, grid, A, P, cap, Q, O, F, gctr, last, gwork, gstride, bin, st);
+                             unsigned long long *gctr, bool last, char *gwork, size_t gstride, int bin, void *help,
+                             int owners, cudaStream_t st) {
+    return fp32 ? launch_block_t<float>(mode, kind, grid, A, P, cap, Q, O, F, gctr, last, gwork, gstride, bin, help,
+                                        owners, st)
+                : launch_block_t<double>(mode, kind, grid, A, P, cap, Q, O, F, gctr, last, gwork, gstride, bin, help,
+                                         owners, st);
 }
 
 int occupancy_bin_warp(bool fp32, int warps, const Caps &cap) {

@@ -59,7 +59,9 @@ template <typename T> struct Work {
     // s <= j - j0.  A reflector factored on its own is a panel of one, T = tau.
     T *Tst;
     int32_t *pnb;
-    char *stage = nullptr;  // panel staging area (shared memory), not part of the carved workspace
+    // not part of the carved workspace (global-memory bins):
+    char *stage = nullptr;    // panel staging area (shared memory)
+    HelpOwner *ho = nullptr;  // sharing of the trailing updates
 
     __host__ __device__ static size_t align16(size_t x) { return (x + 15) & ~size_t(15); }
     __host__ __device__ static size_t bytes(const Caps &c) {
@@ -487,7 +489,7 @@ template <class Team, typename T> struct Column {
                 if (p >= 2 * kPanel) {
                     staged = true;
                     rank_flag = qr_solve_staged<Team, T>(team, w.B, q, p, w.rhs, w.vhead, w.tau, small, (T *)w.stage,
-                                                         cap.stage_bytes, w.Tst, w.pnb, 0);
+                                                         cap.stage_bytes, w.Tst, w.pnb, w.ho, 0);
                 }
             }
             if (!staged) {
@@ -908,11 +910,11 @@ template <class Team, typename T> struct Column {
         bool staged = false;
         if constexpr (Team::STAGED) {
             qr_update_apply_staged<Team, T>(team, w.B, q, p, qo, po, w.vhead, w.tau, (T *)w.stage, cap.stage_bytes,
-                                            w.Tst, w.pnb);
+                                            w.Tst, w.pnb, w.ho);
             if (p >= 2 * kPanel) {
                 staged = true;
                 qr_solve_staged<Team, T>(team, w.B, q, p, w.qte, w.vhead, w.tau, small, (T *)w.stage,
-                                         cap.stage_bytes, w.Tst, w.pnb, po);
+                                         cap.stage_bytes, w.Tst, w.pnb, w.ho, po);
             }
         } else {
             for (int j = 0; j < po; ++j) update_one_reflector(team, w.B, q, p, qo, po, w.vhead, w.tau, j);

@@ -12,19 +12,29 @@ namespace rsai {
 template <typename T, int NT, bool STAGED, int MINB, int MODE>
 __global__ void __launch_bounds__(NT, MINB)
     k_bin_block(DevA A, DevParams P, Caps cap, ColQueue Q, ColOut O, Frozen F, unsigned long long *gctr,
-                int last_bin, char *gwork, size_t gstride, int bin) {
+                int last_bin, char *gwork, size_t gstride, int bin, void *help, int owners) {
     extern __shared__ __align__(16) char smem[];
     __shared__ unsigned long long red[kVirtualWarps + 1];
     __shared__ int redi[kVirtualWarps + 1];
-    Work<T> w;
-    if constexpr (STAGED) {
-        w.carve(gwork + (size_t)blockIdx.x * gstride, cap);
-        w.stage = smem;  // shared memory is free for panel staging
-    } else {
-        w.carve(smem, cap);
-    }
     BlockTeam<NT, STAGED> team{red, redi};
-    run_queue<MODE>(team, w, A, P, cap, Q, O, F, gctr, last_bin != 0, bin);
+    if constexpr (STAGED) {
+        // CTAs beyond the owners have no workspace: they only help
+        __shared__ HelpOwner ho;
+        if (threadIdx.x == 0) ho = HelpOwner{HelpBoard::at(help, owners), (int)blockIdx.x, 0u, O.err};
+        __syncthreads();
+        if ((int)blockIdx.x < owners) {
+            Work<T> w;
+            w.carve(gwork + (size_t)blockIdx.x * gstride, cap);
+            w.stage = smem;  // shared memory is free for panel staging
+            w.ho = &ho;
+            run_queue<MODE>(team, w, A, P, cap, Q, O, F, gctr, last_bin != 0, bin);
+        }
+        help_others<BlockTeam<NT, STAGED>, T>(team, ho.board, *Q.count, (T *)smem);
+    } else {
+        Work<T> w;
+        w.carve(smem, cap);
+        run_queue<MODE>(team, w, A, P, cap, Q, O, F, gctr, last_bin != 0, bin);
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -33,37 +43,41 @@ __global__ void __launch_bounds__(NT, MINB)
 template <typename T, int NT, bool STAGED, int MINB, int MODE>
 static cudaError_t launch_block_k(int grid, const DevA &A, const DevParams &P, const Caps &cap, const ColQueue &Q,
                                   const ColOut &O, const Frozen &F, unsigned long long *gctr, bool last, char *gwork,
-                                  size_t gstride, int bin, cudaStream_t st) {
+                                  size_t gstride, int bin, void *help, int owners, cudaStream_t st) {
     const size_t smem = STAGED ? (size_t)cap.stage_bytes : Work<T>::bytes(cap);
     allow_full_smem(k_bin_block<T, NT, STAGED, MINB, MODE>);
     k_bin_block<T, NT, STAGED, MINB, MODE><<<grid, NT, smem, st>>>(A, P, cap, Q, O, F, gctr, last ? 1 : 0, gwork,
-                                                                  gstride, bin);
+                                                                  gstride, bin, help, owners);
     return cudaGetLastError();
 }
 
 template <typename T, int MODE>
 static cudaError_t launch_block_m(int kind, int grid, const DevA &A, const DevParams &P, const Caps &cap,
                                   const ColQueue &Q, const ColOut &O, const Frozen &F, unsigned long long *gctr,
-                                  bool last, char *gwork, size_t gstride, int bin, cudaStream_t st) {
+                                  bool last, char *gwork, size_t gstride, int bin, void *help, int owners,
+                                  cudaStream_t st) {
     if (kind == CTA_BIN_SMALL)
         return launch_block_k<T, kSmallThreads, false, kSmallCtas<T>, MODE>(grid, A, P, cap, Q, O, F, gctr, last,
-                                                                            nullptr, 0, bin, st);
+                                                                            nullptr, 0, bin, nullptr, 0, st);
     if (kind == CTA_BIN_SHARED)
         return launch_block_k<T, kBlockThreads, false, 1, MODE>(grid, A, P, cap, Q, O, F, gctr, last, nullptr, 0, bin,
-                                                                st);
+                                                                nullptr, 0, st);
     return launch_block_k<T, kBlockThreads, true, 1, MODE>(grid, A, P, cap, Q, O, F, gctr, last, gwork, gstride, bin,
-                                                           st);
+                                                           help, owners, st);
 }
 
 template <typename T>
 cudaError_t launch_block_t(int mode, int kind, int grid, const DevA &A, const DevParams &P, const Caps &cap,
                            const ColQueue &Q, const ColOut &O, const Frozen &F, unsigned long long *gctr, bool last,
-                           char *gwork, size_t gstride, int bin, cudaStream_t st) {
+                           char *gwork, size_t gstride, int bin, void *help, int owners, cudaStream_t st) {
     if (mode == MODE_BUILD)
-        return launch_block_m<T, MODE_BUILD>(kind, grid, A, P, cap, Q, O, F, gctr, last, gwork, gstride, bin, st);
+        return launch_block_m<T, MODE_BUILD>(kind, grid, A, P, cap, Q, O, F, gctr, last, gwork, gstride, bin, help, owners,
+                                             st);
     if (mode == MODE_REFIT)
-        return launch_block_m<T, MODE_REFIT>(kind, grid, A, P, cap, Q, O, F, gctr, last, gwork, gstride, bin, st);
-    return launch_block_m<T, MODE_BACKWARD>(kind, grid, A, P, cap, Q, O, F, gctr, last, gwork, gstride, bin, st);
+        return launch_block_m<T, MODE_REFIT>(kind, grid, A, P, cap, Q, O, F, gctr, last, gwork, gstride, bin, help, owners,
+                                             st);
+    return launch_block_m<T, MODE_BACKWARD>(kind, grid, A, P, cap, Q, O, F, gctr, last, gwork, gstride, bin, help,
+                                            owners, st);
 }
 
 // CTAs per SM of a bin with its workspace in shared memory
@@ -85,7 +99,7 @@ template <typename T> int occupancy_block_t(int kind, const Caps &cap) {
 #define RSAI_INSTANTIATE_CTA_BINS(T)                                                                                \
     template cudaError_t launch_block_t<T>(int, int, int, const DevA &, const DevParams &, const Caps &,            \
                                            const ColQueue &, const ColOut &, const Frozen &, unsigned long long *,  \
-                                           bool, char *, size_t, int, cudaStream_t);                                \
+                                           bool, char *, size_t, int, void *, int, cudaStream_t);                   \
     template int occupancy_block_t<T>(int, const Caps &);
 
 }  // namespace rsai

@@ -67,8 +67,8 @@ cudaError_t launch_bin_half(int mode, bool fp32, int grid, int warps, const DevA
                             unsigned long long *gctr, bool last, cudaStream_t st);
 cudaError_t launch_bin_block(int mode, bool fp32, int kind, int grid, const DevA &A, const DevParams &P,
                              const Caps &cap, const ColQueue &Q, const ColOut &O, const Frozen &F,
-                             unsigned long long *gctr, bool last, char *gwork, size_t gstride, int bin,
-                             cudaStream_t st);
+                             unsigned long long *gctr, bool last, char *gwork, size_t gstride, int bin, void *help,
+                             int owners, cudaStream_t st);
 // per precision (warp_bins_f32.cu, warp_bins_f64.cu, cta_bins_f32.cu, cta_bins_f64.cu)
 template <typename T>
 cudaError_t launch_warp_t(int mode, int grid, int warps, const DevA &A, const DevParams &P, const Caps &cap,
@@ -81,7 +81,7 @@ cudaError_t launch_half_t(int mode, int grid, int warps, const DevA &A, const De
 template <typename T>
 cudaError_t launch_block_t(int mode, int kind, int grid, const DevA &A, const DevParams &P, const Caps &cap,
                            const ColQueue &Q, const ColOut &O, const Frozen &F, unsigned long long *gctr, bool last,
-                           char *gwork, size_t gstride, int bin, cudaStream_t st);
+                           char *gwork, size_t gstride, int bin, void *help, int owners, cudaStream_t st);
 template <typename T> int occupancy_warp_t(int warps, const Caps &cap);
 template <typename T> int occupancy_half_t(int warps, const Caps &cap);
 template <typename T> int occupancy_block_t(int kind, const Caps &cap);

@@ -10,6 +10,7 @@
 // how many instructions carry them.
 #pragma once
 
+#include "help.cuh"
 #include "team_qr.cuh"
 
 namespace rsai {
@@ -312,6 +313,16 @@ __device__ __forceinline__ void panel_factor(const Team &team, T *V, int qq, int
     team.sync();
 }
 
+__device__ __forceinline__ void prefetch_l2(const void *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+
+// Passes between the loads of C and their prefetch to L2 in wy_apply_cols.  152
+// columns of M have 365 MB of trailing matrices at |I| = 2000, |J| = 300, so
+// the first read of a column misses L2: QR of 152 matrices 2800 x 350, 16.8M
+// cycles without the prefetch, 12.4M with 6 passes, 12.5M with 12; where
+// everything fits L2 it costs 2 %.  Prefetching the second read, which hits, too:
+// 13.6M.
+constexpr int kAhead = 6;
+
 // C <- C - V (T^T (V^T C)) for KC columns tc[0..KC) (rows 0..qq-1 of each;
 // has[x] = false: the column repeats tc[0] and is not stored) on one warp,
 // lanes over rows.  Each chain W(u, c) = sum_r V(r,u) C(r,c) runs over the rows
@@ -355,6 +366,8 @@ __device__ __forceinline__ void wy_apply_cols(const T *V, int qq, int nb, const 
                 if (rn < qq) {
 #pragma unroll
                     for (int x = 0; x < KC; ++x) cb[y][x] = tc[x][rn];
+#pragma unroll
+                    for (int x = 0; x < KC; ++x) prefetch_l2(tc[x] + min(rn + 32 * kAhead, qq - 1));
                 }
                 if constexpr (F32) {
                     f32x2 cc[KC];
@@ -532,6 +545,152 @@ __device__ __forceinline__ void wy_apply_any(const Team &team, const T *V, int q
     else wy_apply<false, Team, T>(team, V, qq, nb, tm, B, q, p, rhs, j0, c_lo, c_hi);
 }
 
+// What a CTA of the global bin needs to share its trailing updates
+struct HelpOwner {
+    HelpBoard board;
+    int slot;        // -1: does not share
+    uint32_t epoch;  // of the last published task
+    int32_t *err;    // the launch's error word
+};
+
+// T of a panel (column t at tcol[t * kPanel]) into tm[s * kPanel + t]
+template <class Team, typename T>
+__device__ __forceinline__ void load_T(const Team &team, const T *tcol, int nb, T *tm) {
+    for (int e = team.rank(); e < kPanel * kPanel; e += Team::SIZE) {
+        const int s = e / kPanel, t = e - s * kPanel;
+        tm[e] = (t < nb && s <= t) ? tcol[t * kPanel + s] : T(0);
+    }
+}
+
+// Columns per group of a shared update: a round of the CTA's warps at two (FP64:
+// one) columns each, about as long as staging the panel takes a helper ten times
+template <class Team, typename T> constexpr int kHelpGroup = Team::SIZE / 32 * (sizeof(T) == 8 ? 1 : 2);
+
+// wy_apply, shared with idle CTAs when there are any (`idle`, as seen by the
+// whole team) and at least three groups.  V and T are staged; vhead, tcol: the
+// panel's heads and T in the workspace.
+template <class Team, typename T>
+__device__ __noinline__ void wy_apply_shared(Team team, HelpOwner *ho, bool idle, const T *V, int qq, int nb,
+                                             const T *tm, T *B, int q, int p, T *rhs, int j0, int c_lo, int c_hi,
+                                             const T *vhead, const T *tcol) {
+    constexpr int kGroup = kHelpGroup<Team, T>;
+    const int groups = (c_hi - c_lo + kGroup) / kGroup;
+    if (!idle || groups < 3 || ho->slot < 0) {
+        wy_apply_any(team, V, qq, nb, tm, B, q, p, rhs, j0, c_lo, c_hi);
+        return;
+    }
+    __shared__ int claimed;
+    HelpBoard &b = ho->board;
+    const int slot = ho->slot;
+    const uint32_t epoch = ho->epoch + 1;
+    team.sync();  // the panel, its heads and T are written
+    if (team.rank() == 0) {
+        b.task[slot] = HelpTask{B + (int64_t)j0 * q + j0, vhead, tcol, B, rhs, q, p, qq, nb, j0, c_lo, c_hi, kGroup};
+        b.done[slot] = 0u;
+        __threadfence();
+        atomicExch(&b.word[slot], (unsigned long long)epoch << 32 | (unsigned long long)groups << 16);
+    }
+    int mine = 0;
+    for (;;) {
+        if (team.rank() == 0) claimed = help_claim(&b.word[slot], epoch);
+        team.sync();
+        const int g = claimed;
+        team.sync();
+        if (g < 0) break;
+        ++mine;
+        const int c0 = c_lo + g * kGroup;
+        wy_apply_any(team, V, qq, nb, tm, B, q, p, rhs, j0, c0, min(c_hi, c0 + kGroup - 1));
+    }
+    // groups that helpers have claimed
+    if (team.rank() == 0) {
+        int ok = 1;
+        for (unsigned polls = 0; help_load(&b.done[slot]) != (uint32_t)(groups - mine); ++polls)
+            if (polls >= kHelpPolls) {
+                set_error(ho->err, RSAI_ERR_TIMEOUT);
+                ok = 0;
+                break;
+            }
+        __threadfence();
+        claimed = ok;
+    }
+    team.sync();
+    ho->epoch = epoch;
+    if (!claimed) ho->slot = -1;
+    team.sync();
+}
+
+// A CTA without a column: groups of other CTAs' updates until all `total`
+// columns of the bin are finished.
+template <class Team, typename T>
+__device__ __noinline__ void help_others(Team team, const HelpBoard &b, uint32_t total, T *stage) {
+    __shared__ int pick, claimed, have_slot;
+    __shared__ uint32_t have_epoch;
+    const int me = team.rank();
+    T *tm = stage;
+    T *V = stage + kStageHead<Team>;
+    if (me == 0) {
+        atomicAdd(b.idle, 1u);
+        have_slot = -1;
+    }
+    for (unsigned polls = 0; polls < kHelpPolls; ++polls) {
+        // the open task with the most groups left (ties: spread over the helpers)
+        int key = -1;
+        uint32_t epoch = 0;
+        const int slot = me < b.slots ? (me + blockIdx.x) % b.slots : -1;
+        if (slot >= 0) {
+            const unsigned long long w = help_load(&b.word[slot]);
+            const int left = help_groups(w) - help_next(w);
+            if (left > 0) key = left * 1024 + me;
+            epoch = help_epoch(w);
+        }
+        const int best = team.maxv(key);
+        if (best < 0) {
+            if (me == 0) {
+                pick = help_load(b.cols_done) >= total ? 1 : 0;
+                if (!pick) __nanosleep(400);
+            }
+            team.sync();
+            const bool stop = pick != 0;
+            team.sync();
+            if (stop) break;
+            continue;
+        }
+        if (key == best) {
+            pick = slot;
+            const int g = help_claim(&b.word[slot], epoch);
+            claimed = g;
+            if (g >= 0 && (have_slot != slot || have_epoch != epoch)) {
+                have_slot = slot;
+                have_epoch = epoch;
+                claimed = g | 1 << 20;  // stage the panel first
+            }
+        }
+        team.sync();
+        const int got = claimed, sl = pick;
+        team.sync();
+        if (got < 0) continue;
+        polls = 0;
+        const int g = got & 0xfffff;
+        const HelpTask *tk = &b.task[sl];
+        const int q = __ldcg(&tk->q), p = __ldcg(&tk->p), qq = __ldcg(&tk->qq), nb = __ldcg(&tk->nb);
+        const int j0 = __ldcg(&tk->j0), c_lo = __ldcg(&tk->c_lo), c_hi = __ldcg(&tk->c_hi), group = __ldcg(&tk->group);
+        T *B = (T *)__ldcg((const unsigned long long *)&tk->B);
+        T *rhs = (T *)__ldcg((const unsigned long long *)&tk->rhs);
+        if (got >> 20) {
+            panel_stage(team, (const T *)__ldcg((const unsigned long long *)&tk->src), (int64_t)q, V, qq, nb,
+                        (const T *)__ldcg((const unsigned long long *)&tk->heads));
+            load_T(team, (const T *)__ldcg((const unsigned long long *)&tk->tcol), nb, tm);
+            team.sync();
+        }
+        const int c0 = c_lo + g * group;
+        wy_apply_any(team, V, qq, nb, tm, B, q, p, rhs, j0, c0, min(c_hi, c0 + group - 1));
+        if (me == 0) {
+            __threadfence();
+            atomicAdd(&b.done[sl], 1u);
+        }
+    }
+}
+
 // rhs <- Q^T rhs with the reflectors in the panels they were factored in
 // (pnb, Tst): per panel w = V^T rhs (one CTA reduction), y = T^T w, and
 // rhs <- rhs - V y, with V = the explicit reflectors (vhead on the diagonal,
@@ -630,23 +789,22 @@ __device__ __noinline__ void apply_qt_panels(Team team, const T *B, int q, int p
 // trailing column and the right-hand side get
 //   C <- C - V (T^T (V^T C)),  H_1...H_nb = I - V T V^T,
 // so the trailing matrix in global memory is streamed once per panel instead
-// of once per reflector.  Each panel's size and T are kept (pnb, Tst) for the QR
-// update and the refinement.  A panel that does not fit four columns falls back
-// to single Householder steps (panels of one).  j_start > 0 factors only
-// columns j_start..p-1 (the columns appended to a factor whose first j_start
-// columns are done, Section 3).  Leaves Q^T rhs in rhs; the rank flag is valid
-// on warp 0.
-//
-// One CTA per column of M and SM: what bounds it is the issue rate of the
-// trailing update and the latency of the panel steps, not memory.
+// of once per reflector (by this CTA and, when others have run out of columns,
+// by them: wy_apply_shared).  Each panel's size and T are kept (pnb, Tst) for
+// the QR update and the refinement.  A panel that does not fit four columns
+// falls back to single Householder steps (panels of one).  j_start > 0 factors
+// only columns j_start..p-1 (the columns appended to a factor whose first
+// j_start columns are done, Section 3).  Leaves Q^T rhs in rhs; the rank flag is
+// valid on warp 0.
 template <class Team, typename T>
 __device__ __noinline__ int qr_solve_staged(Team team, T *B, int q, int p, T *rhs, T *vhead, T *taus, T small,
-                                            T *stage, int stage_bytes, T *Tst, int32_t *pnb, int j_start) {
+                                            T *stage, int stage_bytes, T *Tst, int32_t *pnb, HelpOwner *ho,
+                                            int j_start) {
     const int me = team.rank();
     constexpr int NW = Team::SIZE / 32;
     T *tm = stage;                                  // kPanel x kPanel
     T *red = stage + kPanel * kPanel;               // reduction slots
-    T *flag = red + NW * kPanel, *f = flag + kPanel;
+    T *flag = red + NW * kPanel, *f = flag + kPanel;  // flag[0]: tau of the last step, flag[1]: idle CTAs
     T *V = stage + kStageHead<Team>;
     const int64_t velems = (int64_t)stage_bytes / (int64_t)sizeof(T) - kStageHead<Team>;
     int rank_flag = 0;
@@ -665,7 +823,9 @@ __device__ __noinline__ int qr_solve_staged(Team team, T *B, int q, int p, T *rh
             continue;
         }
         T *src = B + (int64_t)j0 * q + j0;
+        const uint32_t idle = me == 0 ? *(volatile uint32_t *)ho->board.idle : 0u;
         panel_stage(team, src, q, V, qq, nb, (const T *)nullptr);
+        if (me == 0) flag[1] = idle ? T(1) : T(0);
         team.sync();
         panel_factor(team, V, qq, nb, src, q, vhead + j0, taus + j0, tm, red, flag, f, small, rank_flag);
         for (int e = me; e < nb * kPanel; e += Team::SIZE) {
@@ -673,7 +833,8 @@ __device__ __noinline__ int qr_solve_staged(Team team, T *B, int q, int p, T *rh
             Tst[(int64_t)(j0 + t) * kPanel + s2] = (s2 <= t) ? tm[s2 * kPanel + t] : T(0);
         }
         if (me == 0) pnb[j0] = nb;
-        wy_apply_any(team, V, qq, nb, tm, B, q, p, rhs, j0, j0 + nb, p);
+        wy_apply_shared(team, ho, flag[1] != T(0), V, qq, nb, tm, B, q, p, rhs, j0, j0 + nb, p, vhead + j0,
+                        Tst + (int64_t)j0 * kPanel);
         j0 += nb;
     }
     return rank_flag;
@@ -689,9 +850,10 @@ __device__ __noinline__ int qr_solve_staged(Team team, T *B, int q, int p, T *rh
 template <class Team, typename T>
 __device__ __noinline__ void qr_update_apply_staged(Team team, T *B, int q, int p, int q0, int p0, const T *vhead,
                                                     const T *taus, T *stage, int stage_bytes, const T *Tst,
-                                                    const int32_t *pnb) {
+                                                    const int32_t *pnb, HelpOwner *ho) {
     const int me = team.rank();
     T *tm = stage;
+    T *flag = stage + kPanel * kPanel + Team::SIZE / 32 * kPanel;
     T *V = stage + kStageHead<Team>;
     const int64_t velems = (int64_t)stage_bytes / (int64_t)sizeof(T) - kStageHead<Team>;
     int j0 = 0;
@@ -707,13 +869,14 @@ __device__ __noinline__ void qr_update_apply_staged(Team team, T *B, int q, int 
                 ++js;
                 continue;
             }
+            const T *tcol = Tst + (int64_t)j1 * kPanel + js;
+            const uint32_t idle = me == 0 ? *(volatile uint32_t *)ho->board.idle : 0u;
             panel_stage(team, B + (int64_t)j1 * q + j1, (int64_t)q, V, qq, ns, vhead + j1);
-            for (int e = me; e < kPanel * kPanel; e += Team::SIZE) {
-                const int s2 = e / kPanel, t = e - s2 * kPanel;
-                tm[e] = (t < ns && s2 <= t) ? Tst[(int64_t)(j1 + t) * kPanel + js + s2] : T(0);
-            }
+            load_T(team, tcol, ns, tm);
+            if (me == 0) flag[1] = idle ? T(1) : T(0);
             team.sync();
-            wy_apply_any(team, V, qq, ns, tm, B, q, p, (T *)nullptr, j1, p0, p - 1);
+            wy_apply_shared(team, ho, flag[1] != T(0), V, qq, ns, tm, B, q, p, (T *)nullptr, j1, p0, p - 1,
+                            vhead + j1, tcol);
             js += ns;
         }
         j0 += nb;

@@ -92,7 +92,9 @@ struct rsai_handle {
     // bin G slab
     char *gwork = nullptr;
     size_t gstride = 0;
-    int grid_g = 0;
+    int grid_g = 0;         // owners: CTAs with a workspace
+    int launch_g = 0;       // CTAs launched: the others only help
+    char *help = nullptr;   // HelpBoard of up to one owner per SM
     // bins
     Caps capH{}, capW{}, capW2{}, capS{}, capC{}, capG{};
     int grid_h = 0, grid_w = 0, grid_w2 = 0, warps_w2 = 0, grid_s = 0, grid_c = 0;
@@ -274,10 +276,10 @@ cudaError_t enqueue_bins(rsai_handle *h, int mode, const DevA &A, const Frozen &
     if (e != cudaSuccess) return e;
     if (ev) cudaEventRecord(ev[2], st);
     e = launch_bin_block(mode, fp32, CTA_BIN_SMALL, h->grid_s, A, P, h->capS, QS, O, F, gctr, false, nullptr, 0, 1,
-                         st);
+                         nullptr, 0, st);
     if (e != cudaSuccess) return e;
     e = launch_bin_block(mode, fp32, CTA_BIN_SHARED, h->grid_c, A, P, h->capC, QC, O, F, gctr, false, nullptr, 0, 1,
-                         st);
+                         nullptr, 0, st);
     if (e != cudaSuccess) return e;
     if (before_global) {
         const int hr = before_global(h, st);
@@ -292,7 +294,9 @@ cudaError_t enqueue_bins(rsai_handle *h, int mode, const DevA &A, const Frozen &
     k_cost_scatter<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(h->ovf3, h->qnext + 6, h->cost_bucket, h->cost_hist,
                                                                  h->ovf3_sorted);
     if (ev) cudaEventRecord(ev[3], st);
-    e = launch_bin_block(mode, fp32, CTA_BIN_GLOBAL, h->grid_g, A, P, h->capG, QG, O, F, gctr, true, h->gwork, h->gstride, 2, st);
+    cudaMemsetAsync(h->help, 0, HelpBoard::bytes(h->grid_g), st);
+    e = launch_bin_block(mode, fp32, CTA_BIN_GLOBAL, h->launch_g, A, P, h->capG, QG, O, F, gctr, true, h->gwork,
+                         h->gstride, 2, h->help, h->grid_g, st);
     return e;
 }
 
@@ -434,7 +438,7 @@ int plan_bins(rsai_handle *h) {
     // bin G: a global-memory slab per CTA, one CTA per SM
     h->capG = Caps{32768, 4096, 131072, 8192, (int64_t)1 << 24, 0, 0, max_optin - 2048, 1, 32768, spai};
     h->gstride = ((fp32 ? work_bytes<float>(h->capG) : work_bytes<double>(h->capG)) + 255) & ~size_t(255);
-    h->grid_g = 1;  // sized by the first build (size_global_slab)
+    h->grid_g = h->launch_g = 1;  // sized by the first build (size_global_slab)
     return RSAI_OK;
 }
 
@@ -509,6 +513,8 @@ int size_global_slab(rsai_handle *h, cudaStream_t st) {
         return RSAI_ERR_CUDA;
     int want = std::max(1, std::min(h->sms, (int)cnt));
     if (h->tuning.global_bin_ctas > 0) want = std::min(h->tuning.global_bin_ctas, h->sms);
+    // every SM helps the columns that are left at the end
+    h->launch_g = std::max(h->launch_g, h->tuning.global_bin_ctas > 0 ? want : cnt > 0 ? h->sms : 1);
     if (want <= h->grid_g) return RSAI_OK;
     // the larger slab first, so that a failed allocation leaves the old one in place
     char *slab = nullptr;
@@ -584,6 +590,7 @@ int build_common(rsai_handle *h, cudaStream_t st) {
     h->scan_tmp_len = (n + 1023) / 1024 + 2;
     TRY(dalloc(h, &h->scan_tmp, h->scan_tmp_len, st));
     TRY(dalloc(h, &h->gwork, h->gstride * (size_t)h->grid_g, st));
+    TRY(dalloc(h, &h->help, HelpBoard::bytes(h->sms), st));
     int status = RSAI_OK;
     {
         Nvtx range("rsai: first build");
@@ -1182,7 +1189,7 @@ rsai_status rsai_set_tuning(rsai_handle *h, const rsai_tuning *t) {
             if (h->gwork) dfree(h, h->gwork, st);
             h->gwork = slab;
         }
-        h->grid_g = want;
+        h->grid_g = h->launch_g = want;
     }
     if (h->graph) {  // the launch shapes are part of the recorded graph
         cudaGraphExecDestroy(h->graph);
