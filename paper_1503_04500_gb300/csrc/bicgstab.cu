@@ -107,6 +107,7 @@ __device__ void product_own(const Solve &S, const CsrView &A, const double *x, d
 struct Shared {
     double x[2][4][kDotThreads], y[2][4][kDotThreads];
     double tree[2][kDotThreads];
+    double scalar;
 };
 
 // f(i, x, y) over the elements that this block owns (all threads; x and y get
@@ -179,6 +180,16 @@ __device__ double grid_total(const double *partials, Shared &sh) {
     return v;
 }
 
+// f() by one thread, its value to all.  An FP64 division or square root by
+// every thread of the grid would take the FP64 units longer than a product with A.
+template <typename F> __device__ __forceinline__ double block_scalar(Shared &sh, F f) {
+    if (threadIdx.x == 0) sh.scalar = f();
+    __syncthreads();
+    const double v = sh.scalar;
+    __syncthreads();
+    return v;
+}
+
 // f(i) over the elements that this block owns, all threads
 template <typename F> __device__ void own_elements(const Solve &S, F f) {
     constexpr int G = kThreads / kDotThreads;
@@ -214,7 +225,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_bicgstab(Solve S) {
     RSAI_SYNC();
     // r = rhat = b: (rhat,r) is also (b,b)
     double rho = grid_total(P + D_RHO * kDotBlocks, sh);
-    const double nb = sqrt(rho);
+    const double nb = block_scalar(sh, [&] { return sqrt(rho); });
     if (nb == 0.0) {
         own_elements(S, [&](int64_t i) { S.x[i] = 0.0; });
         if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -227,8 +238,8 @@ __global__ void __launch_bounds__(kThreads, 2) k_bicgstab(Solve S) {
     double rho_old = 1.0, alpha = 1.0, omega = 1.0;
     int status = RSAI_ERR_NOT_CONVERGED, it = 1;
     for (; it <= S.maxit; ++it) {
+        const double beta = block_scalar(sh, [&] { return (rho / rho_old) * (alpha / omega); });
         own_elements(S, [&](int64_t i) {
-            const double beta = (rho / rho_old) * (alpha / omega);
             S.p[i] = S.r[i] + beta * (S.p[i] - omega * S.v[i]);
         });
         const double *Mp = S.p;
@@ -245,7 +256,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_bicgstab(Solve S) {
         });
         RSAI_SYNC();
         const double rv = grid_total(P + D_RV * kDotBlocks, sh);
-        alpha = rho / rv;
+        alpha = block_scalar(sh, [&] { return rho / rv; });
         chains<1>(S, sh, {D_SS}, [&](int64_t i, double (&a)[1], double (&c)[1]) {
             const double si = S.r[i] - alpha * S.v[i];
             S.s[i] = si;
@@ -255,7 +266,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_bicgstab(Solve S) {
         const double ss = grid_total(P + D_SS * kDotBlocks, sh);
         // rho = r^T r = 0, or r^T v = 0 (alpha undefined): the recurrences break down
         if (rho == 0.0 || rv == 0.0) { status = RSAI_ERR_BREAKDOWN; break; }
-        if (sqrt(ss) / nb < S.rtol) {
+        if (block_scalar(sh, [&] { return sqrt(ss) / nb; }) < S.rtol) {
             own_elements(S, [&](int64_t i) { S.y[i] += alpha * S.p[i]; });
             status = RSAI_OK;
             break;
@@ -274,7 +285,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_bicgstab(Solve S) {
         RSAI_SYNC();
         const double ts = grid_total(P + D_TS * kDotBlocks, sh), tt = grid_total(P + D_TT * kDotBlocks, sh);
         if (tt == 0.0) { status = RSAI_ERR_BREAKDOWN; break; }
-        omega = ts / tt;
+        omega = block_scalar(sh, [&] { return ts / tt; });
         chains<2>(S, sh, {D_RR, D_RHO}, [&](int64_t i, double (&a)[2], double (&c)[2]) {
             S.y[i] += alpha * S.p[i] + omega * S.s[i];
             const double ri = S.s[i] - omega * S.t[i];
@@ -284,7 +295,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_bicgstab(Solve S) {
         });
         RSAI_SYNC();
         const double rr = grid_total(P + D_RR * kDotBlocks, sh);
-        if (sqrt(rr) / nb < S.rtol) { status = RSAI_OK; break; }
+        if (block_scalar(sh, [&] { return sqrt(rr) / nb; }) < S.rtol) { status = RSAI_OK; break; }
         if (omega == 0.0) { status = RSAI_ERR_BREAKDOWN; break; }
         rho_old = rho;
         rho = grid_total(P + D_RHO * kDotBlocks, sh);

@@ -55,14 +55,17 @@ def test_products_and_iterations(n, preconditioned):
         z = rng.standard_normal(n)
         y = h.apply(torch.as_tensor(z, device="cuda")).cpu().numpy()
         np.testing.assert_allclose(y, matvec(M, z), rtol=1e-13, atol=1e-13 * np.abs(y).max())
-    # three iterations are a smooth function of the data on both sides (these matrices, with diagonals
-    # of both signs, need hundreds of iterations without a preconditioner, whose count is decided by
-    # rounding); at n = 1 and 3 the solve is exact before that
+    # three iterations are a smooth function of the data (these matrices, with diagonals of both signs,
+    # need hundreds without a preconditioner, whose count is decided by rounding); at n = 1 and 3 the
+    # solve is exact before that.  The bar is rounding, some ten roundings per sum of n terms, times
+    # the iteration's own sensitivity, from a relative change of 2^-52 in b (n = 1000 is near a breakdown).
     x, iters, relres, status = rsai.bicgstab(dA, h, torch.as_tensor(b, device="cuda"), rtol=1e-8, maxit=3)
     ref, ref_iters = reference(A, apply_M, b, 1e-8, 3)
+    moved, _ = reference(A, apply_M, b * (1 + 2.0**-52), 1e-8, 3)
     assert iters == ref_iters and status == (0 if n <= 3 else 11)
     x = x.cpu().numpy()
-    np.testing.assert_allclose(x, ref, rtol=1e-9, atol=1e-9 * np.abs(ref).max())
+    bar = 1e-10 * np.abs(ref).max() + 30 * np.abs(moved - ref).max()
+    assert np.abs(x - ref).max() <= bar
     np.testing.assert_allclose(relres, np.linalg.norm(b - matvec(A, x)) / np.linalg.norm(b), rtol=1e-9, atol=1e-13)
 
 
