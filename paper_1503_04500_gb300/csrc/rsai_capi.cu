@@ -284,6 +284,9 @@ cudaError_t enqueue_bins(rsai_handle *h, int mode, const DevA &A, const Frozen &
     if (before_global) {
         const int hr = before_global(h, st);
         if (hr != RSAI_OK) return hr == RSAI_ERR_OOM ? cudaErrorMemoryAllocation : cudaErrorUnknown;
+        O.pool_rows = h->pool_rows;
+        O.pool_vals = h->pool_vals;
+        O.pool_cap = h->pool_cap;
     }
     // the columns that reached the global bin, largest first (grids cover n;
     // the device-side count bounds the work)
@@ -435,10 +438,16 @@ int plan_bins(rsai_handle *h) {
     occ = occupancy_bin_block(fp32, CTA_BIN_SHARED, h->capC);
     if (occ < 1) return RSAI_ERR_CUDA;
     h->grid_c = h->sms * occ;
-    // bin G: a global-memory slab per CTA, one CTA per SM
-    h->capG = Caps{32768, 4096, 131072, 8192, (int64_t)1 << 24, 0, 0, max_optin - 2048, 1, 32768, spai};
+    // bin G: a global-memory slab per CTA, one CTA per SM; no set of rows or
+    // columns outgrows n, no list of entries nnz (n = 1111 in FP64: 10 MB per slab
+    // instead of 138)
+    const int64_t n = h->n;
+    const int qg = (int)std::min<int64_t>(32768, n), pg = (int)std::min<int64_t>(4096, n);
+    const int entries = next_pow2((int)std::min<int64_t>(131072, std::max<int64_t>({h->nnz, n, 2 * (int64_t)pg})));
+    h->capG = Caps{qg, pg, std::min(131072, entries), 8192, std::min<int64_t>((int64_t)1 << 24, (int64_t)qg * pg), 0, 0,
+                   max_optin - 2048, 1, qg, spai};
     h->gstride = ((fp32 ? work_bytes<float>(h->capG) : work_bytes<double>(h->capG)) + 255) & ~size_t(255);
-    h->grid_g = h->launch_g = 1;  // sized by the first build (size_global_slab)
+    h->grid_g = h->launch_g = 1;  // sized by the first build (size_global)
     return RSAI_OK;
 }
 
@@ -504,14 +513,64 @@ void rsai_handle_free(rsai_handle *h) {
 
 namespace {
 
-// One CTA of the global bin per column that reached it, up to one per SM: the
-// slab (a few tens of MB per CTA) is sized by the first build only.
-int size_global_slab(rsai_handle *h, cudaStream_t st) {
+// M's arrays for up to c entries, and the scratch of its assembly
+int alloc_m(rsai_handle *h, int64_t c, cudaStream_t st) {
+    int r = dalloc(h, &h->Mrows, c, st);
+    if (r == RSAI_OK) r = dalloc(h, &h->Mvals_csc, c, st);
+    if (r == RSAI_OK) r = dalloc(h, &h->Mcols, c, st);
+    if (r == RSAI_OK) r = dalloc(h, &h->Mvals, c, st);
+    if (r == RSAI_OK) r = dalloc(h, &h->tcols, c, st);
+    if (r == RSAI_OK) r = dalloc(h, &h->tvals, c, st);
+    if (r == RSAI_OK) r = dalloc(h, &h->tsrc, c, st);
+    if (r == RSAI_OK) r = dalloc(h, &h->Mcsc_to_csr, c, st);
+    return r;
+}
+
+// The result pool at `cap` entries, keeping the first `keep`
+int grow_pool(rsai_handle *h, int64_t cap, int64_t keep, cudaStream_t st) {
+    int32_t *nrows = nullptr;
+    double *nvals = nullptr;
+    int rc = dalloc(h, &nrows, cap, st);
+    if (rc == RSAI_OK) rc = dalloc(h, &nvals, cap, st);
+    if (rc != RSAI_OK) return rc;
+    if (cudaMemcpyAsync(nrows, h->pool_rows, sizeof(int32_t) * keep, cudaMemcpyDeviceToDevice, st) != cudaSuccess ||
+        cudaMemcpyAsync(nvals, h->pool_vals, sizeof(double) * keep, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
+        return RSAI_ERR_CUDA;
+    dfree(h, h->pool_rows, st);
+    dfree(h, h->pool_vals, st);
+    h->pool_rows = nrows;
+    h->pool_vals = nvals;
+    h->pool_cap = cap;
+    return RSAI_OK;
+}
+
+// Room in the result pool for a column that reached the global bin: above the
+// mean |J| of these columns on the power-law matrices (150 to 190 entries for n
+// from 1e3 to 1e6).  A column that finds the pool full runs a second time, with
+// the few others as unlucky and nothing else on the GPU: at n = 12000 the rerun
+// of 7 % of the columns took 120 of 495 ms.
+constexpr int64_t kGlobalEntries = 256;
+
+// Before the global bin of a first build: one CTA per column that reached it, up
+// to one per SM (the slab, a few tens of MB per CTA, is sized by the first
+// build only), room for these columns in the result pool, and M's arrays.
+int size_global(rsai_handle *h, cudaStream_t st) {
     uint32_t cnt = 0;
+    unsigned long long top = 0;
     if (cudaMemcpyAsync(&cnt, h->qnext + 6, sizeof(cnt), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+        cudaMemcpyAsync(&top, h->pool_top, sizeof(top), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
         cudaStreamSynchronize(st) != cudaSuccess)
         return RSAI_ERR_CUDA;
-    int want = std::max(1, std::min(h->sms, (int)cnt));
+    const int64_t room = std::min<int64_t>((int64_t)top + (int64_t)cnt * kGlobalEntries, h->n * h->n);
+    if (cnt > 0 && (int64_t)top <= h->pool_cap && room > h->pool_cap) {
+        const int rc = grow_pool(h, room, (int64_t)top, st);
+        if (rc != RSAI_OK) return rc;
+    }
+    if (!h->Mrows) {
+        const int rc = alloc_m(h, h->pool_cap, st);
+        if (rc != RSAI_OK) return rc;
+    }
+    int want = std::max(1, std::min(h->sms, (int)std::min<uint32_t>(cnt, INT32_MAX)));
     if (h->tuning.global_bin_ctas > 0) want = std::min(h->tuning.global_bin_ctas, h->sms);
     // every SM helps the columns that are left at the end
     h->launch_g = std::max(h->launch_g, h->tuning.global_bin_ctas > 0 ? want : cnt > 0 ? h->sms : 1);
@@ -605,20 +664,7 @@ int build_common(rsai_handle *h, cudaStream_t st) {
         h->pool_cap = cap;
         TRY(dalloc(h, &h->pool_rows, cap, st));
         TRY(dalloc(h, &h->pool_vals, cap, st));
-        auto alloc_m = [&](int64_t c) -> int {
-            int r = dalloc(h, &h->Mrows, c, st);
-            if (r == RSAI_OK) r = dalloc(h, &h->Mvals_csc, c, st);
-            if (r == RSAI_OK) r = dalloc(h, &h->Mcols, c, st);
-            if (r == RSAI_OK) r = dalloc(h, &h->Mvals, c, st);
-            if (r == RSAI_OK) r = dalloc(h, &h->tcols, c, st);
-            if (r == RSAI_OK) r = dalloc(h, &h->tvals, c, st);
-            if (r == RSAI_OK) r = dalloc(h, &h->tsrc, c, st);
-            if (r == RSAI_OK) r = dalloc(h, &h->Mcsc_to_csr, c, st);
-            return r;
-        };
-        auto release = [&](void *p) { dfree(h, p, st); };
-        TRY(alloc_m(cap));
-        TRY(cuda_status(enqueue_build(h, st, nullptr, size_global_slab)));
+        TRY(cuda_status(enqueue_build(h, st, nullptr, size_global)));
         int32_t *retry = nullptr;
         constexpr int kMaxRegrow = 6;
         bool settled = false;
@@ -638,19 +684,12 @@ int build_common(rsai_handle *h, cudaStream_t st) {
             const int64_t old_cap = h->pool_cap;
             // new reservations start at `top`; the columns to redo need at most `top`
             cap = std::min<int64_t>((int64_t)(2 * top + 1024), std::max<int64_t>(n * n, (int64_t)top + 1024));
-            int32_t *nrows = nullptr;
-            double *nvals = nullptr;
-            TRY(dalloc(h, &nrows, cap, st));
-            TRY(dalloc(h, &nvals, cap, st));
-            cudaMemcpyAsync(nrows, h->pool_rows, sizeof(int32_t) * old_cap, cudaMemcpyDeviceToDevice, st);
-            cudaMemcpyAsync(nvals, h->pool_vals, sizeof(double) * old_cap, cudaMemcpyDeviceToDevice, st);
-            void *old_bufs[] = {h->pool_rows, h->pool_vals, h->Mrows, h->Mvals_csc, h->Mcols,
-                                h->Mvals, h->tcols, h->tvals, h->tsrc, h->Mcsc_to_csr};
-            for (void *p : old_bufs) release(p);
-            h->pool_rows = nrows;
-            h->pool_vals = nvals;
-            h->pool_cap = cap;
-            TRY(alloc_m(cap));
+            for (void *p : {(void *)h->Mrows, (void *)h->Mvals_csc, (void *)h->Mcols, (void *)h->Mvals, (void *)h->tcols,
+                            (void *)h->tvals, (void *)h->tsrc, (void *)h->Mcsc_to_csr})
+                dfree(h, p, st);
+            h->Mrows = nullptr;
+            TRY(grow_pool(h, cap, old_cap, st));
+            TRY(alloc_m(h, cap, st));
             // the columns that found the pool full run again (from its current top)
             if (!retry) TRY(dalloc(h, &retry, n, st));
             cudaMemsetAsync(h->qnext + 7, 0, sizeof(uint32_t), st);
@@ -660,7 +699,7 @@ int build_common(rsai_handle *h, cudaStream_t st) {
             cudaMemsetAsync(h->row_count, 0, sizeof(int32_t) * (size_t)n, st);
             cudaMemsetAsync(h->cursor, 0, sizeof(int32_t) * (size_t)n, st);
             TRY(cuda_status(enqueue_bins(h, MODE_BUILD, dev_a(h), Frozen{}, h->dscal + kCtr, st, nullptr,
-                                         size_global_slab, retry, h->qnext + 7)));
+                                         size_global, retry, h->qnext + 7)));
             TRY(cuda_status(enqueue_build_tail(h, st, nullptr)));
         }
         // columns still without room in the pool are flagged and counted as failed
