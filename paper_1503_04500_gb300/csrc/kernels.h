@@ -85,11 +85,11 @@ cudaError_t launch_block_t(int mode, int kind, int grid, const DevA &A, const De
 template <typename T> int occupancy_warp_t(int warps, const Caps &cap);
 template <typename T> int occupancy_half_t(int warps, const Caps &cap);
 template <typename T> int occupancy_block_t(int kind, const Caps &cap);
-cudaError_t launch_adjoint_gather(int64_t n, int64_t nnzM, const int64_t *row_ptr, const int32_t *col_idx,
-                                  const int64_t *Mrowptr, const int32_t *Mcols, const int64_t *Mcsc_to_csr,
-                                  int64_t *Mcsr_to_csc, const int64_t *qoff, const int32_t *poolI,
-                                  const double *poolR, const double *poolW, const double *alphaM,
-                                  const double *xM, double *grad, cudaStream_t st);
+cudaError_t launch_adjoint_gather(int64_t n, int64_t nnzA, int64_t nnzM, const int64_t *col_ptr,
+                                  const int32_t *row_idx, const int64_t *csc_to_csr, const int64_t *Mrowptr,
+                                  const int32_t *Mcols, const int64_t *Mcsc_to_csr, int64_t *Mcsr_to_csc,
+                                  const int64_t *qoff, const int32_t *poolI, const double *poolR, const double *poolW,
+                                  const double *alphaM, const double *xM, double *grad, cudaStream_t st);
 int occupancy_bin_warp(bool fp32, int warps, const Caps &cap);
 int occupancy_bin_half(bool fp32, int warps, const Caps &cap);
 int occupancy_bin_block(bool fp32, int kind, const Caps &cap);

@@ -1178,9 +1178,9 @@ rsai_status rsai_backward(rsai_handle *h, const double *A_val, const double *gra
     F.xM = h->xM;
     cudaMemsetAsync(h->err, 0, sizeof(int32_t), st);
     if (enqueue_bins(h, MODE_BACKWARD, A, F, h->fctr, st) != cudaSuccess) return RSAI_ERR_CUDA;
-    if (launch_adjoint_gather(h->n, nnzM, h->row_ptr, h->col_idx, h->Mrowptr, h->Mcols, h->Mcsc_to_csr,
-                              h->Mcsr_to_csc, h->qoff, h->poolI, h->poolR, h->poolW, h->alphaM, h->xM, grad_A,
-                              st) != cudaSuccess)
+    if (launch_adjoint_gather(h->n, h->nnz, nnzM, h->col_ptr, h->row_idx, h->csc_to_csr, h->Mrowptr, h->Mcols,
+                              h->Mcsc_to_csr, h->Mcsr_to_csc, h->qoff, h->poolI, h->poolR, h->poolW, h->alphaM, h->xM,
+                              grad_A, st) != cudaSuccess)
         return RSAI_ERR_CUDA;
     return (rsai_status)finish_frozen(h, st);
 }
