@@ -17,8 +17,8 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 SRC = os.path.join(HERE, "csrc")
 OUT = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT, "librsai.so")
-SOURCES = ["rsai_capi.cu", "cta_bins_f32.cu", "cta_bins_f64.cu", "warp_bins_f32.cu", "warp_bins_f64.cu",
-           "build_kernels.cu", "setup_kernels.cu", "apply_kernels.cu", "bicgstab.cu", "peak_kernels.cu",
+SOURCES = ["rsai_capi.cu", "cta_build_f32.cu", "cta_build_f64.cu", "cta_frozen_f32.cu", "cta_frozen_f64.cu",
+           "warp_build_f32.cu", "warp_build_f64.cu", "warp_frozen_f32.cu", "warp_frozen_f64.cu", "build_kernels.cu", "setup_kernels.cu", "apply_kernels.cu", "bicgstab.cu", "peak_kernels.cu",
            "noalloc_bicgstab.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2"]

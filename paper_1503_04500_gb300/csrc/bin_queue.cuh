@@ -8,24 +8,30 @@
 
 namespace rsai {
 
-// Column k to a larger bin's queue: the next bin, or (a |J| too large) the
-// first one that takes more columns.
-__device__ __forceinline__ void forward_column(const ColQueue &Q, const ColOut &O, int32_t k, bool wide) {
-    const bool to_wide = wide && Q.wide_cols != nullptr;
-    const uint32_t pos = atomicAdd(to_wide ? Q.wide_count : Q.ovf_count, 1u);
-    if ((int64_t)pos < Q.ovf_cap) (to_wide ? Q.wide_cols : Q.ovf_cols)[pos] = k;
+// Column k to a larger bin's queue: the next bin or, where it is known to need
+// |J| = need (0: not known) above wide_from, the first one that takes it.
+__device__ __forceinline__ void forward_column(const ColQueue &Q, const ColOut &O, int32_t k, int need) {
+    int32_t *cols = Q.ovf_cols;
+    uint32_t *count = Q.ovf_count;
+    if (Q.wide[0].cols != nullptr && need > Q.wide_from) {
+        const int w = need <= Q.wide[0].pcap ? 0 : need <= Q.wide[1].pcap ? 1 : 2;
+        cols = Q.wide[w].cols;
+        count = Q.wide[w].count;
+    }
+    const uint32_t pos = atomicAdd(count, 1u);
+    if ((int64_t)pos < Q.ovf_cap) cols[pos] = k;
     else set_error(O.err, RSAI_ERR_WORKSPACE);
 }
 
-template <class Team, typename T>
-__device__ void emit_or_forward(const Team &team, Column<Team, T> &col, int st, const ColQueue &Q,
+template <class Team, typename T, class CapT>
+__device__ void emit_or_forward(const Team &team, Column<Team, T, CapT> &col, int st, const ColQueue &Q,
                                 const ColOut &O, bool last_bin, int bin) {
     const int me = team.rank();
     const int32_t k = col.k;
     Work<T> &w = col.w;
     if (st != COL_DONE) {
         if (!last_bin) {
-            if (me == 0) forward_column(Q, O, k, st == COL_OVERFLOW_J);
+            if (me == 0) forward_column(Q, O, k, st == COL_OVERFLOW_J ? col.need : 0);
         } else if (me == 0) {
             O.col_off[k] = 0;
             O.col_len[k] = 0;
@@ -91,18 +97,18 @@ __device__ void emit_or_forward(const Team &team, Column<Team, T> &col, int st, 
 
 // A frozen-pattern column that does not fit this bin: forward or fail
 __device__ __forceinline__ void forward_frozen(int me, const ColQueue &Q, const ColOut &O, int32_t k,
-                                               bool last_bin, bool wide, long long *ctr) {
+                                               bool last_bin, int need, long long *ctr) {
     if (me != 0) return;
     if (!last_bin) {
-        forward_column(Q, O, k, wide);
+        forward_column(Q, O, k, need);
     } else {
         ctr[CTR_FAILED] += 1;
         set_error(O.err, RSAI_ERR_WORKSPACE);
     }
 }
 
-template <int MODE, class Team, typename T>
-__device__ void run_queue(const Team &team, Work<T> &w, const DevA &A, const DevParams &P, const Caps &cap,
+template <int MODE, class Team, typename T, class CapT>
+__device__ void run_queue(const Team &team, Work<T> &w, const DevA &A, const DevParams &P, const CapT &cap,
                           const ColQueue &Q, const ColOut &O, const Frozen &F, unsigned long long *gctr,
                           bool last_bin, int bin) {
     const int me = team.rank();
@@ -127,7 +133,7 @@ __device__ void run_queue(const Team &team, Work<T> &w, const DevA &A, const Dev
         }
         if (have) {
             const int32_t k = Q.cols ? Q.cols[idx] : (int32_t)idx;
-            Column<Team, T> col(team, A, P, cap, w, k);
+            Column<Team, T, CapT> col(team, A, P, cap, w, k);
             if constexpr (MODE == MODE_BUILD) {
                 int st = col.run();
                 emit_or_forward(team, col, st, Q, O, last_bin, bin);
@@ -140,7 +146,7 @@ __device__ void run_queue(const Team &team, Work<T> &w, const DevA &A, const Dev
                     else ok = col.adjoint(F);
                 }
                 if (!ok) {
-                    forward_frozen(me, Q, O, k, last_bin, pk > cap.pcap, w.ctr);
+                    forward_frozen(me, Q, O, k, last_bin, pk > cap.pcap ? pk : 0, w.ctr);
                 } else {
                     if constexpr (MODE == MODE_REFIT) {
                         for (int c = me; c < pk; c += Team::SIZE) F.Mval_csr[F.Mcsc_to_csr[mo + c]] = w.m[c];

@@ -28,28 +28,44 @@ size_t work_bytes(const Caps &c) { return Work<T>::bytes(c); }
 template size_t work_bytes<float>(const Caps &);
 template size_t work_bytes<double>(const Caps &);
 
+template <typename T, typename... Args> static cudaError_t warp_by_mode(int mode, Args &&...a) {
+    if (mode == MODE_BUILD) return launch_warp_m<T, MODE_BUILD>(a...);
+    if (mode == MODE_REFIT) return launch_warp_m<T, MODE_REFIT>(a...);
+    return launch_warp_m<T, MODE_BACKWARD>(a...);
+}
+template <typename T, typename... Args> static cudaError_t half_by_mode(int mode, Args &&...a) {
+    if (mode == MODE_BUILD) return launch_half_m<T, MODE_BUILD>(a...);
+    if (mode == MODE_REFIT) return launch_half_m<T, MODE_REFIT>(a...);
+    return launch_half_m<T, MODE_BACKWARD>(a...);
+}
+template <typename T, typename... Args> static cudaError_t block_by_mode(int mode, Args &&...a) {
+    if (mode == MODE_BUILD) return launch_block_m<T, MODE_BUILD>(a...);
+    if (mode == MODE_REFIT) return launch_block_m<T, MODE_REFIT>(a...);
+    return launch_block_m<T, MODE_BACKWARD>(a...);
+}
+
 cudaError_t launch_bin_warp(int mode, bool fp32, int grid, int warps, const DevA &A, const DevParams &P,
                             const Caps &cap, const ColQueue &Q, const ColOut &O, const Frozen &F,
                             unsigned long long *gctr, bool last, cudaStream_t st) {
-    return fp32 ? launch_warp_t<float>(mode, grid, warps, A, P, cap, Q, O, F, gctr, last, st)
-                : launch_warp_t<double>(mode, grid, warps, A, P, cap, Q, O, F, gctr, last, st);
+    return fp32 ? warp_by_mode<float>(mode, grid, warps, A, P, cap, Q, O, F, gctr, last, st)
+                : warp_by_mode<double>(mode, grid, warps, A, P, cap, Q, O, F, gctr, last, st);
 }
 
 cudaError_t launch_bin_half(int mode, bool fp32, int grid, int warps, const DevA &A, const DevParams &P,
                             const Caps &cap, const ColQueue &Q, const ColOut &O, const Frozen &F,
                             unsigned long long *gctr, bool last, cudaStream_t st) {
-    return fp32 ? launch_half_t<float>(mode, grid, warps, A, P, cap, Q, O, F, gctr, last, st)
-                : launch_half_t<double>(mode, grid, warps, A, P, cap, Q, O, F, gctr, last, st);
+    return fp32 ? half_by_mode<float>(mode, grid, warps, A, P, cap, Q, O, F, gctr, last, st)
+                : half_by_mode<double>(mode, grid, warps, A, P, cap, Q, O, F, gctr, last, st);
 }
 
 cudaError_t launch_bin_block(int mode, bool fp32, int kind, int grid, const DevA &A, const DevParams &P,
                              const Caps &cap, const ColQueue &Q, const ColOut &O, const Frozen &F,
                              unsigned long long *gctr, bool last, char *gwork, size_t gstride, int bin, void *help,
                              int owners, cudaStream_t st) {
-    return fp32 ? launch_block_t<float>(mode, kind, grid, A, P, cap, Q, O, F, gctr, last, gwork, gstride, bin, help,
-                                        owners, st)
-                : launch_block_t<double>(mode, kind, grid, A, P, cap, Q, O, F, gctr, last, gwork, gstride, bin, help,
-                                         owners, st);
+    return fp32 ? block_by_mode<float>(mode, kind, grid, A, P, cap, Q, O, F, gctr, last, gwork, gstride, bin, help,
+                                       owners, st)
+                : block_by_mode<double>(mode, kind, grid, A, P, cap, Q, O, F, gctr, last, gwork, gstride, bin, help,
+                                        owners, st);
 }
 
 int occupancy_bin_warp(bool fp32, int warps, const Caps &cap) {

@@ -36,7 +36,6 @@ struct Caps {
     int scap;      // sort buffer (power of two)
     int rcap;      // max |R| (dominant rows used so far)
     int64_t bcap;  // max q*p elements of B
-    int hcap;      // slots of the J -> position hash (power of two >= 2*pcap), 0 = none
     int small_p;   // largest |J| solved by the register-resident warp QR (0: never)
     int stage_bytes;  // shared memory for staging QR panels (global-memory bins), 0 = none
     int append;       // CTA bins: room for the kept factor's positions (Section 3)
@@ -44,15 +43,37 @@ struct Caps {
     int spai;         // SPAI selection: a score per candidate column (scap of them)
 };
 
+// Caps of a bin whose sizes are fixed at compile time (no SPAI scores): every address in its workspace is then the warp's base plus a constant, and
+// the workspace is known to be shared memory.
+template <int Q, int P, int S, int R, int D, int APPEND = 0> struct FixedCaps {
+    static constexpr int qcap = Q, pcap = P, scap = S, rcap = R, dcap = D;
+    static constexpr int64_t bcap = (int64_t)Q * P;
+    static constexpr int stage_bytes = 0, append = APPEND, spai = 0;
+    int small_p;
+    // a frozen pass uses neither the set R nor SPAI's scores
+    static bool fits_frozen(const Caps &c) {
+        return c.qcap == Q && c.pcap == P && c.scap == S && c.dcap == D && c.bcap == bcap &&
+               c.stage_bytes == 0 && c.append == APPEND;
+    }
+    static bool fits(const Caps &c) { return fits_frozen(c) && c.rcap == R && c.spai == 0; }
+};
+
 template <typename T> struct Work {
     T *B, *vhead, *tau, *rhs;
     double *m, *r, *z, *wv;
     long long *ctr;
-    int32_t *I, *S, *J, *Jn, *Rset, *buf, *buf2, *Rhat, *hkey, *hval;
+    int32_t *I, *S, *J, *Jn, *Rset, *buf, *buf2, *Rhat;
     int32_t *D;        // columns dropped from J so far, ascending
     double *sc;        // SPAI: the score s_j of each candidate (Caps::spai)
     int32_t *Ip, *Jp;  // factor position of each sorted I / J entry (Caps::append)
     T *qte;            // Q^T e_k(I) of the kept factor, factor row order (Caps::append)
+    // Warp bins: A(I,J) by rows.  Row i of I holds the columns c of J whose bit is
+    // set in rmask[i], ascending; their values in double are the entries
+    // rstart[i], .. of row_vals(), which shares its memory with buf and buf2 and
+    // is valid from a solve until the next use of these.
+    uint32_t *rmask;
+    int32_t *rstart;
+    __device__ __forceinline__ double *row_vals() const { return reinterpret_cast<double *>(buf); }
     // Global-memory bins (Caps::stage_bytes > 0): the reflectors as factored,
     // in panels: pnb[j0] reflectors start at j0, and column j of the panel's
     // compact-WY T (H_j0 ... H_j0+nb-1 = I - V T V^T) is Tst[j * kPanel + s],
@@ -63,8 +84,8 @@ template <typename T> struct Work {
     char *stage = nullptr;    // panel staging area (shared memory)
     HelpOwner *ho = nullptr;  // sharing of the trailing updates
 
-    __host__ __device__ static size_t align16(size_t x) { return (x + 15) & ~size_t(15); }
-    __host__ __device__ static size_t bytes(const Caps &c) {
+    __host__ __device__ static constexpr size_t align16(size_t x) { return (x + 15) & ~size_t(15); }
+    template <class CapT> __host__ __device__ static constexpr size_t bytes(const CapT &c) {
         size_t b = 0;
         b += align16(sizeof(T) * (size_t)c.bcap);
         b += 2 * align16(sizeof(T) * (size_t)c.pcap);
@@ -80,13 +101,14 @@ template <typename T> struct Work {
         b += align16(sizeof(int32_t) * (size_t)c.rcap);
         b += 2 * align16(sizeof(int32_t) * (size_t)c.scap);
         b += align16(sizeof(int32_t) * 32);
-        b += 2 * align16(sizeof(int32_t) * (size_t)c.hcap);
         b += align16(sizeof(int32_t) * (size_t)c.dcap);
         if (c.spai) b += align16(sizeof(double) * (size_t)c.scap);
         if (c.append) {
             b += align16(sizeof(int32_t) * (size_t)c.qcap);
             b += align16(sizeof(int32_t) * (size_t)c.pcap);
             b += align16(sizeof(T) * (size_t)(c.qcap + 1));
+        } else {
+            b += 2 * align16(sizeof(int32_t) * (size_t)c.qcap);
         }
         if (c.stage_bytes > 0) {
             b += align16(sizeof(T) * (size_t)c.pcap * kPanel);
@@ -94,7 +116,7 @@ template <typename T> struct Work {
         }
         return b;
     }
-    __device__ void carve(char *base, const Caps &c) {
+    template <class CapT> __device__ __forceinline__ void carve(char *base, const CapT &c) {
         size_t o = 0;
         B = (T *)(base + o); o += align16(sizeof(T) * (size_t)c.bcap);
         vhead = (T *)(base + o); o += align16(sizeof(T) * (size_t)c.pcap);
@@ -113,8 +135,6 @@ template <typename T> struct Work {
         buf = (int32_t *)(base + o); o += align16(sizeof(int32_t) * (size_t)c.scap);
         buf2 = (int32_t *)(base + o); o += align16(sizeof(int32_t) * (size_t)c.scap);
         Rhat = (int32_t *)(base + o); o += align16(sizeof(int32_t) * 32);
-        hkey = (int32_t *)(base + o); o += align16(sizeof(int32_t) * (size_t)c.hcap);
-        hval = (int32_t *)(base + o); o += align16(sizeof(int32_t) * (size_t)c.hcap);
         D = (int32_t *)(base + o); o += align16(sizeof(int32_t) * (size_t)c.dcap);
         sc = nullptr;
         if (c.spai) {
@@ -126,6 +146,12 @@ template <typename T> struct Work {
             Ip = (int32_t *)(base + o); o += align16(sizeof(int32_t) * (size_t)c.qcap);
             Jp = (int32_t *)(base + o); o += align16(sizeof(int32_t) * (size_t)c.pcap);
             qte = (T *)(base + o); o += align16(sizeof(T) * (size_t)(c.qcap + 1));
+        }
+        rmask = nullptr;
+        rstart = nullptr;
+        if (!c.append) {
+            rmask = (uint32_t *)(base + o); o += align16(sizeof(int32_t) * (size_t)c.qcap);
+            rstart = (int32_t *)(base + o); o += align16(sizeof(int32_t) * (size_t)c.qcap);
         }
         Tst = nullptr;
         pnb = nullptr;
@@ -201,25 +227,11 @@ __device__ __noinline__ int pattern_of_column(Team team, const int64_t *col_ptr,
     return len;
 }
 
-// J -> position in J: an open-addressing hash of J (hcap slots, warp bins)
-// or a binary search of the sorted J (hcap = 0).
+// J -> position in J, by a binary search of the sorted J
 struct JSet {
-    const int32_t *J, *hkey, *hval;
-    int p, hcap;
-    __device__ __forceinline__ unsigned slot(int32_t col) const {
-        return ((unsigned)col * 0x9E3779B1u) >> (32 - __ffs(hcap) + 1);
-    }
-    __device__ __forceinline__ int find(int32_t col) const {
-        if (hcap == 0) return find_i32(J, p, col);
-        const unsigned mask = (unsigned)hcap - 1;
-        unsigned sl = slot(col);
-        for (;;) {
-            const int32_t key = hkey[sl];
-            if (key == col) return hval[sl];
-            if (key == -1) return -1;
-            sl = (sl + 1) & mask;
-        }
-    }
+    const int32_t *J;
+    int p;
+    __device__ __forceinline__ int find(int32_t col) const { return find_i32(J, p, col); }
 };
 
 struct SpaiPick {
@@ -366,14 +378,15 @@ __device__ __noinline__ SpaiPick spai_select(Team team, DevA A, int c, double ti
 }
 
 
-template <class Team, typename T> struct Column {
+template <class Team, typename T, class CapT = Caps> struct Column {
     const Team &team;
     const DevA &A;
     const DevParams &P;
-    const Caps &cap;
+    const CapT &cap;
     Work<T> &w;
     int32_t k;
     int p, q, s, nR, l, nD;
+    int need;  // |J| that did not fit (COL_OVERFLOW_J)
     int64_t q0, p0;
     int rank_flag;
     double rho;
@@ -384,29 +397,10 @@ template <class Team, typename T> struct Column {
     long long c_qr, c_res, c_ref, c_ref64, c_bytes, c_sel;
     int c_solves, c_drops, c_pmax, c_qmax;
 
-    __device__ Column(const Team &t, const DevA &a, const DevParams &pp, const Caps &c, Work<T> &ww, int32_t kk)
+    __device__ Column(const Team &t, const DevA &a, const DevParams &pp, const CapT &c, Work<T> &ww, int32_t kk)
         : team(t), A(a), P(pp), cap(c), w(ww), k(kk) {}
 
-    // J -> position in J: open-addressing hash (warp bins) or binary search.
-    // The table's layout may depend on insertion order; lookups do not.
-    __device__ __forceinline__ JSet jset() const { return JSet{w.J, w.hkey, w.hval, p, cap.hcap}; }
-    __device__ void build_jhash() {
-        if (cap.hcap == 0) return;
-        for (int i = team.rank(); i < cap.hcap; i += Team::SIZE) w.hkey[i] = -1;
-        team.sync();
-        const unsigned mask = (unsigned)cap.hcap - 1;
-        const JSet js = jset();
-        for (int c = team.rank(); c < p; c += Team::SIZE) {
-            const int32_t key = w.J[c];
-            unsigned sl = js.slot(key);
-            for (;;) {
-                int32_t old = atomicCAS(&w.hkey[sl], -1, key);
-                if (old == -1) { w.hval[sl] = c; break; }
-                sl = (sl + 1) & mask;
-            }
-        }
-        team.sync();
-    }
+    __device__ __forceinline__ JSet jset() const { return JSet{w.J, p}; }
     __device__ __forceinline__ int find_J(int32_t col) const { return jset().find(col); }
 
     // The bitmap over indices 0..n-1 in the staging area (global-memory bins;
@@ -637,9 +631,19 @@ template <class Team, typename T> struct Column {
         }
     }
 
-    // S = I u {k}; r = A(:,J) m - e_k on S in double (Eq. 2.4), row by row
-    // through the CSR of A: in ascending j on the warp bins (the oracle's
-    // order), a fixed lane-strided order and butterfly on the CTA bins.
+    // A(I_i, J) x in double, in ascending j (warp bins); *count += its entries
+    __device__ __forceinline__ double row_product(const double *x, int i, int *count) const {
+        const double *v = w.row_vals() + w.rstart[i];
+        double acc = 0.0;
+        uint32_t m = w.rmask[i];
+        *count += __popc(m);
+        for (; m; m &= m - 1u) acc = fma(*v++, x[__ffs(m) - 1], acc);
+        return acc;
+    }
+
+    // S = I u {k}; r = A(:,J) m - e_k on S in double (Eq. 2.4), row by row: from
+    // the rows kept by the solve, in ascending j (the oracle's order), on the warp
+    // bins; through the CSR of A, in row_sums' order, on the CTA bins.
     // `refine`: the residual of a refinement step (counted as refinement work).
     __device__ void residual(bool refine = false) {
         const int me = team.rank();
@@ -661,24 +665,9 @@ template <class Team, typename T> struct Column {
         } else {
             team.sync();
             for (int i = me; i < s; i += Team::SIZE) {
-                const int32_t row = w.S[i];
-                const int64_t e0 = A.row_ptr[row], e1 = A.row_ptr[row + 1];
-                double acc = 0.0;
-                for (int64_t e = e0; e < e1; e += kRowGroup) {
-                    int32_t cj[kRowGroup];
-                    double av[kRowGroup];
-#pragma unroll
-                    for (int u = 0; u < kRowGroup; ++u) {
-                        cj[u] = (e + u < e1) ? A.col_idx[e + u] : -1;
-                        av[u] = (e + u < e1) ? A.val[e + u] : 0.0;
-                    }
-#pragma unroll
-                    for (int u = 0; u < kRowGroup; ++u) {
-                        int pos = (cj[u] >= 0) ? find_J(cj[u]) : -1;
-                        if (pos >= 0) { acc = fma(av[u], w.m[pos], acc); ++cnt; }
-                    }
-                }
-                if (row == k) acc -= 1.0;
+                const bool own = !has_k && i == pk;  // row k, not in I: no entries
+                double acc = own ? 0.0 : row_product(w.m, has_k || i < pk ? i : i - 1, &cnt);
+                if (w.S[i] == k) acc -= 1.0;
                 w.r[i] = acc;
                 if (!refine) ss = fma(acc, acc, ss);
             }
@@ -720,6 +709,86 @@ template <class Team, typename T> struct Column {
         c_qmax = max(c_qmax, q);
     }
 
+    // I = sorted rows of A(:,J) and B = A(I,J) with e_k in rhs, for teams within a warp
+    // (|J| <= their lanes: lane c holds column c): each entry is looked up in I once,
+    // and the rows that the residuals need are kept beside B (row_vals), instead
+    // of walking the rows of A with a search of J per entry: a row holds seven
+    // entries of A and two or three of J on a 3-D stencil.  False on overflow.
+    __device__ __forceinline__ bool gather_lanes(T *fro2s) {
+        const int me = team.rank();
+        int len = 0;
+        int64_t st = 0;
+        if (me < p) {
+            st = A.col_ptr[w.J[me]];
+            len = (int)(A.col_ptr[w.J[me] + 1] - st);
+        }
+        int tot;
+        const int off = team.scan(len, &tot);
+        if (next_pow2(tot) > cap.scap) return false;
+        for (int e = 0; e < len; e += 4) {
+            int32_t v[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) v[u] = (e + u < len) ? A.row_idx[st + e + u] : 0;
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (e + u < len) w.buf[off + e + u] = v[u];
+        }
+        team.sync();
+        team_sort_i32(team, w.buf, tot);
+        const int nq = team_unique_i32(team, w.buf, tot, w.buf2);
+        if (nq > cap.qcap) return false;
+        q = nq;
+        if ((int64_t)q * p > cap.bcap) return false;
+        for (int i = me; i < q; i += Team::SIZE) {
+            const int32_t row = w.buf2[i];
+            w.I[i] = row;
+            w.rhs[i] = row == k ? T(1) : T(0);
+            w.rmask[i] = 0u;
+        }
+        fill_zero(w.B, q * p);
+        team.sync();
+        uint8_t *pos = reinterpret_cast<uint8_t *>(w.wv);  // of every entry in I (|I| <= 128)
+        T fro2 = 0;
+        T *Bc = w.B + (int64_t)me * q;
+        for (int e = 0; e < len; e += 4) {
+            int32_t ri[4];
+            T av[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                ri[u] = (e + u < len) ? A.row_idx[st + e + u] : -1;
+                av[u] = (e + u < len) ? csc_value<T>(A, st + e + u) : T(0);
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                if (ri[u] >= 0) {
+                    const T a = av[u];
+                    const int i = find_i32(w.I, q, ri[u]);
+                    Bc[i] = a;
+                    fro2 += a * a;
+                    pos[off + e + u] = (uint8_t)i;
+                    atomicOr(&w.rmask[i], 1u << me);
+                }
+            }
+        }
+        *fro2s = team.sum(fro2);
+        team.sync();
+        int base = 0;
+        for (int i0 = 0; i0 < q; i0 += Team::SIZE) {
+            const int i = i0 + me;
+            int part;
+            const int at = team.scan(i < q ? __popc(w.rmask[i]) : 0, &part);
+            if (i < q) w.rstart[i] = base + at;
+            base += part;
+        }
+        team.sync();
+        double *rv = w.row_vals();
+        for (int e = 0; e < len; ++e) {
+            const int i = pos[off + e];
+            rv[w.rstart[i] + __popc(w.rmask[i] & ((1u << me) - 1u))] = A.cval[st + e];
+        }
+        return true;
+    }
+
     // x[0..len) = 0 (x 16-byte aligned), 16 bytes per store
     __device__ __forceinline__ void fill_zero(T *x, int len) const {
         constexpr int CW = 16 / (int)sizeof(T);
@@ -754,39 +823,43 @@ template <class Team, typename T> struct Column {
             }
             fact_valid = false;
         }
-        build_jhash();
-        if (!rows_of_J()) return false;
-        if ((int64_t)q * p > cap.bcap) return false;
-        // B = A(I,J), zero-filled
-        fill_zero(w.B, q * p);
-        for (int i = me; i < q; i += Team::SIZE) w.rhs[i] = (w.I[i] == k) ? T(1) : T(0);
-        team.sync();
-        T fro2 = 0;
-        // column by column: column J[c] of A (CSC, the entries rows_of_J has just
-        // read) placed by the position of its rows in I
-        for (int c = me; c < p; c += Team::SIZE) {
-            const int32_t j = w.J[c];
-            const int64_t e0 = A.col_ptr[j], e1 = A.col_ptr[j + 1];
-            T *Bc = w.B + (int64_t)c * q;
-            for (int64_t e = e0; e < e1; e += 4) {
-                int32_t ri[4];
-                T av[4];
+        T fro2s;
+        if constexpr (is_lane_team<Team>::value) {
+            if (!gather_lanes(&fro2s)) return false;
+        } else {
+            if (!rows_of_J()) return false;
+            if ((int64_t)q * p > cap.bcap) return false;
+            // B = A(I,J), zero-filled
+            fill_zero(w.B, q * p);
+            for (int i = me; i < q; i += Team::SIZE) w.rhs[i] = (w.I[i] == k) ? T(1) : T(0);
+            team.sync();
+            T fro2 = 0;
+            // column by column: column J[c] of A (CSC, the entries rows_of_J has just
+            // read) placed by the position of its rows in I
+            for (int c = me; c < p; c += Team::SIZE) {
+                const int32_t j = w.J[c];
+                const int64_t e0 = A.col_ptr[j], e1 = A.col_ptr[j + 1];
+                T *Bc = w.B + (int64_t)c * q;
+                for (int64_t e = e0; e < e1; e += 4) {
+                    int32_t ri[4];
+                    T av[4];
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    ri[u] = (e + u < e1) ? A.row_idx[e + u] : -1;
-                    av[u] = (e + u < e1) ? csc_value<T>(A, e + u) : T(0);
-                }
+                    for (int u = 0; u < 4; ++u) {
+                        ri[u] = (e + u < e1) ? A.row_idx[e + u] : -1;
+                        av[u] = (e + u < e1) ? csc_value<T>(A, e + u) : T(0);
+                    }
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    if (ri[u] >= 0) {
-                        const T a = av[u];
-                        Bc[find_I(ri[u])] = a;
-                        fro2 += a * a;
+                    for (int u = 0; u < 4; ++u) {
+                        if (ri[u] >= 0) {
+                            const T a = av[u];
+                            Bc[find_I(ri[u])] = a;
+                            fro2 += a * a;
+                        }
                     }
                 }
             }
+            fro2s = team.sum(fro2);
         }
-        const T fro2s = team.sum(fro2);
         if constexpr (!is_lane_team<Team>::value) fro2_f = fro2s;
         T fro = sqrt(fro2s);
         team.sync();
@@ -825,7 +898,6 @@ template <class Team, typename T> struct Column {
         for (int b = me; b < nj; b += Team::SIZE) w.Jn[b] = w.buf[b];
         for (int i = me; i < qo; i += Team::SIZE) w.S[i] = w.I[i];
         team.sync();
-        build_jhash();
         if (!rows_of_J()) return 0;
         if ((int64_t)q * p > cap.bcap) return 0;
         if (q < p || q > cap.scap || p > cap.scap) return -1;
@@ -917,7 +989,7 @@ template <class Team, typename T> struct Column {
                                          cap.stage_bytes, w.Tst, w.pnb, w.ho, po);
             }
         } else {
-            for (int j = 0; j < po; ++j) update_one_reflector(team, w.B, q, p, qo, po, w.vhead, w.tau, j);
+            update_reflectors(team, w.B, q, p, qo, po, w.vhead, w.tau, 0, po);
         }
         if (!staged) {
             qr_factor_team<Team, T>(team, w.B, q, p, w.qte, w.vhead, w.tau, small, po);
@@ -1168,7 +1240,8 @@ template <class Team, typename T> struct Column {
     // J = J u Jhat (both sorted, disjoint) by merge ranks
     __device__ bool merge_J(int nj) {
         const int me = team.rank();
-        if (p + nj > cap.pcap) return false;
+        need = p + nj;
+        if (need > cap.pcap) return false;
         for (int a = me; a < p; a += Team::SIZE) w.Jn[a + lower_bound_i32(w.buf, nj, w.J[a])] = w.J[a];
         for (int b = me; b < nj; b += Team::SIZE) w.Jn[b + lower_bound_i32(w.J, p, w.buf[b])] = w.buf[b];
         team.sync();
@@ -1205,6 +1278,12 @@ template <class Team, typename T> struct Column {
 
     // out[i] = sum_c A(I_i, J_c) zc[c] over the rows of I, in double
     __device__ void rows_times(const double *zc, double *out) {
+        if constexpr (is_lane_team<Team>::value) {
+            int entries = 0;
+            for (int i = team.rank(); i < q; i += Team::SIZE) out[i] = row_product(zc, i, &entries);
+            team.sync();
+            return;
+        }
         for (int i = team.rank(); i < q; i += Team::SIZE) {
             const int32_t row = w.I[i];
             const int64_t e0 = A.row_ptr[row], e1 = A.row_ptr[row + 1];
@@ -1270,9 +1349,11 @@ template <class Team, typename T> struct Column {
         normal_solve(small);
         if (P.precision == RSAI_FP32_REFINE) {
             // one refinement step in double: z = z0 + (R^T R)^{-1} (g - B^T B z0);
-            // g stays in z, z0 goes to buf, B z0 to wv, B^T B z0 to buf2
-            double *z0 = reinterpret_cast<double *>(w.buf);
-            double *u = reinterpret_cast<double *>(w.buf2);
+            // g stays in z, B z0 goes to wv, z0 and B^T B z0 to buffers that a frozen
+            // pass does not use otherwise (the warp bins' rows occupy buf and buf2; there
+            // D and R hold at least 2 |J| words)
+            double *z0 = reinterpret_cast<double *>(is_lane_team<Team>::value ? w.D : w.buf);
+            double *u = reinterpret_cast<double *>(is_lane_team<Team>::value ? w.Rset : w.buf2);
             for (int c = me; c < p; c += Team::SIZE) z0[c] = (double)w.rhs[c];
             team.sync();
             rows_times(z0, w.wv);
@@ -1320,6 +1401,11 @@ template <class Team, typename T> struct Column {
             const int32_t r = A.row_idx[e0 + i];
             const double a = A.cval[e0 + i];
             w.I[i] = r;
+            if constexpr (is_lane_team<Team>::value) {
+                w.rmask[i] = 1u;
+                w.rstart[i] = i;
+                w.row_vals()[i] = a;
+            }
             nn = fma(a, a, nn);
             if (r == k) kpos = i;
         }
@@ -1328,7 +1414,6 @@ template <class Team, typename T> struct Column {
         kpos = team.maxv(kpos);
         const double akk = kpos >= 0 ? A.cval[e0 + kpos] : 0.0;
         q = len;
-        build_jhash();
         if (me == 0) w.m[0] = (nn > 0.0) ? akk / nn : 0.0;
         rank_flag = (nn > 0.0) ? 0 : 1;
         c_qr += solve_flops(0, 0, q, 1);
@@ -1354,7 +1439,10 @@ template <class Team, typename T> struct Column {
             // general path below
             long long b = 0;
             const int len = pattern_of_column(team, A.col_ptr, A.row_idx, k, cap.pcap, w.J, &b);
-            if (len < 0) return COL_OVERFLOW_J;
+            if (len < 0) {
+                need = (int)(A.col_ptr[k + 1] - A.col_ptr[k]);
+                return COL_OVERFLOW_J;
+            }
             p = len;
             c_bytes += b;
         } else {

@@ -97,8 +97,10 @@ struct ColQueue {
     int32_t *ovf_cols;        // where columns that outgrow the bin go
     uint32_t *ovf_count;
     int64_t ovf_cap;
-    int32_t *wide_cols;       // columns whose |J| outgrows the bin (NULL: ovf_cols)
-    uint32_t *wide_count;
+    // where columns go that are known to need |J| > wide_from, which the next bin
+    // cannot hold either: the first of these lists whose bin takes their |J|
+    int wide_from;
+    struct { int32_t *cols; uint32_t *count; int pcap; } wide[3];
 };
 
 // ----------------------------------------------------------------------------
@@ -237,10 +239,10 @@ struct WarpTeam {
 // (8 bytes each, holding any reduced type), `redi` as many ints.  STAGED: the
 // bin stages panels in shared memory (its workspace is in global memory).
 //
-// Every CTA size gives the same bits: a float reduction over rows or columns
-// takes one element per thread (the smaller CTAs hold problems of at most NT
-// rows and columns), so it is the same per-warp butterflies, added over the
-// warps in order; the absent warps of a smaller CTA would add zeros.
+// Every CTA size gives the same bits: in the smaller CTAs (at most 128 rows, at
+// most NT columns) a float reduction is over one element per thread of a CTA of
+// 128, the same per-warp butterflies added over the warps in order; the absent
+// warps would add zeros.
 constexpr int kVirtualWarps = 16;
 template <int NT, bool STAGED_ = false> struct BlockTeam {
     static constexpr int SIZE = NT;
@@ -268,6 +270,27 @@ template <int NT, bool STAGED_ = false> struct BlockTeam {
         V s = slot<V>(0);
 #pragma unroll
         for (int w = 1; w < NW; ++w) s += slot<V>(w);
+        return s;
+    }
+    // Sum over the rows of a column, x[v] being this thread's term of virtual warp
+    // wid + NW * v (rows NT * v + rank of the range): one term per thread of a
+    // CTA of VK * NT threads, added in its order.  The CTAs of bins S0 and S
+    // hold at most 128 rows.
+    static constexpr int VK = NT < 128 ? 128 / NT : 1;
+    template <typename V> __device__ __forceinline__ V sum_rows(const V (&x)[VK]) const {
+        if constexpr (VK == 1) return sum(x[0]);
+        V y[VK];
+#pragma unroll
+        for (int v = 0; v < VK; ++v) y[v] = lanes_sum(x[v]);
+        __syncthreads();
+        if ((threadIdx.x & 31) == 0) {
+#pragma unroll
+            for (int v = 0; v < VK; ++v) slot<V>((threadIdx.x >> 5) + NW * v) = y[v];
+        }
+        __syncthreads();
+        V s = slot<V>(0);
+#pragma unroll
+        for (int w = 1; w < NW * VK; ++w) s += slot<V>(w);
         return s;
     }
     template <typename V> __device__ __forceinline__ V maxv(V x) const {

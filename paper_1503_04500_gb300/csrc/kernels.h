@@ -6,14 +6,16 @@
 namespace rsai {
 
 constexpr int kBlockThreads = 512;  // CTA team size of bins C and G (measured: 1.3x faster than 256)
-// Bin S: |I| <= 128 (one row per thread), several CTAs per SM
-constexpr int kSmallThreads = 128;
+// Bins S0 and S: small workspaces, several CTAs per SM
+constexpr int kTinyThreads = 64, kSmallThreads = 128;
+template <typename T> constexpr int kTinyCtas = sizeof(T) == 8 ? 5 : 9;
 template <typename T> constexpr int kSmallCtas = sizeof(T) == 8 ? 3 : 5;
-enum { CTA_BIN_SMALL = 0, CTA_BIN_SHARED = 1, CTA_BIN_GLOBAL = 2 };
+enum { CTA_BIN_TINY = 0, CTA_BIN_SMALL = 1, CTA_BIN_SHARED = 2, CTA_BIN_GLOBAL = 3 };
 constexpr int kWarpsPerCta = 4;     // warps per CTA in bin W
 constexpr int kStatBlocks = 256;    // blocks of the per-column statistics reduction
 // Column counts per bin in the global counters (after the CTR_COUNT work
-// counters): 0 = warp bins W and W2, 1 = CTA bin, 2 = global bin, 3 = bin H
+// counters): 0 = warp bins W0, W and W2, 1 = CTA bins S0, S
+// and C, 2 = global bin, 3 = bin H
 // (also included in 0's total when the statistics are read)
 constexpr int kBinHalf = 3;
 constexpr int kBinSlots = 4;
@@ -69,19 +71,17 @@ cudaError_t launch_bin_block(int mode, bool fp32, int kind, int grid, const DevA
                              const Caps &cap, const ColQueue &Q, const ColOut &O, const Frozen &F,
                              unsigned long long *gctr, bool last, char *gwork, size_t gstride, int bin, void *help,
                              int owners, cudaStream_t st);
-// per precision (warp_bins_f32.cu, warp_bins_f64.cu, cta_bins_f32.cu, cta_bins_f64.cu)
-template <typename T>
-cudaError_t launch_warp_t(int mode, int grid, int warps, const DevA &A, const DevParams &P, const Caps &cap,
-                          const ColQueue &Q, const ColOut &O, const Frozen &F, unsigned long long *gctr, bool last,
-                          cudaStream_t st);
-template <typename T>
-cudaError_t launch_half_t(int mode, int grid, int warps, const DevA &A, const DevParams &P, const Caps &cap,
-                          const ColQueue &Q, const ColOut &O, const Frozen &F, unsigned long long *gctr, bool last,
-                          cudaStream_t st);
-template <typename T>
-cudaError_t launch_block_t(int mode, int kind, int grid, const DevA &A, const DevParams &P, const Caps &cap,
-                           const ColQueue &Q, const ColOut &O, const Frozen &F, unsigned long long *gctr, bool last,
-                           char *gwork, size_t gstride, int bin, void *help, int owners, cudaStream_t st);
+// per precision and mode (warp_build_*.cu, warp_frozen_*.cu, cta_build_*.cu, cta_frozen_*.cu)
+template <typename T, int MODE>
+cudaError_t launch_warp_m(int grid, int warps, const DevA &A, const DevParams &P, const Caps &cap, const ColQueue &Q,
+                          const ColOut &O, const Frozen &F, unsigned long long *gctr, bool last, cudaStream_t st);
+template <typename T, int MODE>
+cudaError_t launch_half_m(int grid, int warps, const DevA &A, const DevParams &P, const Caps &cap, const ColQueue &Q,
+                          const ColOut &O, const Frozen &F, unsigned long long *gctr, bool last, cudaStream_t st);
+template <typename T, int MODE>
+cudaError_t launch_block_m(int kind, int grid, const DevA &A, const DevParams &P, const Caps &cap, const ColQueue &Q,
+                           const ColOut &O, const Frozen &F, unsigned long long *gctr, bool last, char *gwork,
+                           size_t gstride, int bin, void *help, int owners, cudaStream_t st);
 template <typename T> int occupancy_warp_t(int warps, const Caps &cap);
 template <typename T> int occupancy_half_t(int warps, const Caps &cap);
 template <typename T> int occupancy_block_t(int kind, const Caps &cap);

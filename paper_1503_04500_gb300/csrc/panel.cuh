@@ -216,11 +216,8 @@ __device__ __forceinline__ void panel_step(const Team &team, T *V, int qq, int n
         const T sigma = __shfl_sync(0xffffffffu, s, TK);
         const T x0 = panel_at(V, qq, nb, t, t);
         const T cu = u < nb ? panel_at(V, qq, nb, t, u) : T(0);
-        const T nrm = sqrt(sigma);
-        const T alpha = (x0 >= T(0)) ? -nrm : nrm;
-        const T v0 = x0 - alpha;
-        const T vtv = sigma - x0 * x0 + v0 * v0;
-        const T two_over = (vtv > T(0)) ? T(2) / vtv : T(0);
+        T alpha, v0, two_over;
+        reflector(sigma, x0, alpha, v0, two_over);
         __syncwarp();
         if (me < kPanel) {
             if (u == t) {
@@ -241,7 +238,7 @@ __device__ __forceinline__ void panel_step(const Team &team, T *V, int qq, int n
                 }
             }
         }
-        rank_flag |= (fabs(alpha) <= small) ? 1 : 0;
+        rank_flag |= abs_at_most(alpha, small) ? 1 : 0;
     }
     team.sync();
 }
@@ -865,7 +862,7 @@ __device__ __noinline__ void qr_update_apply_staged(Team team, T *B, int q, int 
             const int j1 = j0 + js, qq = q0 - j1;
             const int ns = (int)min((int64_t)(nb - js), qq > 0 ? velems / (int64_t)qq : (int64_t)0);
             if (ns < 4) {
-                update_one_reflector(team, B, q, p, q0, p0, vhead, taus, j1);
+                update_reflectors(team, B, q, p, q0, p0, vhead, taus, j1, j1 + 1);
                 ++js;
                 continue;
             }

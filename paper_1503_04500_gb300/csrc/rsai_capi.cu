@@ -67,9 +67,10 @@ struct rsai_handle {
     // [0..3] queue counters of bins W, W2, C, G; [4..6] overflow counts W->W2,
     // S->C, C->G; [7] columns of a pool-overflow rerun; [8] queue counter of
     // bin H, [9] overflow count H->W; [10] queue counter of bin S, [11]
-    // columns forwarded to it (W and W2)
+    // columns forwarded to it (W and W2); [12] queue counter of bin W0; [13] queue counter of bin
+    // S0, [14] columns forwarded to it
     uint32_t *qnext = nullptr;
-    int32_t *ovf0 = nullptr, *ovf1 = nullptr, *ovf2 = nullptr, *ovf3 = nullptr, *ovf_s = nullptr;
+    int32_t *ovf0 = nullptr, *ovf1 = nullptr, *ovf2 = nullptr, *ovf3 = nullptr, *ovf_s = nullptr, *ovf_s0 = nullptr;
     int32_t *ovf3_sorted = nullptr;  // the global bin's queue, largest column first
     uint8_t *cost_bucket = nullptr;
     uint32_t *cost_hist = nullptr;   // [kCostBuckets]
@@ -96,8 +97,8 @@ struct rsai_handle {
     int launch_g = 0;       // CTAs launched: the others only help
     char *help = nullptr;   // HelpBoard of up to one owner per SM
     // bins
-    Caps capH{}, capW{}, capW2{}, capS{}, capC{}, capG{};
-    int grid_h = 0, grid_w = 0, grid_w2 = 0, warps_w2 = 0, grid_s = 0, grid_c = 0;
+    Caps capH{}, capW0{}, capW{}, capW2{}, capS0{}, capS{}, capC{}, capG{};
+    int grid_h = 0, grid_w0 = 0, grid_w = 0, grid_w2 = 0, warps_w2 = 0, grid_s0 = 0, grid_s = 0, grid_c = 0;
     rsai_tuning tuning{8, 0, kSmallP, 0, 0};
     // refit / backward scratch (allocated on first use)
     double *fval = nullptr, *fcval = nullptr;
@@ -248,26 +249,45 @@ cudaError_t enqueue_bins(rsai_handle *h, int mode, const DevA &A, const Frozen &
                          const int32_t *wlist = nullptr, const uint32_t *wcount = nullptr) {
     const int64_t n = h->n;
     cudaMemsetAsync(h->qnext, 0, sizeof(uint32_t) * 7, st);  // queue and overflow counters; [7] = retry count
-    cudaMemsetAsync(h->qnext + 8, 0, sizeof(uint32_t) * 4, st);
+    cudaMemsetAsync(h->qnext + 8, 0, sizeof(uint32_t) * 7, st);
     const DevParams P = dev_params(h);
     const bool fp32 = h->params.precision == RSAI_FP32_REFINE;
     ColOut O{h->col_off, h->col_len, h->col_q, h->rho, h->loops, h->flags, h->pool_rows, h->pool_vals,
              h->pool_cap, h->pool_top, h->err};
-    // the first bin (H or W) takes the given list (or every column)
-    const bool use_h = h->tuning.half_bin != 0;
-    ColQueue QH{wlist, wcount, n, h->qnext + 8, h->ovf0, h->qnext + 9, h->ovf_cap, nullptr, nullptr};
-    // a column whose |J| outgrows W skips W2, which has the same limit on |J|
-    // and would run it to the same point
-    ColQueue QW{use_h ? h->ovf0 : wlist, use_h ? h->qnext + 9 : wcount, n, h->qnext + 0, h->ovf1, h->qnext + 4,
-                h->ovf_cap, h->ovf_s, h->qnext + 11};
-    ColQueue QW2{h->ovf1, h->qnext + 4, n, h->qnext + 1, h->ovf_s, h->qnext + 11, h->ovf_cap, nullptr, nullptr};
-    ColQueue QS{h->ovf_s, h->qnext + 11, n, h->qnext + 10, h->ovf2, h->qnext + 5, h->ovf_cap, nullptr, nullptr};
-    ColQueue QC{h->ovf2, h->qnext + 5, n, h->qnext + 2, h->ovf3, h->qnext + 6, h->ovf_cap, nullptr, nullptr};
-    ColQueue QG{h->ovf3_sorted, h->qnext + 6, n, h->qnext + 3, nullptr, nullptr, 0, nullptr, nullptr};
+    // the first bin (H, or W0 in FP32, or W) takes the given list (or every
+    // column) and forwards to W through ovf0 / [9]
+    const bool use_h = h->tuning.half_bin != 0, use_w0 = !use_h && h->grid_w0 > 0;
+    const bool first = use_h || use_w0;
+    // Bins W0, W and W2 run the same arithmetic, and so do S0, S and C: a column that
+    // needs more than W's |J| skips W and W2, which would run it to the same
+    // point, and goes to the first CTA bin that takes its |J|.
+    auto queue = [&](const int32_t *cols, const uint32_t *count, int next, int32_t *to, int to_count) {
+        return ColQueue{cols, count, n, h->qnext + next, to, h->qnext + to_count, h->ovf_cap, 0, {}};
+    };
+    auto wide = [&](ColQueue q, int from) {
+        q.wide_from = from;
+        q.wide[0] = {h->ovf_s0, h->qnext + 14, h->capS0.pcap};
+        q.wide[1] = {h->ovf_s, h->qnext + 11, h->capS.pcap};
+        q.wide[2] = {h->ovf2, h->qnext + 5, INT32_MAX};
+        return q;
+    };
+    const ColQueue QW0 = wide(queue(wlist, wcount, 12, h->ovf0, 9), h->capW.pcap);
+    const ColQueue QH = queue(wlist, wcount, 8, h->ovf0, 9);
+    const ColQueue QW =
+        wide(queue(first ? h->ovf0 : wlist, first ? h->qnext + 9 : wcount, 0, h->ovf1, 4), h->capW2.pcap);
+    const ColQueue QW2 = wide(queue(h->ovf1, h->qnext + 4, 1, h->ovf_s0, 14), h->capW2.pcap);
+    const ColQueue QS0 = wide(queue(h->ovf_s0, h->qnext + 14, 13, h->ovf_s, 11), h->capS.pcap);
+    const ColQueue QS = queue(h->ovf_s, h->qnext + 11, 10, h->ovf2, 5);
+    const ColQueue QC = queue(h->ovf2, h->qnext + 5, 2, h->ovf3, 6);
+    const ColQueue QG{h->ovf3_sorted, h->qnext + 6, n, h->qnext + 3, nullptr, nullptr, 0, 0, {}};
     if (ev) cudaEventRecord(ev[1], st);
     cudaError_t e = cudaSuccess;
     if (use_h) {
         e = launch_bin_half(mode, fp32, h->grid_h, h->tuning.warp_bin_warps, A, P, h->capH, QH, O, F, gctr, false, st);
+        if (e != cudaSuccess) return e;
+    }
+    if (use_w0) {
+        e = launch_bin_warp(mode, fp32, h->grid_w0, h->tuning.warp_bin_warps, A, P, h->capW0, QW0, O, F, gctr, false, st);
         if (e != cudaSuccess) return e;
     }
     e = launch_bin_warp(mode, fp32, h->grid_w, h->tuning.warp_bin_warps, A, P, h->capW, QW, O, F, gctr, false, st);
@@ -275,6 +295,9 @@ cudaError_t enqueue_bins(rsai_handle *h, int mode, const DevA &A, const Frozen &
     e = launch_bin_warp(mode, fp32, h->grid_w2, h->warps_w2, A, P, h->capW2, QW2, O, F, gctr, false, st);
     if (e != cudaSuccess) return e;
     if (ev) cudaEventRecord(ev[2], st);
+    e = launch_bin_block(mode, fp32, CTA_BIN_TINY, h->grid_s0, A, P, h->capS0, QS0, O, F, gctr, false, nullptr, 0, 1,
+                         nullptr, 0, st);
+    if (e != cudaSuccess) return e;
     e = launch_bin_block(mode, fp32, CTA_BIN_SMALL, h->grid_s, A, P, h->capS, QS, O, F, gctr, false, nullptr, 0, 1,
                          nullptr, 0, st);
     if (e != cudaSuccess) return e;
@@ -312,7 +335,7 @@ cudaError_t enqueue_build(rsai_handle *h, cudaStream_t st, cudaEvent_t *ev = nul
     if (ev) cudaEventRecord(ev[0], st);
     cudaMemsetAsync(h->dscal, 0, sizeof(unsigned long long) * kScalars, st);
     cudaMemsetAsync(h->err, 0, sizeof(int32_t), st);
-    cudaMemsetAsync(h->qnext, 0, sizeof(uint32_t) * 12, st);
+    cudaMemsetAsync(h->qnext, 0, sizeof(uint32_t) * 15, st);
     cudaMemsetAsync(h->pool_top, 0, sizeof(unsigned long long), st);
     cudaMemsetAsync(h->row_count, 0, sizeof(int32_t) * (size_t)n, st);
     cudaMemsetAsync(h->cursor, 0, sizeof(int32_t) * (size_t)n, st);
@@ -395,13 +418,25 @@ int plan_h(rsai_handle *h, bool fp32) {
     return RSAI_OK;
 }
 
+// launch shape of bin W0 (FP32 only: in FP64 the half-warp bin takes these
+// sizes, and its registers, not the workspace, limit the warp bin's warps per SM)
+int plan_w0(rsai_handle *h, bool fp32) {
+    h->grid_w0 = 0;
+    if (!fp32 || h->capW0.spai) return RSAI_OK;
+    int occ = occupancy_bin_warp(fp32, h->tuning.warp_bin_warps, h->capW0);
+    if (occ < 1) return RSAI_ERR_CUDA;
+    if (h->tuning.warp_bin_ctas_per_sm > 0) occ = std::min(occ, h->tuning.warp_bin_ctas_per_sm);
+    h->grid_w0 = h->sms * occ;
+    return RSAI_OK;
+}
+
 #define TRY_PLAN(x)                        \
     do {                                   \
         const int rc_ = (x);               \
         if (rc_ != RSAI_OK) return rc_;    \
     } while (0)
 
-// choose the capacities of the six bins from the device limits
+// choose the capacities of the eight bins from the device limits
 int plan_bins(rsai_handle *h) {
     const bool fp32 = h->params.precision == RSAI_FP32_REFINE;
     int dev = h->device, max_optin = 0;
@@ -410,26 +445,36 @@ int plan_bins(rsai_handle *h) {
     // bin H: half a warp per column, |I| <= 48, |J| <= 16 (the register QR's
     // three rows per lane), sort buffers of 128 entries
     const int spai = (h->params.flags & RSAI_FLAG_SELECT_SPAI) ? 1 : 0;
-    h->capH = Caps{48, 16, 128, 32, 48 * 16, 32, h->tuning.small_qr_max_p, 0, 0, 32, spai};
+    h->capH = Caps{48, 16, 128, 32, 48 * 16, h->tuning.small_qr_max_p, 0, 0, 32, spai};
     int occ = 0;
     TRY_PLAN(plan_h(h, fp32));
-    h->capW = Caps{64, 32, 256, 64, 64 * 32, 64, h->tuning.small_qr_max_p, 0, 0, 64, spai};
+    // bin W0: the warp bin's algorithm for bin H's sizes: half the workspace, 24
+    // warps per SM instead of 16
+    h->capW0 = h->capH;
+    TRY_PLAN(plan_w0(h, fp32));
+    h->capW = Caps{64, 32, 256, 64, 64 * 32, h->tuning.small_qr_max_p, 0, 0, 64, spai};
     occ = occupancy_bin_warp(fp32, h->tuning.warp_bin_warps, h->capW);
     if (occ < 1) return RSAI_ERR_CUDA;
     if (h->tuning.warp_bin_ctas_per_sm > 0) occ = std::min(occ, h->tuning.warp_bin_ctas_per_sm);
     h->grid_w = h->sms * occ;
     // bin W2: the warp bin's algorithm for |I| <= 128 (B 128 x 32), fewer warps per SM
-    h->capW2 = Caps{128, 32, 512, 64, 128 * 32, 64, h->tuning.small_qr_max_p, 0, 0, 128, spai};
+    h->capW2 = Caps{128, 32, 512, 64, 128 * 32, h->tuning.small_qr_max_p, 0, 0, 128, spai};
     if (plan_w2(h, fp32) != RSAI_OK) return RSAI_ERR_CUDA;
-    // bin S: 128 threads per column, |I| <= 128, |J| <= 64, four or five columns
-    // per SM (FP32; three in FP64) instead of bin C's one: the small end of bin
-    // C, on the same arithmetic bit for bit
-    h->capS = Caps{128, 64, 512, std::min(std::max(64, rneed), 512), 128 * 64, 0, 0, 0, 1, 256, spai};
+    // bins S0 (64 threads per column, |I| <= 96, |J| <= 40) and S (128 threads,
+    // |I| <= 128, |J| <= 64): nine and five columns per SM in FP32 instead of bin C's
+    // one, on the same arithmetic bit for bit.  W2 ends at |J| = 32: 33^3 at
+    // eps = 0.15 has 26941 columns of 33 or 34 (bin C alone 73 ms, S 18 ms).
+    const int rsmall = std::min(std::max(64, rneed), 512);
+    h->capS0 = Caps{96, 40, 256, rsmall, 96 * 40, 0, 0, 1, 128, spai};
+    occ = occupancy_bin_block(fp32, CTA_BIN_TINY, h->capS0);
+    if (occ < 1) return RSAI_ERR_CUDA;
+    h->grid_s0 = h->sms * occ;
+    h->capS = Caps{128, 64, 512, rsmall, 128 * 64, 0, 0, 1, 256, spai};
     occ = occupancy_bin_block(fp32, CTA_BIN_SMALL, h->capS);
     if (occ < 1) return RSAI_ERR_CUDA;
     h->grid_s = h->sms * occ;
     // bin C: shared-memory workspace as large as the opt-in limit allows
-    Caps c{1024, 256, 4096, std::min(rneed * 2, 2048), 0, 0, 0, 0, 1, 1024, spai};
+    Caps c{1024, 256, 4096, std::min(rneed * 2, 2048), 0, 0, 0, 1, 1024, spai};
     size_t base = fp32 ? work_bytes<float>(c) : work_bytes<double>(c);
     size_t avail = (size_t)max_optin - 2048;
     if (base >= avail) return RSAI_ERR_CUDA;
@@ -444,7 +489,7 @@ int plan_bins(rsai_handle *h) {
     const int64_t n = h->n;
     const int qg = (int)std::min<int64_t>(32768, n), pg = (int)std::min<int64_t>(4096, n);
     const int entries = next_pow2((int)std::min<int64_t>(131072, std::max<int64_t>({h->nnz, n, 2 * (int64_t)pg})));
-    h->capG = Caps{qg, pg, std::min(131072, entries), 8192, std::min<int64_t>((int64_t)1 << 24, (int64_t)qg * pg), 0, 0,
+    h->capG = Caps{qg, pg, std::min(131072, entries), 8192, std::min<int64_t>((int64_t)1 << 24, (int64_t)qg * pg), 0,
                    max_optin - 2048, 1, qg, spai};
     h->gstride = ((fp32 ? work_bytes<float>(h->capG) : work_bytes<double>(h->capG)) + 255) & ~size_t(255);
     h->grid_g = h->launch_g = 1;  // sized by the first build (size_global)
@@ -626,12 +671,13 @@ int build_common(rsai_handle *h, cudaStream_t st) {
     if (h->params.precision == RSAI_FP32_REFINE) TRY(dalloc(h, &h->cval32, nnz, st));
     // ---- buffers of the build sequence ----
     h->ovf_cap = n;
-    TRY(dalloc(h, &h->qnext, 12, st));
+    TRY(dalloc(h, &h->qnext, 15, st));
     TRY(dalloc(h, &h->ovf0, n, st));
     TRY(dalloc(h, &h->ovf1, n, st));
     TRY(dalloc(h, &h->ovf2, n, st));
     TRY(dalloc(h, &h->ovf3, n, st));
     TRY(dalloc(h, &h->ovf_s, n, st));
+    TRY(dalloc(h, &h->ovf_s0, n, st));
     TRY(dalloc(h, &h->ovf3_sorted, n, st));
     TRY(dalloc(h, &h->cost_bucket, n, st));
     TRY(dalloc(h, &h->cost_hist, kCostBuckets, st));
@@ -1204,15 +1250,15 @@ rsai_status rsai_set_tuning(rsai_handle *h, const rsai_tuning *t) {
     h->tuning = *t;
     const bool fp32 = h->params.precision == RSAI_FP32_REFINE;
     h->capW.small_p = t->small_qr_max_p;
-    h->capH.small_p = t->small_qr_max_p;
+    h->capH.small_p = h->capW0.small_p = t->small_qr_max_p;
     int occ = occupancy_bin_warp(fp32, w, h->capW);
     if (occ < 1 || occupancy_bin_half(fp32, w, h->capH) < 1) {
         h->tuning = old;
         h->capW.small_p = old.small_qr_max_p;
-        h->capH.small_p = old.small_qr_max_p;
+        h->capH.small_p = h->capW0.small_p = old.small_qr_max_p;
         return RSAI_ERR_INVALID_ARG;
     }
-    if (plan_h(h, fp32) != RSAI_OK) return RSAI_ERR_CUDA;
+    if (plan_h(h, fp32) != RSAI_OK || plan_w0(h, fp32) != RSAI_OK) return RSAI_ERR_CUDA;
     if (t->warp_bin_ctas_per_sm > 0) occ = std::min(occ, t->warp_bin_ctas_per_sm);
     h->grid_w = h->sms * occ;
     h->capW2.small_p = t->small_qr_max_p;

@@ -21,6 +21,105 @@ __device__ void back_substitute_team(const Team &team, const T *B, int q, int p,
     }
 }
 
+// x >= 0, x > 0 and |x| <= y (y >= 0) as the comparisons give them (NaN: false);
+// of doubles on their bit patterns, which keeps the FP64 unit free
+__device__ __forceinline__ bool not_negative(float x) { return x >= 0.0f; }
+__device__ __forceinline__ bool not_negative(double x) {
+    const long long b = __double_as_longlong(x);
+    return (b >= 0 && b <= 0x7ff0000000000000LL) || b == LLONG_MIN;  // LLONG_MIN: -0.0
+}
+__device__ __forceinline__ bool positive(float x) { return x > 0.0f; }
+__device__ __forceinline__ bool positive(double x) {
+    const long long b = __double_as_longlong(x);
+    return b > 0 && b <= 0x7ff0000000000000LL;
+}
+__device__ __forceinline__ bool abs_at_most(float x, float y) { return fabs(x) <= y; }
+__device__ __forceinline__ bool abs_at_most(double x, double y) {
+    return abskey(x) <= __double_as_longlong(y) && __double_as_longlong(y) <= 0x7ff0000000000000LL;
+}
+
+// A Householder update of the M columns c0..c0+M-1 of B (c == p: rhs; past p:
+// nothing), rows j..q-1, on W lanes of one warp: t <- t - f v, f = two_over (v . t).
+// The dot products are summed over the lanes together: a reduce-scatter leaves
+// column u's sum on the lanes u * W / M.., by the additions of M separate
+// butterflies but M - 1 + log2(W / M) of them per lane instead of M log2 W, and
+// with M chains in flight instead of one.  In FP64 (2 lanes per cycle and SM) the
+// additions were as much work as the products: 64^3 in FP64, three rows per lane,
+// 11 FP64 instructions per column and step against 7 to 8.
+template <int M, int W, typename T>
+__device__ __forceinline__ void update_columns(unsigned mask, int lane, T *B, int ld, int q, int p, T *rhs,
+                                               const T *col, T v0, T two_over, int j, int c0) {
+    T x[M];
+    T *t[M];
+#pragma unroll
+    for (int u = 0; u < M; ++u) {
+        x[u] = T(0);
+        t[u] = c0 + u < p ? B + (int64_t)(c0 + u) * ld : rhs;
+    }
+    for (int i = j + lane; i < q; i += W) {
+        const T v = (i == j) ? v0 : col[i];
+#pragma unroll
+        for (int u = 0; u < M; ++u)
+            if (c0 + u <= p) x[u] += v * t[u][i];
+    }
+#pragma unroll
+    for (int h = M / 2, o = W / 2; h >= 1; h >>= 1, o >>= 1) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int u = 0; u < h; ++u) {
+            const T send = up ? x[u] : x[u + h];
+            const T keep = up ? x[u + h] : x[u];
+            x[u] = keep + __shfl_xor_sync(mask, send, o);
+        }
+    }
+#pragma unroll
+    for (int o = W / 2 / M; o > 0; o >>= 1) x[0] += __shfl_xor_sync(mask, x[0], o);
+    const T f = x[0] * two_over;
+    T fu[M];
+#pragma unroll
+    for (int u = 0; u < M; ++u) fu[u] = __shfl_sync(mask, f, u * (W / M), W);
+    for (int i = j + lane; i < q; i += W) {
+        const T v = (i == j) ? v0 : col[i];
+#pragma unroll
+        for (int u = 0; u < M; ++u)
+            if (c0 + u <= p) t[u][i] -= fu[u] * v;
+    }
+}
+
+// lanes of the calling thread's group of W lanes
+template <int W> __device__ __forceinline__ unsigned group_mask() {
+    if constexpr (W == 32) return 0xffffffffu;
+    else return 0xffffu << (threadIdx.x & 16);
+}
+
+// The reflector of a column from its norm^2 and head x0: R_jj, v(j), 2 / v^T v
+template <typename T> __device__ __forceinline__ void reflector(T sigma, T x0, T &alpha, T &v0, T &two_over) {
+    const T nrm = sqrt(sigma);
+    alpha = not_negative(x0) ? -nrm : nrm;
+    v0 = x0 - alpha;
+    const T vtv = sigma - x0 * x0 + v0 * v0;
+    two_over = positive(vtv) ? T(2) / vtv : T(0);
+}
+
+// This thread's terms of the sum of squares of col[j..q) (BlockTeam::sum_rows)
+template <class Team, typename T>
+__device__ __forceinline__ void squares_of_rows(const T *col, int j, int q, int me, T (&part)[Team::VK]) {
+    if constexpr (Team::VK == 1) {
+        part[0] = T(0);
+        for (int i = j + me; i < q; i += Team::SIZE) part[0] += col[i] * col[i];
+    } else {
+#pragma unroll
+        for (int v = 0; v < Team::VK; ++v) {
+            const int i = j + me + v * Team::SIZE;
+            part[v] = i < q ? col[i] * col[i] : T(0);
+        }
+    }
+}
+
+// Columns that a warp's FP32 update takes at a time (33^3 at eps = 0.15: bins W and
+// W2 11.5 ms with one, 9.0 with four)
+constexpr int kLaneBatch32 = 4;
+
 // One Householder step j on B (q x p, ld q) and rhs: the reflector of column j
 // over rows >= j, applied to the columns c in [c_begin, p) and to rhs.  The
 // norm is one team reduction; the columns are dealt out to the team's warps,
@@ -34,23 +133,71 @@ __device__ __forceinline__ void householder_step(const Team &team, T *B, int q, 
     constexpr int NW = Team::SIZE / LN;
     const int lane = me % LN, wid = me / LN;
     T *col = B + (int64_t)j * q;
-    T part = 0;
-    for (int i = j + me; i < q; i += Team::SIZE) part += col[i] * col[i];
-    const T sigma = team.sum(part);
-    const T x0 = col[j];
-    const T nrm = sqrt(sigma);
-    const T alpha = (x0 >= T(0)) ? -nrm : nrm;
-    const T v0 = x0 - alpha;
-    const T vtv = sigma - x0 * x0 + v0 * v0;
-    const T two_over = (vtv > T(0)) ? T(2) / vtv : T(0);
-    if (two_over > T(0)) {
-        for (int c = c_begin + wid; c <= p; c += NW) {
-            T *t = (c < p) ? B + (int64_t)c * q : rhs;
-            T d = 0;
-            for (int i = j + lane; i < q; i += LN) d += ((i == j) ? v0 : col[i]) * t[i];
-            d = team.lanes_sum(d);
-            const T f = d * two_over;
-            for (int i = j + lane; i < q; i += LN) t[i] -= f * ((i == j) ? v0 : col[i]);
+    T alpha, v0, two_over;
+    if constexpr (!is_lane_team<Team>::value && sizeof(T) == 8) {
+        // the warps' sums, the square root and the division on one warp: as
+        // much FP64 work per warp as the update of several columns
+        constexpr int VK = Team::VK;
+        T part[VK];
+        squares_of_rows<Team>(col, j, q, me, part);
+#pragma unroll
+        for (int v = 0; v < VK; ++v) part[v] = team.lanes_sum(part[v]);
+        team.sync();
+        if (lane == 0) {
+#pragma unroll
+            for (int v = 0; v < VK; ++v) team.template slot<T>(wid + NW * v) = part[v];
+        }
+        team.sync();
+        if (wid == 0) {
+            T sigma = team.template slot<T>(0);
+#pragma unroll
+            for (int w = 1; w < NW * VK; ++w) sigma += team.template slot<T>(w);
+            reflector(sigma, col[j], alpha, v0, two_over);
+            __syncwarp();
+            if (lane == 0) {
+                team.template slot<T>(0) = alpha;
+                team.template slot<T>(1) = v0;
+                team.template slot<T>(2) = two_over;
+            }
+        }
+        team.sync();
+        alpha = team.template slot<T>(0);
+        v0 = team.template slot<T>(1);
+        two_over = team.template slot<T>(2);
+    } else if constexpr (!is_lane_team<Team>::value) {
+        T part[Team::VK];
+        squares_of_rows<Team>(col, j, q, me, part);
+        reflector(team.sum_rows(part), col[j], alpha, v0, two_over);
+    } else {
+        T part = 0;
+        for (int i = j + me; i < q; i += Team::SIZE) part += col[i] * col[i];
+        reflector(team.sum(part), col[j], alpha, v0, two_over);
+    }
+    if (positive(two_over)) {
+        const unsigned mask = group_mask<LN>();
+        if constexpr (is_lane_team<Team>::value && sizeof(T) == 4) {
+            for (int c = c_begin; c <= p; c += kLaneBatch32)
+                update_columns<kLaneBatch32, LN>(mask, lane, B, q, q, p, rhs, col, v0, two_over, j, c);
+        } else if constexpr (is_lane_team<Team>::value) {
+            int c = c_begin;
+            for (; c + 4 <= p; c += 8) update_columns<8, LN>(mask, lane, B, q, q, p, rhs, col, v0, two_over, j, c);
+            if (c + 1 < p) {
+                update_columns<4, LN>(mask, lane, B, q, q, p, rhs, col, v0, two_over, j, c);
+                c += 4;
+            }
+            for (; c <= p; c += 2) update_columns<2, LN>(mask, lane, B, q, q, p, rhs, col, v0, two_over, j, c);
+        } else {
+            // an even share per warp, four or two or one at a time
+            const int left = p - c_begin + 1;
+            if (left > 2 * NW) {
+                for (int c = c_begin + 4 * wid; c <= p; c += 4 * NW)
+                    update_columns<4, LN>(mask, lane, B, q, q, p, rhs, col, v0, two_over, j, c);
+            } else if (left > NW) {
+                for (int c = c_begin + 2 * wid; c <= p; c += 2 * NW)
+                    update_columns<2, LN>(mask, lane, B, q, q, p, rhs, col, v0, two_over, j, c);
+            } else if (c_begin + wid <= p) {
+                update_columns<1, LN>(mask, lane, B, q, q, p, rhs, col, v0, two_over, j, c_begin + wid);
+            }
         }
     }
     team.sync();
@@ -59,7 +206,7 @@ __device__ __forceinline__ void householder_step(const Team &team, T *B, int q, 
         vhead[j] = v0;
         taus[j] = two_over;
     }
-    rank_flag |= (fabs(alpha) <= small) ? 1 : 0;
+    rank_flag |= abs_at_most(alpha, small) ? 1 : 0;
     team.sync();
 }
 
@@ -144,10 +291,22 @@ __device__ __noinline__ void apply_qt_team(Team team, const T *B, int q, int p, 
         const T *col = B + (int64_t)j * q;
         const T v0 = vhead[j], tau = taus[j];
         if (tau > T(0)) {
-            T d = 0;
-            for (int i = me; i < q; i += Team::SIZE)
-                if (i >= j) d += ((i == j) ? v0 : col[i]) * rhs[i];
-            T sdot = team.sum(d);
+            T sdot;
+            if constexpr (is_lane_team<Team>::value) {
+                T d = 0;
+                for (int i = me; i < q; i += Team::SIZE)
+                    if (i >= j) d += ((i == j) ? v0 : col[i]) * rhs[i];
+                sdot = team.sum(d);
+            } else {
+                T d[Team::VK];
+#pragma unroll
+                for (int v = 0; v < Team::VK; ++v) {
+                    d[v] = T(0);
+                    for (int i = me + v * Team::SIZE; i < q; i += Team::VK == 1 ? Team::SIZE : q)
+                        if (i >= j) d[v] += ((i == j) ? v0 : col[i]) * rhs[i];
+                }
+                sdot = team.sum_rows(d);
+            }
             T f = sdot * tau;
             for (int i = me; i < q; i += Team::SIZE)
                 if (i >= j) rhs[i] -= f * ((i == j) ? v0 : col[i]);
@@ -158,25 +317,22 @@ __device__ __noinline__ void apply_qt_team(Team team, const T *B, int q, int p, 
     else back_substitute_blocked(team, B, q, p, rhs, small);
 }
 
-// Reflector j (built on q0 rows) applied to the columns p0..p-1 of B (ld q),
-// one warp per column; ends with a team synchronisation.
+// The reflectors j0..j1-1 (built on q0 rows) applied in order to the columns
+// p0..p-1 of B (ld q).  A warp takes its columns through all of them, so nothing
+// is synchronised until the end.
 template <class Team, typename T>
-__device__ __forceinline__ void update_one_reflector(const Team &team, T *B, int q, int p, int q0, int p0,
-                                                     const T *vhead, const T *taus, int j) {
-    const int me = team.rank();
-    const int lane = me & 31, wid = me >> 5;
-    constexpr int NW = (Team::SIZE + 31) / 32;
-    const T *col = B + (int64_t)j * q;
-    const T v0 = vhead[j], two_over = taus[j];
-    if (two_over > T(0)) {
-        for (int c = p0 + wid; c < p; c += NW) {
-            T *t = B + (int64_t)c * q;
-            T d = 0;
-            for (int i = j + lane; i < q0; i += 32) d += ((i == j) ? v0 : col[i]) * t[i];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
-            const T f = d * two_over;
-            for (int i = j + lane; i < q0; i += 32) t[i] -= f * ((i == j) ? v0 : col[i]);
+__device__ __forceinline__ void update_reflectors(const Team &team, T *B, int q, int p, int q0, int p0,
+                                                  const T *vhead, const T *taus, int j0, int j1) {
+    const int lane = team.rank() & 31, wid = team.rank() >> 5;
+    constexpr int NW = Team::SIZE / 32, M = 2;
+    for (int c = p0 + M * wid; c < p; c += M * NW) {
+        for (int j = j0; j < j1; ++j) {
+            const T two_over = taus[j];
+            // p - 1: the last column is not a right-hand side here
+            if (positive(two_over))
+                update_columns<M, 32>(0xffffffffu, lane, B, q, q0, p - 1, B + (int64_t)(p - 1) * q, B + (int64_t)j * q,
+                                      vhead[j], two_over, j, c);
+            __syncwarp();
         }
     }
     team.sync();

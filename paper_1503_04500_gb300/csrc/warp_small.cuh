@@ -124,7 +124,7 @@ __device__ __forceinline__ void step_update(int j, T (&b)[R][kSmallP], T (&rr)[R
 // skipped.  Not inlined: the unrolled body is large and the column algorithm
 // calls the solve from several places.
 template <int W, int R, typename T>
-__device__ __noinline__ int lanes_qr_small(T *B, int q, int p, T *rhs, T *vhead, T *tau, T small) {
+__device__ __forceinline__ int lanes_qr_small(T *B, int q, int p, T *rhs, T *vhead, T *tau, T small) {
     static_assert(kSmallP <= W, "row i < 16 of R lives in lane i");
     const unsigned mask = lanes_mask<W>();
     const int lane = threadIdx.x & (W - 1);
@@ -206,7 +206,7 @@ __device__ __noinline__ int lanes_qr_small(T *B, int q, int p, T *rhs, T *vhead,
 
 // rhs <- R^{-1} Q^T rhs with the reflectors left in B, vhead and tau by lanes_qr_small
 template <int W, int R, typename T>
-__device__ __noinline__ void lanes_apply_qt_small(const T *B, int q, int p, T *rhs, const T *vhead, const T *tau,
+__device__ __forceinline__ void lanes_apply_qt_small(const T *B, int q, int p, T *rhs, const T *vhead, const T *tau,
                                                   T small) {
     const unsigned mask = lanes_mask<W>();
     const int lane = threadIdx.x & (W - 1);
