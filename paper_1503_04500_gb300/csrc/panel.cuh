@@ -10,6 +10,8 @@
 // how many instructions carry them.
 #pragma once
 
+#include <type_traits>
+
 #include "help.cuh"
 #include "team_qr.cuh"
 
@@ -48,10 +50,10 @@ __device__ __forceinline__ Chunk<T> panel_chunk(const T *V, int qq, int nb, int 
     for (int k = 0; k < CW; ++k) x.v[k] = (c * CW + k < nb) ? V[(c * CW + k) * qq + r] : T(0);
     return x;
 }
-template <typename T>
+template <bool FULL, typename T>
 __device__ __forceinline__ void panel_store_chunk(T *V, int qq, int nb, int r, int c, const Chunk<T> &x) {
     constexpr int CW = kChunk<T>;
-    if ((c + 1) * CW <= nb) {
+    if (FULL || (c + 1) * CW <= nb) {
         *reinterpret_cast<Chunk<T> *>(V + c * CW * qq + r * CW) = x;
     } else {
 #pragma unroll
@@ -89,7 +91,7 @@ __device__ __forceinline__ void panel_stage(const Team &team, const T *src, int6
                 }
             }
 #pragma unroll
-            for (int c = 0; c < kPanel / CW; ++c) panel_store_chunk(V, qq, nb, r, c, x[b][c]);
+            for (int c = 0; c < kPanel / CW; ++c) panel_store_chunk<false>(V, qq, nb, r, c, x[b][c]);
         }
     }
 }
@@ -109,6 +111,59 @@ __device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
     f32x2 d;
     asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
     return d;
+}
+
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+    f32x2 d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+    f32x2 d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+
+// a -= f p and acc += a x + b y, acc += a x, element by element of a chunk (each
+// element rounded as the scalar expressions contract: one product, then fused)
+__device__ __forceinline__ void chunk_sub(Chunk<float> &a, const Chunk<float> &f, float p) {
+    const f32x2 np = pack2(-p, -p);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const f32x2 r = fma2(pack2(f.v[2 * h], f.v[2 * h + 1]), np, pack2(a.v[2 * h], a.v[2 * h + 1]));
+        unpack2(r, a.v[2 * h], a.v[2 * h + 1]);
+    }
+}
+__device__ __forceinline__ void chunk_sub(Chunk<double> &a, const Chunk<double> &f, double p) {
+#pragma unroll
+    for (int k = 0; k < 2; ++k) a.v[k] -= f.v[k] * p;
+}
+__device__ __forceinline__ void chunk_dot(float *acc, const Chunk<float> &a, float x, const Chunk<float> &b, float y) {
+    const f32x2 xx = pack2(x, x), yy = pack2(y, y);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        f32x2 t = mul2(pack2(b.v[2 * h], b.v[2 * h + 1]), yy);
+        t = fma2(pack2(a.v[2 * h], a.v[2 * h + 1]), xx, t);
+        t = add2(pack2(acc[2 * h], acc[2 * h + 1]), t);
+        unpack2(t, acc[2 * h], acc[2 * h + 1]);
+    }
+}
+__device__ __forceinline__ void chunk_dot(float *acc, const Chunk<float> &a, float x) {
+    const f32x2 xx = pack2(x, x);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const f32x2 t = fma2(pack2(a.v[2 * h], a.v[2 * h + 1]), xx, pack2(acc[2 * h], acc[2 * h + 1]));
+        unpack2(t, acc[2 * h], acc[2 * h + 1]);
+    }
+}
+__device__ __forceinline__ void chunk_dot(double *acc, const Chunk<double> &a, double x, const Chunk<double> &b,
+                                          double y) {
+#pragma unroll
+    for (int k = 0; k < 2; ++k) acc[k] += a.v[k] * x + b.v[k] * y;
+}
+__device__ __forceinline__ void chunk_dot(double *acc, const Chunk<double> &a, double x) {
+#pragma unroll
+    for (int k = 0; k < 2; ++k) acc[k] += a.v[k] * x;
 }
 
 // Sum of kPanel values over the 32 lanes of a warp by halving exchanges (a
@@ -157,7 +212,7 @@ __device__ __forceinline__ T team_sum16_warp0(const Team &team, T (&v)[kPanel], 
 // warp 0 then forms the reflector, the factors f of the next pass and row t.
 // Chunks are visited from the one that holds column t (rotated by tc) so that
 // every register index is a constant.
-template <int TK, class Team, typename T>
+template <int TK, bool FULL, class Team, typename T>
 __device__ __forceinline__ void panel_step(const Team &team, T *V, int qq, int nb, int tc, T *vhead, T *taus, T *tm,
                                            T *red, T *flag, T *f, T small, int &rank_flag) {
     constexpr int CW = kChunk<T>, NC = kPanel / CW;
@@ -173,39 +228,37 @@ __device__ __forceinline__ void panel_step(const Team &team, T *V, int qq, int n
         const bool two = rb < qq;
         T pa = T(0), pb = T(0);  // column t - 1
         if (upd) {
-            pa = panel_at(V, qq, nb, ra, t - 1);
-            if (two) pb = panel_at(V, qq, nb, rb, t - 1);
+            pa = panel_at(V, qq, FULL ? kPanel : nb, ra, t - 1);
+            if (two) pb = panel_at(V, qq, FULL ? kPanel : nb, rb, t - 1);
         }
         T xa = T(0), xb = T(0);  // column t
 #pragma unroll
         for (int j = 0; j < NC; ++j) {
             const int c = (tc + j) & (NC - 1);
-            if (c * CW >= nb) continue;
-            Chunk<T> a = panel_chunk<false>(V, qq, nb, ra, c), b = a;
-            if (two) b = panel_chunk<false>(V, qq, nb, rb, c);
+            if (!FULL && c * CW >= nb) continue;
+            Chunk<T> a = panel_chunk<FULL>(V, qq, nb, ra, c), b = a;
+            if (two) b = panel_chunk<FULL>(V, qq, nb, rb, c);
             if (upd && (j == 0 || c > tc)) {
-                const Chunk<T> fc = *reinterpret_cast<const Chunk<T> *>(f + c * CW);
+                Chunk<T> fc = *reinterpret_cast<const Chunk<T> *>(f + c * CW);
+                const Chunk<T> a0 = a, b0 = b;
+                chunk_sub(a, fc, pa);
+                chunk_sub(b, fc, pb);
+                if (j == 0) {  // the columns before t are finished
 #pragma unroll
-                for (int k = 0; k < CW; ++k) {
-                    if (j > 0 || k >= TK) {
-                        a.v[k] -= fc.v[k] * pa;
-                        b.v[k] -= fc.v[k] * pb;
+                    for (int k = 0; k < TK; ++k) {
+                        a.v[k] = a0.v[k];
+                        b.v[k] = b0.v[k];
                     }
                 }
-                panel_store_chunk(V, qq, nb, ra, c, a);
-                if (two) panel_store_chunk(V, qq, nb, rb, c, b);
+                panel_store_chunk<FULL>(V, qq, nb, ra, c, a);
+                if (two) panel_store_chunk<FULL>(V, qq, nb, rb, c, b);
             }
             if (j == 0) {
                 xa = a.v[TK];
                 xb = b.v[TK];
             }
-            if (two) {
-#pragma unroll
-                for (int k = 0; k < CW; ++k) acc[j * CW + k] += a.v[k] * xa + b.v[k] * xb;
-            } else {
-#pragma unroll
-                for (int k = 0; k < CW; ++k) acc[j * CW + k] += a.v[k] * xa;
-            }
+            if (two) chunk_dot(acc + j * CW, a, xa, b, xb);
+            else chunk_dot(acc + j * CW, a, xa);
         }
     }
     const T s = team_sum16_warp0(team, acc, red);
@@ -258,14 +311,22 @@ __device__ __forceinline__ void panel_factor(const Team &team, T *V, int qq, int
     constexpr int CW = kChunk<T>;
     const int me = team.rank();
     if (me < kPanel) f[me] = T(0);
-    for (int tc = 0; tc * CW < nb; ++tc) {
-        panel_step<0>(team, V, qq, nb, tc, vhead, taus, tm, red, flag, f, small, rank_flag);
-        if (tc * CW + 1 < nb) panel_step<1>(team, V, qq, nb, tc, vhead, taus, tm, red, flag, f, small, rank_flag);
-        if constexpr (CW == 4) {
-            if (tc * CW + 2 < nb) panel_step<2>(team, V, qq, nb, tc, vhead, taus, tm, red, flag, f, small, rank_flag);
-            if (tc * CW + 3 < nb) panel_step<3>(team, V, qq, nb, tc, vhead, taus, tm, red, flag, f, small, rank_flag);
+    auto steps = [&](auto full) {
+        constexpr bool FULL = decltype(full)::value;
+        for (int tc = 0; tc * CW < nb; ++tc) {
+            panel_step<0, FULL>(team, V, qq, nb, tc, vhead, taus, tm, red, flag, f, small, rank_flag);
+            if (FULL || tc * CW + 1 < nb)
+                panel_step<1, FULL>(team, V, qq, nb, tc, vhead, taus, tm, red, flag, f, small, rank_flag);
+            if constexpr (CW == 4) {
+                if (FULL || tc * CW + 2 < nb)
+                    panel_step<2, FULL>(team, V, qq, nb, tc, vhead, taus, tm, red, flag, f, small, rank_flag);
+                if (FULL || tc * CW + 3 < nb)
+                    panel_step<3, FULL>(team, V, qq, nb, tc, vhead, taus, tm, red, flag, f, small, rank_flag);
+            }
         }
-    }
+    };
+    if (nb == kPanel) steps(std::true_type{});
+    else steps(std::false_type{});
     // T from Y and tau: lane s of warp 0 holds row s of T
     if (me < 32) {
         const int sr = me;
@@ -304,7 +365,7 @@ __device__ __forceinline__ void panel_factor(const Team &team, T *V, int qq, int
                 else if (u == r) x[u / CW].v[u % CW] = vhead[u];
             }
 #pragma unroll
-            for (int c = 0; c < kPanel / CW; ++c) panel_store_chunk(V, qq, nb, r, c, x[c]);
+            for (int c = 0; c < kPanel / CW; ++c) panel_store_chunk<false>(V, qq, nb, r, c, x[c]);
         }
     }
     team.sync();
@@ -331,41 +392,65 @@ template <int KC, int D, bool FULL, typename T>
 __device__ __forceinline__ void wy_apply_cols(const T *V, int qq, int nb, const T *tm, T *const (&tc)[KC],
                                               const bool (&has)[KC], int lane) {
     constexpr int CW = kChunk<T>, NC = kPanel / CW;
-    constexpr bool F32 = sizeof(T) == 4;
-    T nw[KC][kPanel];  // W, then -T^T W
+    constexpr bool F32 = sizeof(T) == 4, P2 = F32 && KC >= 2;
+    const int full = qq >> 5;  // passes in which every lane has a row
     T cb[D][KC];
-    // W = V^T C
-    {
-        f32x2 w2[F32 ? KC : 1][F32 ? kPanel / 2 : 1];
-        if constexpr (F32) {
+    auto load = [&](T (&c)[KC], int r) {
 #pragma unroll
-            for (int x = 0; x < KC; ++x)
+        for (int x = 0; x < KC; ++x) c[x] = tc[x][r];
+    };
+    // f(r, row r of C) over all rows, the loads D passes ahead (the first ones in cb)
+    auto stream = [&](auto ahead, auto f) {
+        int r = lane, k = 0;
+        for (; k + 2 * D <= full; k += D) {
 #pragma unroll
-                for (int u = 0; u < kPanel / 2; ++u) w2[x][u] = 0ull;
-        } else {
-#pragma unroll
-            for (int x = 0; x < KC; ++x)
-#pragma unroll
-                for (int u = 0; u < kPanel; ++u) nw[x][u] = T(0);
-        }
-#pragma unroll
-        for (int y = 0; y < D; ++y)
-#pragma unroll
-            for (int x = 0; x < KC; ++x) cb[y][x] = (lane + 32 * y < qq) ? tc[x][lane + 32 * y] : T(0);
-        for (int r0 = lane; r0 < qq; r0 += 32 * D) {
-#pragma unroll
-            for (int y = 0; y < D; ++y) {
-                const int r = r0 + 32 * y, rn = r + 32 * D;
-                if (r >= qq) break;
+            for (int y = 0; y < D; ++y, r += 32) {
                 T cur[KC];
 #pragma unroll
                 for (int x = 0; x < KC; ++x) cur[x] = cb[y][x];
-                if (rn < qq) {
+                load(cb[y], r + 32 * D);
+                ahead(r + 32 * D);
+                f(r, cur);
+            }
+        }
+        if (k + D <= full) {
 #pragma unroll
-                    for (int x = 0; x < KC; ++x) cb[y][x] = tc[x][rn];
+            for (int y = 0; y < D; ++y, r += 32) f(r, cb[y]);
+            k += D;
+        }
+        for (; r < qq; r += 32) {
+            T cur[KC];
+            load(cur, r);
+            f(r, cur);
+        }
+    };
+    auto first = [&] {
+        if (full >= D) {
 #pragma unroll
-                    for (int x = 0; x < KC; ++x) prefetch_l2(tc[x] + min(rn + 32 * kAhead, qq - 1));
+            for (int y = 0; y < D; ++y) load(cb[y], lane + 32 * y);
+        }
+    };
+    T nw[KC][kPanel];  // W, then -T^T W
+    // W = V^T C
+    first();
+    {
+        f32x2 w2[F32 ? KC : 1][F32 ? kPanel / 2 : 1];
+#pragma unroll
+        for (int x = 0; x < KC; ++x) {
+#pragma unroll
+            for (int u = 0; u < kPanel; ++u) {
+                if constexpr (F32) w2[x][u / 2] = 0ull;
+                else nw[x][u] = T(0);
+            }
+        }
+        stream(
+            [&](int r) {
+                if (r + 32 * kAhead < qq) {
+#pragma unroll
+                    for (int x = 0; x < KC; ++x) prefetch_l2(tc[x] + r + 32 * kAhead);
                 }
+            },
+            [&](int r, const T (&cur)[KC]) {
                 if constexpr (F32) {
                     f32x2 cc[KC];
 #pragma unroll
@@ -390,8 +475,7 @@ __device__ __forceinline__ void wy_apply_cols(const T *V, int qq, int nb, const 
                             for (int x = 0; x < KC; ++x) nw[x][c * CW + k] += v.v[k] * cur[x];
                     }
                 }
-            }
-        }
+            });
         if constexpr (F32) {
 #pragma unroll
             for (int x = 0; x < KC; ++x)
@@ -399,11 +483,7 @@ __device__ __forceinline__ void wy_apply_cols(const T *V, int qq, int nb, const 
                 for (int u = 0; u < kPanel / 2; ++u) unpack2(w2[x][u], nw[x][2 * u], nw[x][2 * u + 1]);
         }
     }
-    // the first entries of the second pass, in flight during the reduction
-#pragma unroll
-    for (int y = 0; y < D; ++y)
-#pragma unroll
-        for (int x = 0; x < KC; ++x) cb[y][x] = (lane + 32 * y < qq) ? tc[x][lane + 32 * y] : T(0);
+    first();  // of the second pass, in flight during the reduction
     // totals: lane l keeps entry u = l >> 1, of column 2g + (l & 1) in sel[g];
     // then -T^T W, one entry per lane and group, and the broadcast to every lane
     {
@@ -435,59 +515,48 @@ __device__ __forceinline__ void wy_apply_cols(const T *V, int qq, int nb, const 
             for (int v = 0; v < kPanel; ++v) nw[x][v] = __shfl_sync(0xffffffffu, acc[x / 2], 2 * v + (x & 1));
     }
     // C <- C + V (-T^T W)
-    {
-        constexpr bool P2 = F32 && KC >= 2;
-        f32x2 n2[P2 ? KC / 2 : 1][P2 ? kPanel : 1];
-        if constexpr (P2) {
+    f32x2 n2[P2 ? KC / 2 : 1][P2 ? kPanel : 1];
+    if constexpr (P2) {
 #pragma unroll
-            for (int g = 0; g < KC / 2; ++g)
+        for (int g = 0; g < KC / 2; ++g)
 #pragma unroll
-                for (int u = 0; u < kPanel; ++u) n2[g][u] = pack2(nw[2 * g][u], nw[2 * g + 1][u]);
-        }
-        for (int r0 = lane; r0 < qq; r0 += 32 * D) {
-#pragma unroll
-            for (int y = 0; y < D; ++y) {
-                const int r = r0 + 32 * y, rn = r + 32 * D;
-                if (r >= qq) break;
-                T cur[KC];
-#pragma unroll
-                for (int x = 0; x < KC; ++x) cur[x] = cb[y][x];
-                if (rn < qq) {
-#pragma unroll
-                    for (int x = 0; x < KC; ++x) cb[y][x] = tc[x][rn];
-                }
-                if constexpr (P2) {
-                    f32x2 a2[KC / 2];
-#pragma unroll
-                    for (int g = 0; g < KC / 2; ++g) a2[g] = pack2(cur[2 * g], cur[2 * g + 1]);
-#pragma unroll
-                    for (int c = 0; c < NC; ++c) {
-                        const Chunk<T> v = panel_chunk<FULL>(V, qq, nb, r, c);
-#pragma unroll
-                        for (int k = 0; k < CW; ++k) {
-                            const f32x2 vv = pack2(v.v[k], v.v[k]);
-#pragma unroll
-                            for (int g = 0; g < KC / 2; ++g) a2[g] = fma2(vv, n2[g][c * CW + k], a2[g]);
-                        }
-                    }
-#pragma unroll
-                    for (int g = 0; g < KC / 2; ++g) unpack2(a2[g], cur[2 * g], cur[2 * g + 1]);
-                } else {
-#pragma unroll
-                    for (int c = 0; c < NC; ++c) {
-                        const Chunk<T> v = panel_chunk<FULL>(V, qq, nb, r, c);
-#pragma unroll
-                        for (int k = 0; k < CW; ++k)
-#pragma unroll
-                            for (int x = 0; x < KC; ++x) cur[x] += v.v[k] * nw[x][c * CW + k];
-                    }
-                }
-#pragma unroll
-                for (int x = 0; x < KC; ++x)
-                    if (has[x]) tc[x][r] = cur[x];
-            }
-        }
+            for (int u = 0; u < kPanel; ++u) n2[g][u] = pack2(nw[2 * g][u], nw[2 * g + 1][u]);
     }
+    stream([](int) {},
+           [&](int r, const T (&c0)[KC]) {
+               T cur[KC];
+#pragma unroll
+               for (int x = 0; x < KC; ++x) cur[x] = c0[x];
+               if constexpr (P2) {
+                   f32x2 a2[KC / 2];
+#pragma unroll
+                   for (int g = 0; g < KC / 2; ++g) a2[g] = pack2(cur[2 * g], cur[2 * g + 1]);
+#pragma unroll
+                   for (int c = 0; c < NC; ++c) {
+                       const Chunk<T> v = panel_chunk<FULL>(V, qq, nb, r, c);
+#pragma unroll
+                       for (int k = 0; k < CW; ++k) {
+                           const f32x2 vv = pack2(v.v[k], v.v[k]);
+#pragma unroll
+                           for (int g = 0; g < KC / 2; ++g) a2[g] = fma2(vv, n2[g][c * CW + k], a2[g]);
+                       }
+                   }
+#pragma unroll
+                   for (int g = 0; g < KC / 2; ++g) unpack2(a2[g], cur[2 * g], cur[2 * g + 1]);
+               } else {
+#pragma unroll
+                   for (int c = 0; c < NC; ++c) {
+                       const Chunk<T> v = panel_chunk<FULL>(V, qq, nb, r, c);
+#pragma unroll
+                       for (int k = 0; k < CW; ++k)
+#pragma unroll
+                           for (int x = 0; x < KC; ++x) cur[x] += v.v[k] * nw[x][c * CW + k];
+                   }
+               }
+#pragma unroll
+               for (int x = 0; x < KC; ++x)
+                   if (has[x]) tc[x][r] = cur[x];
+           });
 }
 
 // Columns c in [c_lo, c_hi] of B (ld q; c == p stands for rhs), rows
@@ -735,7 +804,7 @@ __device__ __noinline__ void apply_qt_panels(Team team, const T *B, int q, int p
                 }
                 if (staged) {
 #pragma unroll
-                    for (int c = 0; c < NC; ++c) panel_store_chunk(V, qq, nb, r, c, v[c]);
+                    for (int c = 0; c < NC; ++c) panel_store_chunk<false>(V, qq, nb, r, c, v[c]);
                 }
 #pragma unroll
                 for (int u = 0; u < kPanel; ++u)
