@@ -17,6 +17,7 @@ template <typename T, int NT, bool STAGED, int MINB, int MODE, class CapT>
 __global__ void __launch_bounds__(NT, MINB)
     k_bin_block(DevA A, DevParams P, CapT cap, ColQueue Q, ColOut O, Frozen F, unsigned long long *gctr,
                 int last_bin, char *gwork, size_t gstride, int bin, void *help, int owners) {
+    if (queue_empty(Q)) return;
     extern __shared__ __align__(16) char smem[];
     __shared__ unsigned long long red[kVirtualWarps + 1];
     __shared__ int redi[kVirtualWarps + 1];

@@ -50,6 +50,9 @@ __global__ void k_tau_fixed(const double *norm1, double tol, double *tau, int32_
 __global__ void k_scan_blocks(const int32_t *in, int64_t n, int64_t *out, int64_t *block_sums);
 __global__ void k_scan_sums(int64_t *block_sums, int64_t nb, int64_t *total);
 __global__ void k_scan_add(int64_t *out, int64_t n, const int64_t *block_sums, const int64_t *total);
+// most blocks of 1024 counts that k_scan_add_fold takes
+constexpr int64_t kScanFold = 4096;
+__global__ void k_scan_add_fold(int64_t *out, int64_t n, const int64_t *block_sums);
 __global__ void k_pool_to_csc(const int64_t *col_off, const int32_t *col_len, const int32_t *pool_rows,
                               const double *pool_vals, const int64_t *Mcolptr, int32_t *Mrows, double *Mvals,
                               int32_t *row_count, int64_t n);

@@ -53,6 +53,11 @@ struct rsai_handle {
     double *val = nullptr, *cval = nullptr;
     float *cval32 = nullptr;  // FP32 copy of cval (FP32_REFINE builds), refreshed by every build
     // 8-byte words: (unused), (unused), frob2, counters, column counts, partial sums
+    // One buffer that every build zeroes: the error word, the result pool's top,
+    // ||A||_1 per block, the scalar block and the rows' counters (`zeroed_bytes`); the words before
+    // the scalar block's statistics are read back together (rsai_get_stats).
+    unsigned long long *zeroed = nullptr;
+    size_t zeroed_bytes = 0;
     unsigned long long *dscal = nullptr;
     // blocks (a batch of independent matrices as one block-diagonal matrix)
     int32_t nblocks = 1;
@@ -65,10 +70,10 @@ struct rsai_handle {
     long long *bnc = nullptr, *bnnz = nullptr;
     int32_t *err = nullptr;
     // [0..3] queue counters of bins W, W2, C, G; [4..6] overflow counts W->W2,
-    // S->C, C->G; [7] columns of a pool-overflow rerun; [8] queue counter of
+    // S->C, C->G; [7] unused; [8] queue counter of
     // bin H, [9] overflow count H->W; [10] queue counter of bin S, [11]
     // columns forwarded to it (W and W2); [12] queue counter of bin W0; [13] queue counter of bin
-    // S0, [14] columns forwarded to it
+    // S0, [14] columns forwarded to it; then cost_hist; [kRerun] columns of a pool-overflow rerun
     uint32_t *qnext = nullptr;
     int32_t *ovf0 = nullptr, *ovf1 = nullptr, *ovf2 = nullptr, *ovf3 = nullptr, *ovf_s = nullptr, *ovf_s0 = nullptr;
     int32_t *ovf3_sorted = nullptr;  // the global bin's queue, largest column first
@@ -117,6 +122,11 @@ struct rsai_handle {
 };
 
 namespace {
+
+// qnext: the bins' counters, the cost histogram (zeroed with them) and the count of a rerun
+constexpr int kQueueWords = 16, kRerun = kQueueWords + kCostBuckets;
+// the zeroed buffer (8-byte words): error, pool top, ||A||_1 per block, then the scalar block
+constexpr int kErrWord = 0, kTopWord = 1, kNormWord = 2;
 
 // layout of the scalar block (8-byte words); words 0 and 1 are unused since
 // ||A||_1 and the drop threshold moved to per-block arrays
@@ -190,6 +200,23 @@ template <typename P> int dalloc(rsai_handle *h, P **ptr, size_t count, cudaStre
     return RSAI_OK;
 }
 
+// Several buffers of a handle's lifetime from one allocation, 256 bytes apart
+struct Carve {
+    std::vector<std::pair<void **, size_t>> parts;
+    size_t total = 0;
+    template <typename P> void add(P **ptr, size_t count) {
+        parts.push_back({(void **)ptr, total});
+        total += (sizeof(P) * (count ? count : 1) + 255) & ~size_t(255);
+    }
+    int commit(rsai_handle *h, cudaStream_t st) {
+        char *base = nullptr;
+        const int rc = dalloc(h, &base, total, st);
+        if (rc != RSAI_OK) return rc;
+        for (auto &p : parts) *p.first = base + p.second;
+        return RSAI_OK;
+    }
+};
+
 // frees one buffer taken by dalloc (stream-ordered on st)
 void dfree(rsai_handle *h, void *p, cudaStream_t st) {
     for (size_t i = 0; i < h->allocs.size(); ++i) {
@@ -233,8 +260,14 @@ cudaError_t scan_counts(rsai_handle *h, const int32_t *in, int64_t *out, cudaStr
     int64_t nb = (h->n + 1023) / 1024;
     if (nb < 1) nb = 1;
     k_scan_blocks<<<(unsigned)nb, 1024, 0, st>>>(in, h->n, out, h->scan_tmp);
-    k_scan_sums<<<1, 1024, 0, st>>>(h->scan_tmp, nb, h->scan_tmp + h->scan_tmp_len - 1);
-    k_scan_add<<<(unsigned)nb, 1024, 0, st>>>(out, h->n, h->scan_tmp, h->scan_tmp + h->scan_tmp_len - 1);
+    // up to kScanFold blocks (4M columns): each block adds up the sums before it, one
+    // launch less (about 2 us) for at most four loads per thread
+    if (nb > kScanFold) {
+        k_scan_sums<<<1, 1024, 0, st>>>(h->scan_tmp, nb, h->scan_tmp + h->scan_tmp_len - 1);
+        k_scan_add<<<(unsigned)nb, 1024, 0, st>>>(out, h->n, h->scan_tmp, h->scan_tmp + h->scan_tmp_len - 1);
+    } else {
+        k_scan_add_fold<<<(unsigned)nb, 1024, 0, st>>>(out, h->n, h->scan_tmp);
+    }
     return cudaGetLastError();
 }
 
@@ -248,8 +281,7 @@ cudaError_t enqueue_bins(rsai_handle *h, int mode, const DevA &A, const Frozen &
                          cudaStream_t st, cudaEvent_t *ev = nullptr, BinHook before_global = nullptr,
                          const int32_t *wlist = nullptr, const uint32_t *wcount = nullptr) {
     const int64_t n = h->n;
-    cudaMemsetAsync(h->qnext, 0, sizeof(uint32_t) * 7, st);  // queue and overflow counters; [7] = retry count
-    cudaMemsetAsync(h->qnext + 8, 0, sizeof(uint32_t) * 7, st);
+    cudaMemsetAsync(h->qnext, 0, sizeof(uint32_t) * kRerun, st);
     const DevParams P = dev_params(h);
     const bool fp32 = h->params.precision == RSAI_FP32_REFINE;
     ColOut O{h->col_off, h->col_len, h->col_q, h->rho, h->loops, h->flags, h->pool_rows, h->pool_vals,
@@ -313,7 +345,6 @@ cudaError_t enqueue_bins(rsai_handle *h, int mode, const DevA &A, const Frozen &
     }
     // the columns that reached the global bin, largest first (grids cover n;
     // the device-side count bounds the work)
-    cudaMemsetAsync(h->cost_hist, 0, sizeof(uint32_t) * kCostBuckets, st);
     k_cost_buckets<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(h->ovf3, h->qnext + 6, A.col_ptr, A.row_idx,
                                                                  A.row_ptr, h->cost_bucket, h->cost_hist);
     k_cost_offsets<<<1, 32, 0, st>>>(h->cost_hist);
@@ -333,13 +364,7 @@ cudaError_t enqueue_build_tail(rsai_handle *h, cudaStream_t st, cudaEvent_t *ev)
 cudaError_t enqueue_build(rsai_handle *h, cudaStream_t st, cudaEvent_t *ev = nullptr, BinHook hook = nullptr) {
     const int64_t n = h->n;
     if (ev) cudaEventRecord(ev[0], st);
-    cudaMemsetAsync(h->dscal, 0, sizeof(unsigned long long) * kScalars, st);
-    cudaMemsetAsync(h->err, 0, sizeof(int32_t), st);
-    cudaMemsetAsync(h->qnext, 0, sizeof(uint32_t) * 15, st);
-    cudaMemsetAsync(h->pool_top, 0, sizeof(unsigned long long), st);
-    cudaMemsetAsync(h->row_count, 0, sizeof(int32_t) * (size_t)n, st);
-    cudaMemsetAsync(h->cursor, 0, sizeof(int32_t) * (size_t)n, st);
-    cudaMemsetAsync(h->norm1_arr, 0, sizeof(double) * (size_t)h->nblocks, st);
+    cudaMemsetAsync(h->zeroed, 0, h->zeroed_bytes, st);
     k_norm1<<<blocks(n, 256), 256, 0, st>>>(h->col_ptr, h->cval, n, h->col_block, h->norm1_arr);
     if (h->cval32) k_to_f32<<<blocks(h->nnz, 256), 256, 0, st>>>(h->cval, h->cval32, h->nnz);
     k_tau_fixed<<<blocks(h->nblocks, 256), 256, 0, st>>>(h->norm1_arr, h->params.tol, h->tau_arr, h->nblocks);
@@ -354,7 +379,6 @@ cudaError_t enqueue_build(rsai_handle *h, cudaStream_t st, cudaEvent_t *ev = nul
 cudaError_t enqueue_build_tail(rsai_handle *h, cudaStream_t st, cudaEvent_t *ev) {
     const int64_t n = h->n;
     cudaError_t e;
-    cudaMemsetAsync(h->dscal + kCounts, 0, sizeof(unsigned long long) * 2, st);  // n_c, nnz(M): accumulated
     k_column_stats<<<kStatBlocks, 256, 0, st>>>(h->rho, h->flags, h->col_len, n, h->params.eps,
                                                 dword(h, kPartial), h->dscal + kCounts);
     k_column_stats_final<<<1, kStatBlocks, 0, st>>>(dword(h, kPartial), dword(h, kFrob2));
@@ -641,10 +665,43 @@ int build_common(rsai_handle *h, cudaStream_t st) {
         rc = (x);                     \
         if (rc != RSAI_OK) return rc; \
     } while (0)
-    TRY(dalloc(h, &h->dscal, kScalars, st));
-    TRY(dalloc(h, &h->err, 1, st));
-    TRY(dalloc(h, &h->norm1_arr, h->nblocks, st));
-    TRY(dalloc(h, &h->tau_arr, h->nblocks, st));
+    // The build's buffers whose sizes follow from n and the blocks, from one
+    // allocation: 22 of them took a tenth of the smallest builds.
+    {
+        const size_t words = kNormWord + (size_t)h->nblocks + kScalars;
+        h->zeroed_bytes = sizeof(unsigned long long) * words + 2 * sizeof(int32_t) * (size_t)n;
+        h->scan_tmp_len = (n + 1023) / 1024 + 2;
+        Carve c;
+        c.add(&h->zeroed, (h->zeroed_bytes + 7) / 8);
+        c.add(&h->tau_arr, h->nblocks);
+        c.add(&h->qnext, kRerun + 1);
+        c.add(&h->ovf0, n);
+        c.add(&h->ovf1, n);
+        c.add(&h->ovf2, n);
+        c.add(&h->ovf3, n);
+        c.add(&h->ovf_s, n);
+        c.add(&h->ovf_s0, n);
+        c.add(&h->ovf3_sorted, n);
+        c.add(&h->cost_bucket, n);
+        c.add(&h->col_off, n);
+        c.add(&h->col_len, n);
+        c.add(&h->col_q, n);
+        c.add(&h->loops, n);
+        c.add(&h->flags, n);
+        c.add(&h->rho, n);
+        c.add(&h->Mcolptr, n + 1);
+        c.add(&h->Mrowptr, n + 1);
+        c.add(&h->scan_tmp, h->scan_tmp_len);
+        c.add(&h->help, HelpBoard::bytes(h->sms));
+        TRY(c.commit(h, st));
+        h->err = reinterpret_cast<int32_t *>(h->zeroed + kErrWord);
+        h->pool_top = h->zeroed + kTopWord;
+        h->norm1_arr = reinterpret_cast<double *>(h->zeroed + kNormWord);
+        h->dscal = h->zeroed + kNormWord + h->nblocks;
+        h->row_count = reinterpret_cast<int32_t *>(h->dscal + kScalars);
+        h->cursor = h->row_count + n;
+        h->cost_hist = h->qnext + kQueueWords;
+    }
     // ---- validation of A (device kernels, error codes) ----
     // One pass on the stream, one read of the first error: each check after
     // the pointer checks returns at once if an earlier one set the error word,
@@ -671,31 +728,7 @@ int build_common(rsai_handle *h, cudaStream_t st) {
     if (h->params.precision == RSAI_FP32_REFINE) TRY(dalloc(h, &h->cval32, nnz, st));
     // ---- buffers of the build sequence ----
     h->ovf_cap = n;
-    TRY(dalloc(h, &h->qnext, 15, st));
-    TRY(dalloc(h, &h->ovf0, n, st));
-    TRY(dalloc(h, &h->ovf1, n, st));
-    TRY(dalloc(h, &h->ovf2, n, st));
-    TRY(dalloc(h, &h->ovf3, n, st));
-    TRY(dalloc(h, &h->ovf_s, n, st));
-    TRY(dalloc(h, &h->ovf_s0, n, st));
-    TRY(dalloc(h, &h->ovf3_sorted, n, st));
-    TRY(dalloc(h, &h->cost_bucket, n, st));
-    TRY(dalloc(h, &h->cost_hist, kCostBuckets, st));
-    TRY(dalloc(h, &h->col_off, n, st));
-    TRY(dalloc(h, &h->col_len, n, st));
-    TRY(dalloc(h, &h->col_q, n, st));
-    TRY(dalloc(h, &h->loops, n, st));
-    TRY(dalloc(h, &h->flags, n, st));
-    TRY(dalloc(h, &h->rho, n, st));
-    TRY(dalloc(h, &h->pool_top, 1, st));
-    TRY(dalloc(h, &h->Mcolptr, n + 1, st));
-    TRY(dalloc(h, &h->Mrowptr, n + 1, st));
-    TRY(dalloc(h, &h->row_count, n, st));
-    TRY(dalloc(h, &h->cursor, n, st));
-    h->scan_tmp_len = (n + 1023) / 1024 + 2;
-    TRY(dalloc(h, &h->scan_tmp, h->scan_tmp_len, st));
     TRY(dalloc(h, &h->gwork, h->gstride * (size_t)h->grid_g, st));
-    TRY(dalloc(h, &h->help, HelpBoard::bytes(h->sms), st));
     int status = RSAI_OK;
     {
         Nvtx range("rsai: first build");
@@ -717,9 +750,11 @@ int build_common(rsai_handle *h, cudaStream_t st) {
         for (int attempt = 0; attempt <= kMaxRegrow; ++attempt) {
             unsigned long long top = 0;
             int32_t herr = 0;
-            cudaMemcpyAsync(&top, h->pool_top, sizeof(top), cudaMemcpyDeviceToHost, st);
-            cudaMemcpyAsync(&herr, h->err, sizeof(herr), cudaMemcpyDeviceToHost, st);
+            unsigned long long both[2] = {0, 0};  // kErrWord, kTopWord
+            cudaMemcpyAsync(both, h->zeroed, sizeof(both), cudaMemcpyDeviceToHost, st);
             TRY(cuda_status(cudaStreamSynchronize(st)));
+            memcpy(&herr, &both[kErrWord], sizeof(herr));
+            top = both[kTopWord];
             if ((int64_t)top <= h->pool_cap) {
                 if (herr != 0) status = herr;
                 settled = true;
@@ -738,14 +773,14 @@ int build_common(rsai_handle *h, cudaStream_t st) {
             TRY(alloc_m(h, cap, st));
             // the columns that found the pool full run again (from its current top)
             if (!retry) TRY(dalloc(h, &retry, n, st));
-            cudaMemsetAsync(h->qnext + 7, 0, sizeof(uint32_t), st);
-            k_collect_failed<<<blocks(n, 256), 256, 0, st>>>(h->flags, n, retry, h->qnext + 7);
+            cudaMemsetAsync(h->qnext + kRerun, 0, sizeof(uint32_t), st);
+            k_collect_failed<<<blocks(n, 256), 256, 0, st>>>(h->flags, n, retry, h->qnext + kRerun);
             cudaMemsetAsync(h->dscal + kCtr + CTR_FAILED, 0, sizeof(unsigned long long), st);
             cudaMemsetAsync(h->err, 0, sizeof(int32_t), st);
-            cudaMemsetAsync(h->row_count, 0, sizeof(int32_t) * (size_t)n, st);
-            cudaMemsetAsync(h->cursor, 0, sizeof(int32_t) * (size_t)n, st);
+            cudaMemsetAsync(h->row_count, 0, sizeof(int32_t) * 2 * (size_t)n, st);  // and cursor, which follows
+            cudaMemsetAsync(h->dscal + kCounts, 0, sizeof(unsigned long long) * 2, st);  // n_c, nnz(M): accumulated
             TRY(cuda_status(enqueue_bins(h, MODE_BUILD, dev_a(h), Frozen{}, h->dscal + kCtr, st, nullptr,
-                                         size_global, retry, h->qnext + 7)));
+                                         size_global, retry, h->qnext + kRerun)));
             TRY(cuda_status(enqueue_build_tail(h, st, nullptr)));
         }
         // columns still without room in the pool are flagged and counted as failed
@@ -967,16 +1002,17 @@ rsai_status rsai_rebuild(rsai_handle *h, void *stream) {
 rsai_status rsai_get_stats(rsai_handle *h, void *stream, rsai_stats *out) {
     if (!h || !out) return RSAI_ERR_INVALID_ARG;
     cudaStream_t st = (cudaStream_t)stream;
-    unsigned long long s[kCounts + 2];
     int32_t herr = 0;
     std::vector<double> nb((size_t)h->nblocks);
-    // every read on the caller's stream, one wait
-    if (cudaMemcpyAsync(s, h->dscal, sizeof(s), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-        cudaMemcpyAsync(&herr, h->err, sizeof(herr), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-        cudaMemcpyAsync(nb.data(), h->norm1_arr, sizeof(double) * nb.size(), cudaMemcpyDeviceToHost, st) !=
+    // one read on the caller's stream (a copy to pageable memory waits for the stream)
+    std::vector<unsigned long long> all(kNormWord + nb.size() + kCounts + 2);
+    if (cudaMemcpyAsync(all.data(), h->zeroed, sizeof(all[0]) * all.size(), cudaMemcpyDeviceToHost, st) !=
             cudaSuccess ||
         cudaStreamSynchronize(st) != cudaSuccess)
         return RSAI_ERR_CUDA;
+    memcpy(&herr, &all[kErrWord], sizeof(herr));
+    memcpy(nb.data(), &all[kNormWord], sizeof(double) * nb.size());
+    const unsigned long long *s = all.data() + kNormWord + nb.size();
     auto dbl = [&](int at) {
         double v;
         memcpy(&v, &s[at], sizeof(v));
@@ -1153,13 +1189,13 @@ rsai_status rsai_refit(rsai_handle *h, const double *A_val, double *M_val, doubl
     Nvtx range("rsai_refit");
     if (!h || !A_val) return RSAI_ERR_INVALID_ARG;
     cudaStream_t st = (cudaStream_t)stream;
-    const int64_t nnzM = nnz_of_M(h, st);
-    if (nnzM < 0) return RSAI_ERR_CUDA;
     DevA A;
     int rc = frozen_values(h, A_val, st, &A);
     if (rc != RSAI_OK) return (rsai_status)rc;
     double *mv = M_val, *r2 = rho2;
     double *tmp = nullptr;
+    const int64_t nnzM = mv && r2 ? 0 : nnz_of_M(h, st);  // the size of the temporary
+    if (nnzM < 0) return RSAI_ERR_CUDA;
     const size_t tmp_bytes = sizeof(double) * (size_t)(nnzM + h->n + 1);
     if (!mv || !r2) {  // outputs the caller skipped go to a temporary
         tmp = (double *)raw_alloc(h->allocator, tmp_bytes, st);

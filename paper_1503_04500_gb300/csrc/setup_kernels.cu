@@ -244,7 +244,7 @@ __global__ void k_tau_fixed(const double *norm1, double tol, double *tau, int32_
 }
 
 // ---------------------------------------------------------------------------
-// exclusive scan of int32 counts into int64 offsets (three passes)
+// exclusive scan of int32 counts into int64 offsets (two passes; three above kScanFold blocks)
 
 __global__ void k_scan_blocks(const int32_t *in, int64_t n, int64_t *out, int64_t *block_sums) {
     __shared__ int64_t sh[1024];
@@ -291,6 +291,23 @@ __global__ void k_scan_add(int64_t *out, int64_t n, const int64_t *block_sums, c
     int64_t i = blockIdx.x * 1024LL + threadIdx.x;
     if (i < n) out[i] += block_sums[blockIdx.x];
     if (i == 0) out[n] = *total;
+}
+
+// k_scan_sums and k_scan_add in one: every block adds up the sums of the blocks before it
+__global__ void k_scan_add_fold(int64_t *out, int64_t n, const int64_t *block_sums) {
+    __shared__ int64_t sh[32];
+    int64_t a = 0;
+    for (int64_t b = threadIdx.x; b < (int64_t)blockIdx.x; b += 1024) a += block_sums[b];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = a;
+    __syncthreads();
+    a = 0;
+#pragma unroll
+    for (int w = 0; w < 32; ++w) a += sh[w];
+    const int64_t i = blockIdx.x * 1024LL + threadIdx.x;
+    if (i < n) out[i] += a;
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) out[n] = a + block_sums[blockIdx.x];
 }
 
 // ---------------------------------------------------------------------------

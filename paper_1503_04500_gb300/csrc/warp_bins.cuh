@@ -20,6 +20,7 @@ template <typename T> constexpr int kWarpCtas<T, Caps> = sizeof(T) == 8 ? 1 : 2;
 template <typename T, int MODE, class CapT>
 __global__ void __launch_bounds__(256, kWarpCtas<T, CapT>)
     k_bin_warp(DevA A, DevParams P, CapT cap, ColQueue Q, ColOut O, Frozen F, unsigned long long *gctr, int last_bin) {
+    if (queue_empty(Q)) return;
     extern __shared__ __align__(16) char smem[];
     const int wid = threadIdx.x >> 5;
     Work<T> w;
@@ -32,6 +33,7 @@ __global__ void __launch_bounds__(256, kWarpCtas<T, CapT>)
 template <typename T, int MODE, class CapT>
 __global__ void __launch_bounds__(256, (sizeof(T) == 8 ? 1 : 2))
     k_bin_half(DevA A, DevParams P, CapT cap, ColQueue Q, ColOut O, Frozen F, unsigned long long *gctr, int last_bin) {
+    if (queue_empty(Q)) return;
     extern __shared__ __align__(16) char smem[];
     const int tid = threadIdx.x >> 4;
     Work<T> w;
