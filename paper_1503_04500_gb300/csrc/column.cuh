@@ -539,7 +539,8 @@ template <class Team, typename T, class CapT = Caps> struct Column {
             back_substitute_blocked(team, w.B, q, p, w.rhs, small);
             return;
         }
-        apply_qt_team<Team, T>(team, w.B, q, p, w.rhs, w.vhead, w.tau, small);
+        if constexpr (is_lane_team<Team>::value) apply_qt_lanes<Team, T>(team, w.B, q, p, w.rhs, w.vhead, w.tau, small);
+        else apply_qt_team<Team, T>(team, w.B, q, p, w.rhs, w.vhead, w.tau, small);
     }
 
     // r on the rows of S and, unless `refine`, rho (CTA teams).  The sum of a row
@@ -1311,6 +1312,11 @@ template <class Team, typename T, class CapT = Caps> struct Column {
 
     // rhs[0..p) <- (R^T R)^{-1} rhs[0..p) with R from the last solve
     __device__ void normal_solve(T small) {
+        if constexpr (is_lane_team<Team>::value) {
+            triangular_lanes<false>(team, w.B, q, p, w.rhs, small);
+            triangular_lanes<true>(team, w.B, q, p, w.rhs, small);
+            return;
+        }
         const int me = team.rank();
         for (int i = 0; i < p; ++i) {  // R^T y = rhs (forward, column-oriented)
             T d = w.B[(int64_t)i * q + i];
@@ -1320,8 +1326,7 @@ template <class Team, typename T, class CapT = Caps> struct Column {
             if (me == 0) w.rhs[i] = yi;
             team.sync();
         }
-        if constexpr (is_lane_team<Team>::value) back_substitute_team(team, w.B, q, p, w.rhs, small);
-        else back_substitute_blocked(team, w.B, q, p, w.rhs, small);
+        back_substitute_blocked(team, w.B, q, p, w.rhs, small);
     }
 
     // Refit: solve on the loaded pattern, then the residual.  Returns false on

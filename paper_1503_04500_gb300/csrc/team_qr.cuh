@@ -7,20 +7,6 @@
 
 namespace rsai {
 
-// rhs[0..p) <- R^{-1} rhs[0..p) (column-oriented, in place)
-template <class Team, typename T>
-__device__ void back_substitute_team(const Team &team, const T *B, int q, int p, T *rhs, T small) {
-    const int me = team.rank();
-    for (int i = p - 1; i >= 0; --i) {
-        T d = B[(int64_t)i * q + i];
-        T xi = (fabs(d) <= small) ? T(0) : rhs[i] / d;
-        team.sync();
-        for (int c = me; c < i; c += Team::SIZE) rhs[c] -= B[(int64_t)i * q + c] * xi;
-        if (me == 0) rhs[i] = xi;
-        team.sync();
-    }
-}
-
 // x >= 0, x > 0 and |x| <= y (y >= 0) as the comparisons give them (NaN: false);
 // of doubles on their bit patterns, which keeps the FP64 unit free
 __device__ __forceinline__ bool not_negative(float x) { return x >= 0.0f; }
@@ -36,6 +22,114 @@ __device__ __forceinline__ bool positive(double x) {
 __device__ __forceinline__ bool abs_at_most(float x, float y) { return fabs(x) <= y; }
 __device__ __forceinline__ bool abs_at_most(double x, double y) {
     return abskey(x) <= __double_as_longlong(y) && __double_as_longlong(y) <= 0x7ff0000000000000LL;
+}
+
+// 2 / x.  In FP64 twice the rounded reciprocal, which is the rounded quotient (a
+// power of two scales exactly) for three FP64 instructions less.
+__device__ __forceinline__ float two_over_of(float x) { return 2.0f / x; }
+__device__ __forceinline__ double two_over_of(double x) { return 2.0 * (1.0 / x); }
+
+// a / d for several a with one d.  FP64: Markstein's quotient (IBM J. Res. Dev. 34,
+// 1990) from the rounded reciprocal r of d, an estimate and one correction by its
+// remainder, three FP64 instructions; the plain division where an operand is so
+// small or large that one of them could leave the range.
+template <typename T> struct Divisor;
+template <> struct Divisor<float> {
+    float d;
+    __device__ __forceinline__ explicit Divisor(float x) : d(x) {}
+    __device__ __forceinline__ float into(float a) const { return a / d; }
+};
+__device__ __forceinline__ bool mid_range(double x) {  // 2^-500 <= |x| < 2^500
+    const unsigned e = ((unsigned)__double2hiint(x) >> 20) & 0x7ffu;
+    return e - 523u < 1000u;
+}
+__device__ __forceinline__ bool is_zero(double x) {  // on the bits: the FP64 unit stays free
+    return ((unsigned)__double2hiint(x) << 1 | (unsigned)__double2loint(x)) == 0u;
+}
+template <> struct Divisor<double> {
+    double d, r;
+    bool mid;
+    __device__ __forceinline__ explicit Divisor(double x) : d(x), r(1.0 / x), mid(mid_range(x)) {}
+    __device__ __forceinline__ double into(double a) const {
+        if (mid && (mid_range(a) || is_zero(a))) {
+            const double e = a * r;
+            return fma(fma(-e, d, a), r, e);
+        }
+        return a / d;
+    }
+};
+
+// Triangular solves on a team within a warp, p <= its lanes: lane c keeps rhs[c], and
+// its quotient is formed by every lane beforehand, so that a step is a quotient,
+// a shuffle and one fused multiply-add instead of a trip through shared memory with
+// two synchronisations.  UP: R x = rhs, from the last row; else R^T y = rhs.
+template <bool UP, class Team, typename T>
+__device__ __forceinline__ void triangular_lanes(const Team &team, const T *B, int q, int p, T *rhs, T small) {
+    const int me = team.rank();
+    const bool mine = me < p;
+    const T dd = mine ? B[me * q + me] : T(1);
+    const bool zero = abs_at_most(dd, small);
+    const Divisor<T> div(dd);
+    T x = mine ? rhs[me] : T(0);
+    const T *row = UP ? B + me : B + (mine ? me : 0) * q;
+    const int step = UP ? q : 1;
+    for (int t = 0; t < p; ++t) {
+        const int i = UP ? p - 1 - t : t;
+        const bool below = mine && (UP ? me < i : me > i);
+        const T b = below ? row[i * step] : T(0);
+        const T xi = team.bcast(zero ? T(0) : div.into(x), i);
+        if (below) x -= b * xi;
+        else if (me == i) x = xi;
+    }
+    if (mine) rhs[me] = x;
+    team.sync();
+}
+
+// rhs <- Q^T rhs with the stored reflectors, then R^{-1}, on a team within a warp:
+// rows me, me + W, .. of rhs stay in registers (q <= 4 W in every such bin), and the
+// next reflector is read while the dot product of one is reduced.
+template <class Team, typename T>
+__device__ __noinline__ void apply_qt_lanes(Team team, const T *B, int q, int p, T *rhs, const T *vhead, const T *taus,
+                                            T small) {
+    constexpr int W = Team::SIZE, R = 4;
+    const int me = team.rank();
+    T x[R], vn[R], v0n = vhead[0], taun = taus[0];
+#pragma unroll
+    for (int u = 0; u < R; ++u) {
+        const int i = me + W * u;
+        x[u] = i < q ? rhs[i] : T(0);
+        vn[u] = i < q ? B[i] : T(0);
+    }
+    for (int j = 0; j < p; ++j) {
+        T v[R];
+        const T tau = taun;
+#pragma unroll
+        for (int u = 0; u < R; ++u) v[u] = me + W * u == j ? v0n : vn[u];
+        if (j + 1 < p) {
+            v0n = vhead[j + 1];
+            taun = taus[j + 1];
+#pragma unroll
+            for (int u = 0; u < R; ++u) {
+                const int i = me + W * u;
+                vn[u] = i < q ? B[(j + 1) * q + i] : T(0);
+            }
+        }
+        if (tau > T(0)) {
+            T d = T(0);
+#pragma unroll
+            for (int u = 0; u < R; ++u)
+                if (me + W * u >= j && me + W * u < q) d += v[u] * x[u];
+            const T f = team.sum(d) * tau;
+#pragma unroll
+            for (int u = 0; u < R; ++u)
+                if (me + W * u >= j) x[u] -= f * v[u];
+        }
+    }
+#pragma unroll
+    for (int u = 0; u < R; ++u)
+        if (me + W * u < q) rhs[me + W * u] = x[u];
+    team.sync();
+    triangular_lanes<true>(team, B, q, p, rhs, small);
 }
 
 // A Householder update of the M columns c0..c0+M-1 of B (c == p: rhs; past p:
@@ -98,7 +192,7 @@ template <typename T> __device__ __forceinline__ void reflector(T sigma, T x0, T
     alpha = not_negative(x0) ? -nrm : nrm;
     v0 = x0 - alpha;
     const T vtv = sigma - x0 * x0 + v0 * v0;
-    two_over = positive(vtv) ? T(2) / vtv : T(0);
+    two_over = positive(vtv) ? two_over_of(vtv) : T(0);
 }
 
 // This thread's terms of the sum of squares of col[j..q) (BlockTeam::sum_rows)
@@ -211,14 +305,14 @@ __device__ __forceinline__ void householder_step(const Team &team, T *B, int q, 
 }
 
 // Householder QR of B (q x p, column-major, ld q) applied to rhs, then back
-// substitution into rhs[0..p).  Keeps the reflectors (v_j below the diagonal
-// of B, heads in vhead, tau = 2 / v^T v in tau) for the refinement solve.  Returns the
-// rank flag.  Team-generic, one team synchronisation per step; not inlined.
+// substitution into rhs[0..p), on a team within a warp.  Keeps the reflectors (v_j below
+// the diagonal of B, heads in vhead, tau = 2 / v^T v in tau) for the refinement solve.
+// Returns the rank flag.  Not inlined.
 template <class Team, typename T>
 __device__ __noinline__ int qr_solve_team(Team team, T *B, int q, int p, T *rhs, T *vhead, T *taus, T small) {
     int rank_flag = 0;
     for (int j = 0; j < p; ++j) householder_step(team, B, q, p, rhs, vhead, taus, j, j + 1, small, rank_flag);
-    back_substitute_team(team, B, q, p, rhs, small);
+    triangular_lanes<true>(team, B, q, p, rhs, small);
     return rank_flag;
 }
 
@@ -282,7 +376,7 @@ __device__ void back_substitute_blocked(const Team &team, const T *B, int q, int
     }
 }
 
-// rhs <- Q^T rhs with the stored reflectors, then R^{-1}; not inlined
+// rhs <- Q^T rhs with the stored reflectors, then R^{-1}, on a CTA; not inlined
 template <class Team, typename T>
 __device__ __noinline__ void apply_qt_team(Team team, const T *B, int q, int p, T *rhs, const T *vhead,
                                            const T *taus, T small) {
@@ -291,30 +385,20 @@ __device__ __noinline__ void apply_qt_team(Team team, const T *B, int q, int p, 
         const T *col = B + (int64_t)j * q;
         const T v0 = vhead[j], tau = taus[j];
         if (tau > T(0)) {
-            T sdot;
-            if constexpr (is_lane_team<Team>::value) {
-                T d = 0;
-                for (int i = me; i < q; i += Team::SIZE)
-                    if (i >= j) d += ((i == j) ? v0 : col[i]) * rhs[i];
-                sdot = team.sum(d);
-            } else {
-                T d[Team::VK];
+            T d[Team::VK];
 #pragma unroll
-                for (int v = 0; v < Team::VK; ++v) {
-                    d[v] = T(0);
-                    for (int i = me + v * Team::SIZE; i < q; i += Team::VK == 1 ? Team::SIZE : q)
-                        if (i >= j) d[v] += ((i == j) ? v0 : col[i]) * rhs[i];
-                }
-                sdot = team.sum_rows(d);
+            for (int v = 0; v < Team::VK; ++v) {
+                d[v] = T(0);
+                for (int i = me + v * Team::SIZE; i < q; i += Team::VK == 1 ? Team::SIZE : q)
+                    if (i >= j) d[v] += ((i == j) ? v0 : col[i]) * rhs[i];
             }
-            T f = sdot * tau;
+            const T f = team.sum_rows(d) * tau;
             for (int i = me; i < q; i += Team::SIZE)
                 if (i >= j) rhs[i] -= f * ((i == j) ? v0 : col[i]);
         }
         team.sync();
     }
-    if constexpr (is_lane_team<Team>::value) back_substitute_team(team, B, q, p, rhs, small);
-    else back_substitute_blocked(team, B, q, p, rhs, small);
+    back_substitute_blocked(team, B, q, p, rhs, small);
 }
 
 // The reflectors j0..j1-1 (built on q0 rows) applied in order to the columns
