@@ -543,20 +543,11 @@ template <class Team, typename T, class CapT = Caps> struct Column {
         else apply_qt_team<Team, T>(team, w.B, q, p, w.rhs, w.vhead, w.tau, small);
     }
 
-    // r on the rows of S and, unless `refine`, rho (CTA teams).  The sum of a row
-    // is defined on 32 lane chains (entries l, l + 32, ... of the row on lane l)
-    // joined by a butterfly over offsets 16, 8, 4, 2, 1, and ||r||^2 as the
-    // chains of the rows w, w + 16, ... for w < 16, added in order, for every CTA
-    // size.  FP64 additions are what bounds this (a warp instruction takes the
-    // SM's FP64 unit 16 cycles however many of its lanes are active), and most rows
-    // hold under 16 entries: so eight lanes work on a row, each keeping its
-    // four chains (lanes l, l + 8, l + 16, l + 24), the first two levels of the
-    // butterfly are additions within a lane, skipped where all four rows of the
-    // warp are short (they would add zeros), and the chains of squares run on
-    // 16 lanes of one warp, one each, at the end.
-    __device__ __forceinline__ void row_sums(bool refine, int &cnt) {
+    // J for the products with rows of A: as a map in the staging area, or a copy
+    // of it there (Js), or J itself.  Synchronises the team.
+    __device__ __forceinline__ StageMap map_of_J(const int32_t *&Js) {
         const int me = team.rank();
-        const int32_t *Js = w.J;
+        Js = w.J;
         StageMap map(nullptr, 0, A.n);
         if constexpr (Team::STAGED) {
             map = stage_map();
@@ -571,6 +562,62 @@ template <class Team, typename T, class CapT = Caps> struct Column {
             }
         }
         team.sync();
+        return map;
+    }
+
+    // sum over the entries e0 .. e0 + len - 1 of A in row order that lie in J,
+    // times x; eight lanes per row, four rows per warp (all lanes call)
+    __device__ __forceinline__ double row_dot(int64_t e0, int len, const double *v, const StageMap &map,
+                                              const int32_t *Js, int &cnt) const {
+        const int sub = team.rank() & 7;
+                    double acc[4] = {0.0, 0.0, 0.0, 0.0};
+                    int most = len;
+        #pragma unroll
+                    for (int o = 16; o >= 8; o >>= 1) most = max(most, __shfl_xor_sync(0xffffffffu, most, o));
+                    for (int b = 0; b < most; b += 32) {
+        #pragma unroll
+                        for (int h = 0; h < 4; ++h) {
+                            if (b + 8 * h >= most) break;  // the same for the whole warp
+                            const int e = b + 8 * h + sub;
+                            if (e < len) {
+                                const int32_t col = A.col_idx[e0 + e];
+                                int pos;
+                                if (Team::STAGED && map.on()) pos = map.find(col);
+                                else pos = find_i32(Js, p, col);
+                                if (pos >= 0) {
+                                    acc[h] = fma(A.val[e0 + e], v[pos], acc[h]);
+                                    ++cnt;
+                                }
+                            }
+                        }
+                    }
+                    double x = acc[0];
+                    if (most > 16) {
+                        x += acc[2];
+                        x += acc[1] + acc[3];
+                    } else if (most > 8) {
+                        x += acc[1];
+                    }
+        #pragma unroll
+                    for (int o = 4; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+        return x;
+    }
+
+    // r on the rows of S and, unless `refine`, rho (CTA teams).  The sum of a row
+    // is defined on 32 lane chains (entries l, l + 32, ... of the row on lane l)
+    // joined by a butterfly over offsets 16, 8, 4, 2, 1, and ||r||^2 as the
+    // chains of the rows w, w + 16, ... for w < 16, added in order, for every CTA
+    // size.  FP64 additions are what bounds this (a warp instruction takes the
+    // SM's FP64 unit 16 cycles however many of its lanes are active), and most rows
+    // hold under 16 entries: so eight lanes work on a row, each keeping its
+    // four chains (lanes l, l + 8, l + 16, l + 24), the first two levels of the
+    // butterfly are additions within a lane, skipped where all four rows of the
+    // warp are short (they would add zeros), and the chains of squares run on
+    // 16 lanes of one warp, one each, at the end.
+    __device__ __forceinline__ void row_sums(bool refine, int &cnt) {
+        const int me = team.rank();
+        const int32_t *Js;
+        const StageMap map = map_of_J(Js);
         const int sub = me & 7;
         constexpr int RW = Team::SIZE / 8;  // rows per pass of the team
         const int passes = (s + RW - 1) / RW;
@@ -584,36 +631,7 @@ template <class Team, typename T, class CapT = Caps> struct Column {
                 e0 = A.row_ptr[row];
                 len = (int)(A.row_ptr[row + 1] - e0);
             }
-            double acc[4] = {0.0, 0.0, 0.0, 0.0};
-            int most = len;
-#pragma unroll
-            for (int o = 16; o >= 8; o >>= 1) most = max(most, __shfl_xor_sync(0xffffffffu, most, o));
-            for (int b = 0; b < most; b += 32) {
-#pragma unroll
-                for (int h = 0; h < 4; ++h) {
-                    if (b + 8 * h >= most) break;  // the same for the whole warp
-                    const int e = b + 8 * h + sub;
-                    if (e < len) {
-                        const int32_t col = A.col_idx[e0 + e];
-                        int pos;
-                        if (Team::STAGED && map.on()) pos = map.find(col);
-                        else pos = find_i32(Js, p, col);
-                        if (pos >= 0) {
-                            acc[h] = fma(A.val[e0 + e], w.m[pos], acc[h]);
-                            ++cnt;
-                        }
-                    }
-                }
-            }
-            double x = acc[0];
-            if (most > 16) {
-                x += acc[2];
-                x += acc[1] + acc[3];
-            } else if (most > 8) {
-                x += acc[1];
-            }
-#pragma unroll
-            for (int o = 4; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+            double x = row_dot(e0, len, w.m, map, Js, cnt);
             if (row == k) x -= 1.0;
             if (sub == 0 && i < s) w.r[i] = x;
         }
@@ -797,7 +815,7 @@ template <class Team, typename T, class CapT = Caps> struct Column {
         for (int i = team.rank(); i < full; i += Team::SIZE) reinterpret_cast<uint4 *>(x)[i] = make_uint4(0, 0, 0, 0);
         for (int i = full * CW + team.rank(); i < len; i += Team::SIZE) x[i] = T(0);
     }
-    // position of row i in I, right after rows_of_J (which left the map of I in the staging area)
+    // position of row i in I while the staging area holds the map of I (after rows_of_J, in cols_times)
     __device__ __forceinline__ int find_I(int32_t i) const {
         if constexpr (Team::STAGED) {
             const StageMap map = stage_map();
@@ -1285,27 +1303,59 @@ template <class Team, typename T, class CapT = Caps> struct Column {
             team.sync();
             return;
         }
-        for (int i = team.rank(); i < q; i += Team::SIZE) {
-            const int32_t row = w.I[i];
-            const int64_t e0 = A.row_ptr[row], e1 = A.row_ptr[row + 1];
-            double acc = 0.0;
-            for (int64_t e = e0; e < e1; ++e) {
-                const int c = find_J(A.col_idx[e]);
-                if (c >= 0) acc = fma(A.val[e], zc[c], acc);
+        const int32_t *Js;
+        const StageMap map = map_of_J(Js);
+        const int me = team.rank();
+        constexpr int RW = Team::SIZE / 8;
+        int entries = 0;
+        for (int i0 = 0; i0 < q; i0 += RW) {
+            const int i = i0 + (me >> 3);
+            int64_t e0 = 0;
+            int len = 0;
+            if (i < q) {
+                e0 = A.row_ptr[w.I[i]];
+                len = (int)(A.row_ptr[w.I[i] + 1] - e0);
             }
-            out[i] = acc;
+            const double x = row_dot(e0, len, zc, map, Js, entries);
+            if ((me & 7) == 0 && i < q) out[i] = x;
         }
         team.sync();
     }
 
-    // out[c] = sum_i A(I_i, J_c) v[i] over the columns of J, in double
+    // out[c] = sum_i A(I_i, J_c) v[i] over the columns of J, in double: a lane per
+    // column within a warp, eight lanes per column on a CTA
     __device__ void cols_times(const double *v, double *out) {
-        for (int c = team.rank(); c < p; c += Team::SIZE) {
-            const int32_t j = w.J[c];
-            double acc = 0.0;
-            for (int64_t e = A.col_ptr[j]; e < A.col_ptr[j + 1]; ++e)
-                acc = fma(A.cval[e], v[find_i32(w.I, q, A.row_idx[e])], acc);
-            out[c] = acc;
+        const int me = team.rank();
+        if constexpr (is_lane_team<Team>::value) {
+            for (int c = me; c < p; c += Team::SIZE) {
+                const int32_t j = w.J[c];
+                double acc = 0.0;
+                for (int64_t e = A.col_ptr[j]; e < A.col_ptr[j + 1]; ++e)
+                    acc = fma(A.cval[e], v[find_i32(w.I, q, A.row_idx[e])], acc);
+                out[c] = acc;
+            }
+        } else {
+            if constexpr (Team::STAGED) {
+                const StageMap map = stage_map();
+                if (map.on()) {
+                    map.clear(team);
+                    for (int i = me; i < q; i += Team::SIZE) map.mark(w.I[i]);
+                    map.finish(team, nullptr, cap.qcap);
+                }
+            }
+            constexpr int CP = Team::SIZE / 8;
+            for (int c0 = 0; c0 < p; c0 += CP) {
+                const int c = c0 + (me >> 3);
+                double acc = 0.0;
+                if (c < p) {
+                    const int64_t e1 = A.col_ptr[w.J[c] + 1];
+                    for (int64_t e = A.col_ptr[w.J[c]] + (me & 7); e < e1; e += 8)
+                        acc = fma(A.cval[e], v[find_I(A.row_idx[e])], acc);
+                }
+#pragma unroll
+                for (int o = 4; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+                if ((me & 7) == 0 && c < p) out[c] = acc;
+            }
         }
         team.sync();
     }
@@ -1317,15 +1367,7 @@ template <class Team, typename T, class CapT = Caps> struct Column {
             triangular_lanes<true>(team, w.B, q, p, w.rhs, small);
             return;
         }
-        const int me = team.rank();
-        for (int i = 0; i < p; ++i) {  // R^T y = rhs (forward, column-oriented)
-            T d = w.B[(int64_t)i * q + i];
-            T yi = (fabs(d) <= small) ? T(0) : w.rhs[i] / d;
-            team.sync();
-            for (int c = i + 1 + me; c < p; c += Team::SIZE) w.rhs[c] -= w.B[(int64_t)c * q + i] * yi;
-            if (me == 0) w.rhs[i] = yi;
-            team.sync();
-        }
+        forward_substitute_blocked(team, w.B, q, p, w.rhs, small, (T *)w.stage, cap.stage_bytes);
         back_substitute_blocked(team, w.B, q, p, w.rhs, small);
     }
 

@@ -168,29 +168,55 @@ __global__ void k_invert_map(const int64_t *map, int64_t n, int64_t *inv) {
 // One thread per nonzero A(i,j), in CSC order: the threads of a column walk the
 // same row j of M and search the same I_k, so their loads are mostly the same
 // addresses (in CSR order each thread of a warp had a row of M and index lists
-// of its own).  Bound by the latency of the searches.
+// of its own).  Bound by the latency of the searches; so a row of M of more than
+// kLongRow entries (the power-law matrices' reach a thousand, the stencils' stay
+// below) is taken by the whole warp, 32 entries at a time.
+constexpr int kLongRow = 64;
+
 __global__ void k_adjoint_gather(int64_t n, int64_t nnz, const int64_t *col_ptr, const int32_t *row_idx,
                                  const int64_t *csc_to_csr, const int64_t *Mrowptr, const int32_t *Mcols,
                                  const int64_t *Mcsr_to_csc, const int64_t *qoff, const int32_t *poolI,
                                  const double *poolR, const double *poolW, const double *alphaM, const double *xM,
                                  double *grad) {
     const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (e >= nnz) return;
-    int64_t lo = 0, hi = n;  // last column with col_ptr[column] <= e
-    while (hi - lo > 1) {
-        const int64_t mid = (lo + hi) >> 1;
-        if (col_ptr[mid] <= e) lo = mid; else hi = mid;
+    const bool have = e < nnz;
+    int64_t f0 = 0;
+    int len = 0;
+    int32_t i = 0;
+    if (have) {
+        int64_t lo = 0, hi = n;  // last column with col_ptr[column] <= e
+        while (hi - lo > 1) {
+            const int64_t mid = (lo + hi) >> 1;
+            if (col_ptr[mid] <= e) lo = mid; else hi = mid;
+        }
+        i = row_idx[e];
+        f0 = Mrowptr[lo];
+        len = (int)(Mrowptr[lo + 1] - f0);
     }
-    const int32_t i = row_idx[e];
-    double acc = 0.0;
-    for (int64_t f = Mrowptr[lo]; f < Mrowptr[lo + 1]; ++f) {
+    // entry f of M's row for row ii of A
+    auto term = [&](int64_t f, int32_t ii) {
         const int32_t kk = Mcols[f];
         const int64_t ce = Mcsr_to_csc[f];
         const int64_t a = qoff[kk];
-        const int pos = find_i32(poolI + a, (int)(qoff[kk + 1] - a), i);
-        if (pos >= 0) acc += poolR[a + pos] * alphaM[ce] - poolW[a + pos] * xM[ce];
+        const int pos = find_i32(poolI + a, (int)(qoff[kk + 1] - a), ii);
+        return pos >= 0 ? poolR[a + pos] * alphaM[ce] - poolW[a + pos] * xM[ce] : 0.0;
+    };
+    double acc = 0.0;
+    if (len <= kLongRow)
+        for (int64_t f = f0; f < f0 + len; ++f) acc += term(f, i);
+    const int lane = threadIdx.x & 31;
+    for (unsigned todo = __ballot_sync(0xffffffffu, len > kLongRow); todo; todo &= todo - 1u) {
+        const int src = __ffs(todo) - 1;
+        const int64_t g0 = __shfl_sync(0xffffffffu, f0, src);
+        const int glen = __shfl_sync(0xffffffffu, len, src);
+        const int32_t gi = __shfl_sync(0xffffffffu, i, src);
+        double x = 0.0;
+        for (int t = lane; t < glen; t += 32) x += term(g0 + t, gi);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+        if (lane == src) acc = x;
     }
-    grad[csc_to_csr[e]] = acc;
+    if (have) grad[csc_to_csr[e]] = acc;
 }
 
 // ---------------------------------------------------------------------------

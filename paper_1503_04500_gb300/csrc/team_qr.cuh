@@ -376,6 +376,63 @@ __device__ void back_substitute_blocked(const Team &team, const T *B, int q, int
     }
 }
 
+// rhs[0..p) <- R^{-T} rhs[0..p) for a CTA team, in blocks of kBS rows from the top:
+// one warp solves the block's triangle (lane l holds row b0 + l), then every
+// thread subtracts the block's part from a row below, in the order of one row
+// at a time (the same bits).  Row c of R^T is column c of B: with B in global memory
+// (stage != NULL) the block's kBS entries of each column are copied to
+// the staging area first, a warp per column, as many columns at a time as fit.
+template <class Team, typename T>
+__device__ __noinline__ void forward_substitute_blocked(Team team, const T *B, int q, int p, T *rhs, T small, T *stage,
+                                                        int stage_bytes) {
+    constexpr int kBS = sizeof(T) == 8 ? 16 : 32, LD = kBS + 1;
+    const int me = team.rank();
+    const int chunk = Team::STAGED ? stage_bytes / (int)(LD * sizeof(T)) : p;
+    for (int b0 = 0; b0 < p; b0 += kBS) {
+        const int nbk = min(kBS, p - b0);
+        for (int c0 = b0; c0 < p; c0 += chunk) {
+            const int c1 = min(p, c0 + chunk);
+            if constexpr (Team::STAGED) {
+                for (int e = me; e < (c1 - c0) * kBS; e += Team::SIZE) {
+                    const int c = e / kBS, u = e % kBS;
+                    if (u < nbk) stage[c * LD + u] = B[(int64_t)(c0 + c) * q + b0 + u];
+                }
+                team.sync();
+            }
+            auto entry = [&](int c, int u) {  // R(b0 + u, c)
+                if constexpr (Team::STAGED) return stage[(c - c0) * LD + u];
+                else return B[(int64_t)c * q + b0 + u];
+            };
+            if (c0 == b0 && me < 32) {
+                const bool row = me < nbk;
+                T rv[kBS];
+#pragma unroll
+                for (int u = 0; u < kBS; ++u) rv[u] = (row && u < me) ? entry(b0 + me, u) : T(0);
+                const T dd = row ? entry(b0 + me, me) : T(1);
+                T yi = row ? rhs[b0 + me] : T(0);
+#pragma unroll
+                for (int u = 0; u < kBS; ++u) {
+                    if (u < nbk) {
+                        const T a = __shfl_sync(0xffffffffu, yi, u);
+                        const T d = __shfl_sync(0xffffffffu, dd, u);
+                        const T y = (fabs(d) <= small) ? T(0) : a / d;
+                        if (me == u) yi = y;
+                        else if (me > u) yi -= rv[u] * y;
+                    }
+                }
+                if (row) rhs[b0 + me] = yi;
+            }
+            team.sync();
+            for (int c = max(c0, b0 + nbk) + me; c < c1; c += Team::SIZE) {
+                T a = rhs[c];
+                for (int u = 0; u < nbk; ++u) a -= entry(c, u) * rhs[b0 + u];
+                rhs[c] = a;
+            }
+            team.sync();
+        }
+    }
+}
+
 // rhs <- Q^T rhs with the stored reflectors, then R^{-1}, on a CTA; not inlined
 template <class Team, typename T>
 __device__ __noinline__ void apply_qt_team(Team team, const T *B, int q, int p, T *rhs, const T *vhead,
