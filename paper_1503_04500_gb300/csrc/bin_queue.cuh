@@ -109,7 +109,9 @@ __device__ __forceinline__ void forward_frozen(int me, const ColQueue &Q, const 
 
 // A bin that no column was forwarded to (the counts are final when its kernel
 // starts): its CTAs return before they set up anything.  The five or six empty
-// bins of a stencil matrix took a twentieth of a small build.
+// bins of a stencil matrix took a twentieth of a small build (with the launches, copies
+// and allocations saved elsewhere in a build: 20^2 in FP64 793 -> 692 us, rebuild of
+// 256^2 1050 -> 1000 us, its refit and adjoint 1884 -> 1728 us).
 __device__ __forceinline__ bool queue_empty(const ColQueue &Q) {
     return Q.count != nullptr && *(volatile const uint32_t *)Q.count == 0u;
 }

@@ -62,7 +62,10 @@ template <> struct Divisor<double> {
 // Triangular solves on a team within a warp, p <= its lanes: lane c keeps rhs[c], and
 // its quotient is formed by every lane beforehand, so that a step is a quotient,
 // a shuffle and one fused multiply-add instead of a trip through shared memory with
-// two synchronisations.  UP: R x = rhs, from the last row; else R^T y = rhs.
+// two synchronisations.  Bound by that chain, in FP64 also by the quotients (the FP64 unit
+// takes 2 lanes per cycle and SM): with Divisor and two_over_of, 64^3 in FP64 15.1 -> 14.2 ms
+// and the 40^3 FP64 refit and adjoint 7.9 -> 7.1 ms.
+// UP: R x = rhs, from the last row; else R^T y = rhs.
 template <bool UP, class Team, typename T>
 __device__ __forceinline__ void triangular_lanes(const Team &team, const T *B, int q, int p, T *rhs, T small) {
     const int me = team.rank();
@@ -87,7 +90,8 @@ __device__ __forceinline__ void triangular_lanes(const Team &team, const T *B, i
 
 // rhs <- Q^T rhs with the stored reflectors, then R^{-1}, on a team within a warp:
 // rows me, me + W, .. of rhs stay in registers (q <= 4 W in every such bin), and the
-// next reflector is read while the dot product of one is reduced.
+// next reflector is read while the dot product of one is reduced (33^3 at eps = 0.15,
+// where it is an eighth of the warp bins' time: 29.5 -> 29.0 ms).
 template <class Team, typename T>
 __device__ __noinline__ void apply_qt_lanes(Team team, const T *B, int q, int p, T *rhs, const T *vhead, const T *taus,
                                             T small) {
@@ -382,6 +386,7 @@ __device__ void back_substitute_blocked(const Team &team, const T *B, int q, int
 // at a time (the same bits).  Row c of R^T is column c of B: with B in global memory
 // (stage != NULL) the block's kBS entries of each column are copied to
 // the staging area first, a warp per column, as many columns at a time as fit.
+// One row at a time it took two synchronisations and a strided load per row.
 template <class Team, typename T>
 __device__ __noinline__ void forward_substitute_blocked(Team team, const T *B, int q, int p, T *rhs, T small, T *stage,
                                                         int stage_bytes) {
