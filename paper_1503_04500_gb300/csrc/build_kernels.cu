@@ -5,16 +5,17 @@
 // Bins (one persistent launch each, columns pulled from an atomic queue; the
 // columns are independent, Section 2 Eq. 2.2):
 //   H  half a warp per column, two columns per warp, workspace in shared
-//      memory (the smallest LS problems: |I| <= 48, |J| <= 16, e.g. 3-D
-//      7-point stencils)
-//   W  one warp per column, workspace in shared memory (small LS problems,
-//      e.g. stencil matrices: |I| <= 64, |J| <= 32)
+//      memory (|I| <= 48, |J| <= 16, e.g. 3-D 7-point stencils; first bin in FP64)
+//   W0 one warp per column, the same sizes (first bin in FP32)
+//   W  one warp per column (|I| <= 64, |J| <= 32)
 //   W2 the same kernel with |I| <= 128 (fewer warps per SM)
+//   S0 one CTA of 64 threads per column, workspace in shared memory (|I| <= 96, |J| <= 40)
+//   S  one CTA of 128 threads (|I| <= 128, |J| <= 64)
 //   C  one CTA per column, workspace in shared memory (up to ~200 KB)
 //   G  one CTA per column, workspace in a global-memory slab per CTA (the
 //      long tail of matrices with dense rows, Section 4 "row irregular")
-// A column that outgrows a bin is pushed to the next bin's queue and
-// restarted there from J = {k}; the result is the same column of M.
+// A column that outgrows a bin is pushed to the next bin's queue (past those too
+// narrow for its |J|) and restarted there from J = {k}; the result is the same column of M.
 #include "kernels.h"
 
 namespace rsai {
