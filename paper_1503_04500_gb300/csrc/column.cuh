@@ -273,12 +273,12 @@ __device__ __noinline__ SpaiPick spai_select(Team team, DevA A, int c, double ti
         if (i < s && abskey(r[i]) > bk) {
             const int32_t row = S[i];
             st = A.row_ptr[row];
-            len = (int)(A.row_ptr[row + 1] - st);
+            len = counted_entries(A.row_ptr[row + 1] - st, scap);
             byt += 4LL * len + 16;
         }
         int part;
         const int off = tot + team.scan(len, &part);
-        if (next_pow2(tot + part) > scap) {
+        if (tot + part > scap) {
             out.na = -1;
             return out;
         }
@@ -417,7 +417,7 @@ template <class Team, typename T, class CapT = Caps> struct Column {
                 int entries = 0;
                 for (int c = team.rank(); c < p; c += Team::SIZE) {
                     const int64_t st = A.col_ptr[w.J[c]];
-                    const int len = (int)(A.col_ptr[w.J[c] + 1] - st);
+                    const int len = counted_entries(A.col_ptr[w.J[c] + 1] - st, cap.scap);
                     entries += len;
                     for (int e = 0; e < len; e += 4) {
                         int32_t v[4];
@@ -430,7 +430,7 @@ template <class Team, typename T, class CapT = Caps> struct Column {
                 }
                 entries = team.sum(entries);
                 const int nq = map.finish(team, w.I, cap.qcap);
-                if (next_pow2(entries) > cap.scap || nq > cap.qcap) return false;
+                if (entries > cap.scap || nq > cap.qcap) return false;
                 q = nq;
                 return true;
             }
@@ -442,11 +442,11 @@ template <class Team, typename T, class CapT = Caps> struct Column {
             int64_t st = 0;
             if (c < p) {
                 st = A.col_ptr[w.J[c]];
-                len = (int)(A.col_ptr[w.J[c] + 1] - st);
+                len = counted_entries(A.col_ptr[w.J[c] + 1] - st, cap.scap);
             }
             int tot;
             int off = team.scan(len, &tot);
-            if (next_pow2(base + tot) > cap.scap) return false;
+            if (base + tot > cap.scap) return false;
             for (int e = 0; e < len; e += 4) {
                 int32_t v[4];
 #pragma unroll
@@ -739,11 +739,11 @@ template <class Team, typename T, class CapT = Caps> struct Column {
         int64_t st = 0;
         if (me < p) {
             st = A.col_ptr[w.J[me]];
-            len = (int)(A.col_ptr[w.J[me] + 1] - st);
+            len = counted_entries(A.col_ptr[w.J[me] + 1] - st, cap.scap);
         }
         int tot;
         const int off = team.scan(len, &tot);
-        if (next_pow2(tot) > cap.scap) return false;
+        if (tot > cap.scap) return false;
         for (int e = 0; e < len; e += 4) {
             int32_t v[4];
 #pragma unroll
@@ -1207,12 +1207,13 @@ template <class Team, typename T, class CapT = Caps> struct Column {
                 map.clear(team);
                 int entries = 0;
                 for (int t = me >> 5; t < nh; t += Team::SIZE / 32) {
-                    const int64_t st = A.row_ptr[w.Rhat[t]], en = A.row_ptr[w.Rhat[t] + 1];
-                    if ((me & 31) == 0) entries += (int)(en - st);
-                    for (int64_t e = st + (me & 31); e < en; e += 32) map.mark(A.col_idx[e]);
+                    const int64_t st = A.row_ptr[w.Rhat[t]];
+                    const int len = counted_entries(A.row_ptr[w.Rhat[t] + 1] - st, cap.scap);
+                    if ((me & 31) == 0) entries += len;
+                    for (int e = me & 31; e < len; e += 32) map.mark(A.col_idx[st + e]);
                 }
                 entries = team.sum(entries);
-                if (next_pow2(entries) > cap.scap) return -1;
+                if (entries > cap.scap) return -1;
                 for (int c = me; c < p; c += Team::SIZE) map.unmark(w.J[c]);
                 // at most `entries` <= scap columns: buf holds them
                 return map.finish(team, w.buf, cap.scap);
@@ -1225,11 +1226,11 @@ template <class Team, typename T, class CapT = Caps> struct Column {
             int64_t st = 0;
             if (t < nh) {
                 st = A.row_ptr[w.Rhat[t]];
-                len = (int)(A.row_ptr[w.Rhat[t] + 1] - st);
+                len = counted_entries(A.row_ptr[w.Rhat[t] + 1] - st, cap.scap);
             }
             int part;
             const int off = tot + team.scan(len, &part);
-            if (next_pow2(tot + part) > cap.scap) return -1;
+            if (tot + part > cap.scap) return -1;
             for (int e = 0; e < len; e += 4) {
                 int32_t v[4];
 #pragma unroll

@@ -108,6 +108,14 @@ template <typename T> struct Unit;
 template <> struct Unit<float> { static constexpr double u = 5.9604644775390625e-08; };
 template <> struct Unit<double> { static constexpr double u = 1.1102230246251565e-16; };
 
+// Entries of a row or column that go to a buffer of `room`: all of them, or room + 1 when
+// they do not fit.  Sums over the rows or columns of a bin (at most 4096 of them,
+// room <= 131072) stay within 32 bits whatever the matrix holds (a thousand dense columns
+// of a million rows pass 2^30), and are above `room` exactly when the true sum is.
+__host__ __device__ __forceinline__ int counted_entries(int64_t len, int room) {
+    return len > room ? room + 1 : (int)len;
+}
+
 __device__ __forceinline__ int lower_bound_i32(const int32_t *a, int len, int32_t v) {
     int lo = 0, hi = len;
     while (lo < hi) {
