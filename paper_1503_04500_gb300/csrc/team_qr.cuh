@@ -24,15 +24,20 @@ __device__ __forceinline__ bool abs_at_most(double x, double y) {
     return abskey(x) <= __double_as_longlong(y) && __double_as_longlong(y) <= 0x7ff0000000000000LL;
 }
 
-// 2 / x.  In FP64 twice the rounded reciprocal, which is the rounded quotient (a
-// power of two scales exactly) for three FP64 instructions less.
+// 2 / x, x > 0.  In FP64 twice the rounded reciprocal, which is the rounded quotient (a
+// power of two scales exactly) for three FP64 instructions less; from 2^1021 on, where
+// the reciprocal comes near the subnormals and is rounded to fewer bits, the division.
 __device__ __forceinline__ float two_over_of(float x) { return 2.0f / x; }
-__device__ __forceinline__ double two_over_of(double x) { return 2.0 * (1.0 / x); }
+__device__ __forceinline__ double two_over_of(double x) {
+    return __double2hiint(x) < 0x7fc00000 ? 2.0 * (1.0 / x) : 2.0 / x;
+}
 
 // a / d for several a with one d.  FP64: Markstein's quotient (IBM J. Res. Dev. 34,
 // 1990) from the rounded reciprocal r of d, an estimate and one correction by its
 // remainder, three FP64 instructions; the plain division where an operand is so
-// small or large that one of them could leave the range.
+// small or large that one of them could leave the range.  The bits of the division
+// in every case: of a zero the estimate, which has the quotient's sign (the
+// correction would add +0 to it).
 template <typename T> struct Divisor;
 template <> struct Divisor<float> {
     float d;
@@ -52,8 +57,8 @@ template <> struct Divisor<double> {
     __device__ __forceinline__ explicit Divisor(double x) : d(x), r(1.0 / x), mid(mid_range(x)) {}
     __device__ __forceinline__ double into(double a) const {
         if (mid && (mid_range(a) || is_zero(a))) {
-            const double e = a * r;
-            return fma(fma(-e, d, a), r, e);
+            const double e = a * r, x = fma(fma(-e, d, a), r, e);
+            return is_zero(a) ? e : x;
         }
         return a / d;
     }
