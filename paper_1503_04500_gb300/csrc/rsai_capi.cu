@@ -89,7 +89,11 @@ struct rsai_handle {
     double *pool_vals = nullptr;
     int64_t pool_cap = 0;
     unsigned long long *pool_top = nullptr;
-    // M
+    // entries that the columns of a first build reserved, once none is left for the
+    // global bin (-1: not known yet)
+    int64_t top_before_global = -1;
+    // M: room for pool_cap entries, so that whatever the columns find room for in the
+    // pool also fits M
     int64_t *Mcolptr = nullptr, *Mrowptr = nullptr, *Mcsc_to_csr = nullptr, *tsrc = nullptr;
     int32_t *Mrows = nullptr, *Mcols = nullptr, *row_count = nullptr, *cursor = nullptr, *tcols = nullptr;
     double *Mvals_csc = nullptr, *Mvals = nullptr, *tvals = nullptr;
@@ -359,20 +363,14 @@ cudaError_t enqueue_bins(rsai_handle *h, int mode, const DevA &A, const Frozen &
 
 // The build sequence: no allocation, no host synchronisation (capturable).
 // `ev` (optional, RSAI_PHASE_COUNT + 1 events) are recorded between phases.
-cudaError_t enqueue_build_tail(rsai_handle *h, cudaStream_t st, cudaEvent_t *ev);
-
-cudaError_t enqueue_build(rsai_handle *h, cudaStream_t st, cudaEvent_t *ev = nullptr, BinHook hook = nullptr) {
+cudaError_t enqueue_columns(rsai_handle *h, cudaStream_t st, cudaEvent_t *ev = nullptr, BinHook hook = nullptr) {
     const int64_t n = h->n;
     if (ev) cudaEventRecord(ev[0], st);
     cudaMemsetAsync(h->zeroed, 0, h->zeroed_bytes, st);
     k_norm1<<<blocks(n, 256), 256, 0, st>>>(h->col_ptr, h->cval, n, h->col_block, h->norm1_arr);
     if (h->cval32) k_to_f32<<<blocks(h->nnz, 256), 256, 0, st>>>(h->cval, h->cval32, h->nnz);
     k_tau_fixed<<<blocks(h->nblocks, 256), 256, 0, st>>>(h->norm1_arr, h->params.tol, h->tau_arr, h->nblocks);
-
-    cudaError_t e = enqueue_bins(h, MODE_BUILD, dev_a(h), Frozen{}, h->dscal + kCtr, st, ev, hook);
-    if (e != cudaSuccess) return e;
-    if (ev) cudaEventRecord(ev[4], st);
-    return enqueue_build_tail(h, st, ev);
+    return enqueue_bins(h, MODE_BUILD, dev_a(h), Frozen{}, h->dscal + kCtr, st, ev, hook);
 }
 
 // statistics and the assembly of M (the end of the build sequence)
@@ -395,6 +393,14 @@ cudaError_t enqueue_build_tail(rsai_handle *h, cudaStream_t st, cudaEvent_t *ev)
                                                      h->Mcsc_to_csr, n);
     if (ev) cudaEventRecord(ev[5], st);
     return cudaGetLastError();
+}
+
+// the whole build on the buffers of the first one (rebuild, phase times)
+cudaError_t enqueue_build(rsai_handle *h, cudaStream_t st, cudaEvent_t *ev = nullptr) {
+    const cudaError_t e = enqueue_columns(h, st, ev);
+    if (e != cudaSuccess) return e;
+    if (ev) cudaEventRecord(ev[4], st);
+    return enqueue_build_tail(h, st, ev);
 }
 
 void free_all(rsai_handle *h) {
@@ -622,7 +628,7 @@ constexpr int64_t kGlobalEntries = 256;
 
 // Before the global bin of a first build: one CTA per column that reached it, up
 // to one per SM (the slab, a few tens of MB per CTA, is sized by the first
-// build only), room for these columns in the result pool, and M's arrays.
+// build only), and room for these columns in the result pool.
 int size_global(rsai_handle *h, cudaStream_t st) {
     uint32_t cnt = 0;
     unsigned long long top = 0;
@@ -635,10 +641,7 @@ int size_global(rsai_handle *h, cudaStream_t st) {
         const int rc = grow_pool(h, room, (int64_t)top, st);
         if (rc != RSAI_OK) return rc;
     }
-    if (!h->Mrows) {
-        const int rc = alloc_m(h, h->pool_cap, st);
-        if (rc != RSAI_OK) return rc;
-    }
+    h->top_before_global = cnt == 0 ? (int64_t)top : -1;
     int want = std::max(1, std::min(h->sms, (int)std::min<uint32_t>(cnt, INT32_MAX)));
     if (h->tuning.global_bin_ctas > 0) want = std::min(h->tuning.global_bin_ctas, h->sms);
     // every SM helps the columns that are left at the end
@@ -743,46 +746,41 @@ int build_common(rsai_handle *h, cudaStream_t st) {
         h->pool_cap = cap;
         TRY(dalloc(h, &h->pool_rows, cap, st));
         TRY(dalloc(h, &h->pool_vals, cap, st));
-        TRY(cuda_status(enqueue_build(h, st, nullptr, size_global)));
+        TRY(cuda_status(enqueue_columns(h, st, nullptr, size_global)));
         int32_t *retry = nullptr;
         constexpr int kMaxRegrow = 6;
         bool settled = false;
         for (int attempt = 0; attempt <= kMaxRegrow; ++attempt) {
-            unsigned long long top = 0;
-            int32_t herr = 0;
-            unsigned long long both[2] = {0, 0};  // kErrWord, kTopWord
-            cudaMemcpyAsync(both, h->zeroed, sizeof(both), cudaMemcpyDeviceToHost, st);
-            TRY(cuda_status(cudaStreamSynchronize(st)));
-            memcpy(&herr, &both[kErrWord], sizeof(herr));
-            top = both[kTopWord];
-            if ((int64_t)top <= h->pool_cap) {
-                if (herr != 0) status = herr;
+            int64_t top = h->top_before_global;
+            if (top < 0) {
+                cudaMemcpyAsync(&top, h->pool_top, sizeof(top), cudaMemcpyDeviceToHost, st);
+                TRY(cuda_status(cudaStreamSynchronize(st)));
+            }
+            if (top <= h->pool_cap) {
                 settled = true;
                 break;
             }
             if (attempt == kMaxRegrow) break;  // the last rerun still found the pool full
-            // grow the pool (copying what fits), M's buffers with it
+            // grow the pool, keeping what fits
             const int64_t old_cap = h->pool_cap;
             // new reservations start at `top`; the columns to redo need at most `top`
-            cap = std::min<int64_t>((int64_t)(2 * top + 1024), std::max<int64_t>(n * n, (int64_t)top + 1024));
-            for (void *p : {(void *)h->Mrows, (void *)h->Mvals_csc, (void *)h->Mcols, (void *)h->Mvals, (void *)h->tcols,
-                            (void *)h->tvals, (void *)h->tsrc, (void *)h->Mcsc_to_csr})
-                dfree(h, p, st);
-            h->Mrows = nullptr;
+            cap = std::min<int64_t>(2 * top + 1024, std::max<int64_t>(n * n, top + 1024));
             TRY(grow_pool(h, cap, old_cap, st));
-            TRY(alloc_m(h, cap, st));
             // the columns that found the pool full run again (from its current top)
             if (!retry) TRY(dalloc(h, &retry, n, st));
             cudaMemsetAsync(h->qnext + kRerun, 0, sizeof(uint32_t), st);
             k_collect_failed<<<blocks(n, 256), 256, 0, st>>>(h->flags, n, retry, h->qnext + kRerun);
             cudaMemsetAsync(h->dscal + kCtr + CTR_FAILED, 0, sizeof(unsigned long long), st);
             cudaMemsetAsync(h->err, 0, sizeof(int32_t), st);
-            cudaMemsetAsync(h->row_count, 0, sizeof(int32_t) * 2 * (size_t)n, st);  // and cursor, which follows
-            cudaMemsetAsync(h->dscal + kCounts, 0, sizeof(unsigned long long) * 2, st);  // n_c, nnz(M): accumulated
             TRY(cuda_status(enqueue_bins(h, MODE_BUILD, dev_a(h), Frozen{}, h->dscal + kCtr, st, nullptr,
                                          size_global, retry, h->qnext + kRerun)));
-            TRY(cuda_status(enqueue_build_tail(h, st, nullptr)));
         }
+        TRY(alloc_m(h, h->pool_cap, st));
+        TRY(cuda_status(enqueue_build_tail(h, st, nullptr)));
+        int32_t herr = 0;
+        cudaMemcpyAsync(&herr, h->err, sizeof(herr), cudaMemcpyDeviceToHost, st);
+        TRY(cuda_status(cudaStreamSynchronize(st)));
+        if (herr != 0) status = herr;
         // columns still without room in the pool are flagged and counted as failed
         if (!settled) status = RSAI_ERR_WORKSPACE;
     }
