@@ -89,6 +89,7 @@ struct rsai_handle {
     double *pool_vals = nullptr;
     int64_t pool_cap = 0;
     unsigned long long *pool_top = nullptr;
+    int64_t room_cap = 0;  // most entries that the room for the global bin's columns makes it
     // entries that the columns of a first build reserved, once none is left for the
     // global bin (-1: not known yet)
     int64_t top_before_global = -1;
@@ -602,7 +603,7 @@ int alloc_m(rsai_handle *h, int64_t c, cudaStream_t st) {
 }
 
 // The result pool at `cap` entries, keeping the first `keep`
-int grow_pool(rsai_handle *h, int64_t cap, int64_t keep, cudaStream_t st) {
+int resize_pool(rsai_handle *h, int64_t cap, int64_t keep, cudaStream_t st) {
     int32_t *nrows = nullptr;
     double *nvals = nullptr;
     int rc = dalloc(h, &nrows, cap, st);
@@ -625,6 +626,11 @@ int grow_pool(rsai_handle *h, int64_t cap, int64_t keep, cudaStream_t st) {
 // the few others as unlucky and nothing else on the GPU: at n = 12000 the rerun
 // of 7 % of the columns took 120 of 495 ms.
 constexpr int64_t kGlobalEntries = 256;
+// The room stays within this many times the pool's first estimate.  With M's arrays
+// (52 bytes per entry to the pool's 12) still to come, the old and the new pool
+// then take no more (12 + 48 bytes per entry of the estimate) than pool and M did from the
+// start before there was any room (64), so no build that fitted runs out of memory for it.
+constexpr int64_t kRoomBound = 4;
 
 // Before the global bin of a first build: one CTA per column that reached it, up
 // to one per SM (the slab, a few tens of MB per CTA, is sized by the first
@@ -636,9 +642,9 @@ int size_global(rsai_handle *h, cudaStream_t st) {
         cudaMemcpyAsync(&top, h->pool_top, sizeof(top), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
         cudaStreamSynchronize(st) != cudaSuccess)
         return RSAI_ERR_CUDA;
-    const int64_t room = std::min<int64_t>((int64_t)top + (int64_t)cnt * kGlobalEntries, h->n * h->n);
+    const int64_t room = std::min<int64_t>({(int64_t)top + (int64_t)cnt * kGlobalEntries, h->n * h->n, h->room_cap});
     if (cnt > 0 && (int64_t)top <= h->pool_cap && room > h->pool_cap) {
-        const int rc = grow_pool(h, room, (int64_t)top, st);
+        const int rc = resize_pool(h, room, (int64_t)top, st);
         if (rc != RSAI_OK) return rc;
     }
     h->top_before_global = cnt == 0 ? (int64_t)top : -1;
@@ -744,12 +750,16 @@ int build_common(rsai_handle *h, cudaStream_t st) {
         const int64_t g_est = std::max<int64_t>(32, 10 * (nnz / std::max<int64_t>(1, n)) + 16);
         int64_t cap = std::min<int64_t>(n * g_est, n * n);
         h->pool_cap = cap;
+        h->room_cap = kRoomBound * cap;
         TRY(dalloc(h, &h->pool_rows, cap, st));
         TRY(dalloc(h, &h->pool_vals, cap, st));
         TRY(cuda_status(enqueue_columns(h, st, nullptr, size_global)));
         int32_t *retry = nullptr;
         constexpr int kMaxRegrow = 6;
         bool settled = false;
+        int64_t final_cap = cap;  // the pool's capacity for rebuilds
+        // room for a rerun, or for a rebuild, after `top` entries did not fit the estimate
+        auto doubled = [n](int64_t top) { return std::min<int64_t>(2 * top + 1024, std::max<int64_t>(n * n, top + 1024)); };
         for (int attempt = 0; attempt <= kMaxRegrow; ++attempt) {
             int64_t top = h->top_before_global;
             if (top < 0) {
@@ -758,14 +768,18 @@ int build_common(rsai_handle *h, cudaStream_t st) {
             }
             if (top <= h->pool_cap) {
                 settled = true;
+                if (!retry && top > cap) final_cap = doubled(top);
+                // the room that was not needed goes back
+                if (final_cap < h->pool_cap) TRY(resize_pool(h, final_cap, top, st));
                 break;
             }
             if (attempt == kMaxRegrow) break;  // the last rerun still found the pool full
             // grow the pool, keeping what fits
             const int64_t old_cap = h->pool_cap;
             // new reservations start at `top`; the columns to redo need at most `top`
-            cap = std::min<int64_t>(2 * top + 1024, std::max<int64_t>(n * n, top + 1024));
-            TRY(grow_pool(h, cap, old_cap, st));
+            final_cap = doubled(top);
+            TRY(resize_pool(h, final_cap, old_cap, st));
+            h->room_cap = final_cap;
             // the columns that found the pool full run again (from its current top)
             if (!retry) TRY(dalloc(h, &retry, n, st));
             cudaMemsetAsync(h->qnext + kRerun, 0, sizeof(uint32_t), st);
@@ -775,8 +789,15 @@ int build_common(rsai_handle *h, cudaStream_t st) {
             TRY(cuda_status(enqueue_bins(h, MODE_BUILD, dev_a(h), Frozen{}, h->dscal + kCtr, st, nullptr,
                                          size_global, retry, h->qnext + kRerun)));
         }
-        TRY(alloc_m(h, h->pool_cap, st));
+        TRY(alloc_m(h, final_cap, st));
         TRY(cuda_status(enqueue_build_tail(h, st, nullptr)));
+        if (final_cap > h->pool_cap) {  // its contents are in M by now
+            dfree(h, h->pool_rows, st);
+            dfree(h, h->pool_vals, st);
+            TRY(dalloc(h, &h->pool_rows, final_cap, st));
+            TRY(dalloc(h, &h->pool_vals, final_cap, st));
+            h->pool_cap = final_cap;
+        }
         int32_t herr = 0;
         cudaMemcpyAsync(&herr, h->err, sizeof(herr), cudaMemcpyDeviceToHost, st);
         TRY(cuda_status(cudaStreamSynchronize(st)));

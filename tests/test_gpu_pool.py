@@ -92,6 +92,42 @@ def test_columns_that_find_the_pool_full_run_again(problem, precision):
     fresh.free()
 
 
+class Requests(dict):
+    """What is outstanding, and the size of every request so far."""
+
+    def __init__(self):
+        super().__init__()
+        self.sizes = []
+
+    def __setitem__(self, ptr, nbytes):
+        self.sizes.append(nbytes)
+        super().__setitem__(ptr, nbytes)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32_refine"])
+@pytest.mark.parametrize("problem, kw, reruns", [
+    (lambda: gen.powerlaw(500, seed=3), dict(c=5, l_max=8, eps=0.4, drop="fixed"), False),  # fits the estimate
+    (lambda: gen.powerlaw(600, seed=5, dmax=40), dict(c=5, l_max=6, eps=0.05, drop="none"), False),  # does not
+    (long_columns, KW, True)])
+def test_room_for_the_global_bin_is_bounded_and_given_back(precision, problem, kw, reruns):
+    """Room for the global bin's columns is made (at most four times the estimate) and given
+    back: the handle keeps the estimate, or twice the entries that did not fit it."""
+    A = problem()
+    cap = first_estimate(A)
+    with FailingAllocator() as fa:
+        fa.live = Requests()
+        h = rsai.build(rsai.DeviceMatrix.from_host(A), precision=precision, **kw)
+        st = h.stats()
+        nnz, room = st["nnz_M"], st["cols_bin"][2] * 256
+        kept = capacity(fa, nnz)
+        if reruns:
+            assert 8 * 4 * cap in fa.live.sizes and kept >= min(2 * nnz + 1024, A.n**2)
+        else:
+            assert any(8 * max(cap, room) < b <= 8 * 4 * cap for b in fa.live.sizes)
+            assert kept == (cap if nnz <= cap else min(2 * nnz + 1024, max(A.n**2, nnz + 1024)))
+        h.free()
+
+
 @pytest.mark.parametrize("problem", [full_before_the_global_bin, long_columns])
 def test_every_failed_allocation_of_a_rerun_is_oom_and_leaks_nothing(problem):
     dA = rsai.DeviceMatrix.from_host(problem())
