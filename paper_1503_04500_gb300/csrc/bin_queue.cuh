@@ -35,6 +35,7 @@ __device__ void emit_or_forward(const Team &team, Column<Team, T, CapT> &col, in
         } else if (me == 0) {
             O.col_off[k] = 0;
             O.col_len[k] = 0;
+            O.col_q[k] = 0;
             O.rho[k] = NAN;
             O.loops[k] = 0;
             O.flags[k] = RSAI_COL_FAILED;
@@ -52,7 +53,9 @@ __device__ void emit_or_forward(const Team &team, Column<Team, T, CapT> &col, in
         if (me == 0) {
             O.col_off[k] = 0;
             O.col_len[k] = 0;
+            O.col_q[k] = 0;
             O.rho[k] = NAN;
+            O.loops[k] = 0;
             O.flags[k] = RSAI_COL_FAILED;
             w.ctr[CTR_FAILED] += 1;
             set_error(O.err, RSAI_ERR_WORKSPACE);
