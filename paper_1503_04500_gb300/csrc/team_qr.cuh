@@ -471,11 +471,12 @@ __device__ __noinline__ void apply_qt_team(Team team, const T *B, int q, int p, 
 // The reflectors j0..j1-1 (built on q0 rows) applied in order to the columns
 // p0..p-1 of B (ld q).  A warp takes its columns through all of them, so nothing
 // is synchronised until the end.
-template <class Team, typename T>
-__device__ __forceinline__ void update_reflectors(const Team &team, T *B, int q, int p, int q0, int p0,
-                                                  const T *vhead, const T *taus, int j0, int j1) {
+// M columns per warp at a time.
+template <int M, class Team, typename T>
+__device__ __forceinline__ void update_reflectors_m(const Team &team, T *B, int q, int p, int q0, int p0,
+                                                    const T *vhead, const T *taus, int j0, int j1) {
     const int lane = team.rank() & 31, wid = team.rank() >> 5;
-    constexpr int NW = Team::SIZE / 32, M = 2;
+    constexpr int NW = Team::SIZE / 32;
     for (int c = p0 + M * wid; c < p; c += M * NW) {
         for (int j = j0; j < j1; ++j) {
             const T two_over = taus[j];
@@ -487,6 +488,15 @@ __device__ __forceinline__ void update_reflectors(const Team &team, T *B, int q,
         }
     }
     team.sync();
+}
+// Two columns share the loads of a reflector, but are twice as long a chain: with at most one
+// column per warp (SPAI appends c at a time) one each (SPAI on the n = 20000 power law in FP64:
+// global bin 136 ms with two, 129 with one).
+template <class Team, typename T>
+__device__ __forceinline__ void update_reflectors(const Team &team, T *B, int q, int p, int q0, int p0,
+                                                  const T *vhead, const T *taus, int j0, int j1) {
+    if (p - p0 <= Team::SIZE / 32) update_reflectors_m<1>(team, B, q, p, q0, p0, vhead, taus, j0, j1);
+    else update_reflectors_m<2>(team, B, q, p, q0, p0, vhead, taus, j0, j1);
 }
 
 }  // namespace rsai
