@@ -5,10 +5,16 @@
 
 namespace rsai {
 
-// Four rows per 8 lanes
-__global__ void __launch_bounds__(256) k_spmv(int64_t n, CsrView A, const double *__restrict__ x, double *__restrict__ y) {
+// R rows per 8 lanes; 128 threads per CTA spread the groups with long rows better than 256
+constexpr int kSpmvThreads = 128;
+template <int R>
+__global__ void __launch_bounds__(kSpmvThreads)
+    k_spmv(int64_t n, CsrView A, const double *__restrict__ x, double *__restrict__ y) {
     const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    spmv_rows(A, x, y, (g >> 3) * kRowsPerGroup, n, threadIdx.x & 7);
+    const int sub = threadIdx.x & 7;
+    const int64_t row0 = (g >> 3) * R;
+    if constexpr (R == 1) spmv_row<2>(A, x, y, row0, row0 < n, sub);
+    else spmv_long_rows<R>(A, x, y, row0, spmv_short_rows<R>(A, x, y, row0, n, sub), sub);
 }
 
 // gval[e] = gy[i] x[col(e)] for every stored entry e of row i: the gradient
@@ -34,11 +40,16 @@ cudaError_t launch_spmv_grad_values(int64_t n, const int64_t *row_ptr, const int
     return cudaGetLastError();
 }
 
-cudaError_t launch_spmv(int64_t n, const int64_t *row_ptr, const int32_t *col_idx, const double *val,
+cudaError_t launch_spmv(int64_t n, int64_t nnz, const int64_t *row_ptr, const int32_t *col_idx, const double *val,
                         const double *x, double *y, cudaStream_t st) {
     if (n == 0) return cudaSuccess;
-    const int64_t groups = (n + kRowsPerGroup - 1) / kRowsPerGroup;
-    k_spmv<<<(unsigned)((groups * 8 + 255) / 256), 256, 0, st>>>(n, CsrView{row_ptr, col_idx, val}, x, y);
+    const int R = spmv_rows_per_group(n, nnz);
+    const int64_t groups = (n + R - 1) / R;
+    const unsigned grid = (unsigned)((groups * 8 + kSpmvThreads - 1) / kSpmvThreads);
+    const CsrView A{row_ptr, col_idx, val};
+    if (R == 1) k_spmv<1><<<grid, kSpmvThreads, 0, st>>>(n, A, x, y);
+    else if (R == 2) k_spmv<2><<<grid, kSpmvThreads, 0, st>>>(n, A, x, y);
+    else k_spmv<4><<<grid, kSpmvThreads, 0, st>>>(n, A, x, y);
     return cudaGetLastError();
 }
 

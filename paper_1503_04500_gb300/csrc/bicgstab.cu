@@ -48,6 +48,7 @@ struct Solve {
     int64_t n;
     int vblocks;  // virtual blocks that hold rows
     CsrView A, M;
+    bool long_A, long_M;  // rows of kLongAverage entries and more on the average
     const double *b;
     double *x;
     double *r, *rhat, *p, *v, *s, *t, *y, *tmp, *tmp2, *partials;
@@ -83,23 +84,34 @@ __device__ bool grid_sync(Control *ctl, unsigned &epoch) {
     return ok_sh != 0;
 }
 
-// rows that a block takes at a time (kRowsPerGroup per 8 lanes)
-constexpr int kBlockRows = kThreads / 8 * kRowsPerGroup;
-static_assert(kBlockRows == kDotThreads, "one round of a virtual block is one pass of a block");
+// y[r0 .. end) = (A x) of these rows by one block, four rows per 8 lanes, or one where rows are long
+constexpr int kGroups = kThreads / 8;
+static_assert(kGroups * 4 == kDotThreads, "one round of a virtual block is one pass of a block");
+__device__ __forceinline__ void block_rows(const CsrView &A, bool is_long, const double *x, double *y, int64_t r0,
+                                           int64_t end) {
+    const int g = threadIdx.x >> 3, sub = threadIdx.x & 7;
+    if (is_long) {
+        for (; r0 < end; r0 += kGroups) spmv_row<2>(A, x, y, r0 + g, r0 + g < end, sub);
+    } else {
+        unsigned any = 0;  // long rows (none of a stencil) in a second pass: the loop stays short
+        for (int64_t r = r0; r < end; r += kGroups * 4) any |= spmv_short_rows<4>(A, x, y, r + g * 4, end, sub);
+        if (__any_sync(0xffffffffu, any != 0u))
+            for (; r0 < end; r0 += kGroups * 4)
+                spmv_long_rows<4>(A, x, y, r0 + g * 4, long_rows<4>(A, r0 + g * 4, end), sub);
+    }
+}
 
 // y = A x, an even share of the rows per block
-__device__ void product(const CsrView &A, int64_t n, const double *x, double *y) {
-    const int64_t share = ((n + gridDim.x - 1) / gridDim.x + kRowsPerGroup - 1) / kRowsPerGroup * kRowsPerGroup;
-    const int64_t end = min(n, (blockIdx.x + 1) * share);
-    for (int64_t r0 = blockIdx.x * share; r0 < end; r0 += kBlockRows)
-        spmv_rows(A, x, y, r0 + (threadIdx.x >> 3) * kRowsPerGroup, end, threadIdx.x & 7);
+__device__ void product(const CsrView &A, bool is_long, int64_t n, const double *x, double *y) {
+    const int64_t share = ((n + gridDim.x - 1) / gridDim.x + 3) / 4 * 4;
+    block_rows(A, is_long, x, y, blockIdx.x * share, min(n, (blockIdx.x + 1) * share));
 }
 
 // y = A x on the rows that this block owns
-__device__ void product_own(const Solve &S, const CsrView &A, const double *x, double *y) {
+__device__ void product_own(const Solve &S, const double *x, double *y) {
     for (int vb = blockIdx.x; vb < S.vblocks; vb += gridDim.x)
         for (int64_t r0 = (int64_t)vb * kDotThreads; r0 < S.n; r0 += kRound)
-            spmv_rows(A, x, y, r0 + (threadIdx.x >> 3) * kRowsPerGroup, S.n, threadIdx.x & 7);
+            block_rows(S.A, S.long_A, x, y, r0, min(S.n, r0 + kDotThreads));
     __syncthreads();
 }
 
@@ -245,11 +257,11 @@ __global__ void __launch_bounds__(kThreads, 2) k_bicgstab(Solve S) {
         const double *Mp = S.p;
         RSAI_SYNC();
         if (prec) {
-            product(S.M, n, S.p, S.tmp);
+            product(S.M, S.long_M, n, S.p, S.tmp);
             Mp = S.tmp;
             RSAI_SYNC();
         }
-        product_own(S, S.A, Mp, S.v);
+        product_own(S, Mp, S.v);
         chains<1>(S, sh, {D_RV}, [&](int64_t i, double (&a)[1], double (&c)[1]) {
             a[0] = S.rhat[i];
             c[0] = S.v[i];
@@ -273,11 +285,11 @@ __global__ void __launch_bounds__(kThreads, 2) k_bicgstab(Solve S) {
         }
         const double *Ms = S.s;
         if (prec) {
-            product(S.M, n, S.s, S.tmp);
+            product(S.M, S.long_M, n, S.s, S.tmp);
             Ms = S.tmp;
             RSAI_SYNC();
         }
-        product_own(S, S.A, Ms, S.t);
+        product_own(S, Ms, S.t);
         chains<2>(S, sh, {D_TS, D_TT}, [&](int64_t i, double (&a)[2], double (&c)[2]) {
             a[0] = a[1] = c[1] = S.t[i];
             c[0] = S.s[i];
@@ -303,10 +315,10 @@ __global__ void __launch_bounds__(kThreads, 2) k_bicgstab(Solve S) {
     if (it > S.maxit) it = S.maxit;
     // x = M y, true residual
     RSAI_SYNC();
-    if (prec) product(S.M, n, S.y, S.x);
+    if (prec) product(S.M, S.long_M, n, S.y, S.x);
     else own_elements(S, [&](int64_t i) { S.x[i] = S.y[i]; });
     RSAI_SYNC();
-    product_own(S, S.A, S.x, S.tmp2);
+    product_own(S, S.x, S.tmp2);
     chains<1>(S, sh, {D_RV}, [&](int64_t i, double (&a)[1], double (&c)[1]) { a[0] = c[0] = S.b[i] - S.tmp2[i]; });
     RSAI_SYNC();
     const double res = grid_total(P + D_RV * kDotBlocks, sh);
@@ -324,8 +336,8 @@ size_t bicgstab_workspace_bytes(int64_t n) {
     return sizeof(double) * ((size_t)(n > 0 ? n : 1) * 9 + (size_t)D_COUNT * kDotBlocks + kControlWords);
 }
 
-int bicgstab_run(int64_t n, const int64_t *Arp, const int32_t *Aci, const double *Av, const int64_t *Mrp,
-                 const int32_t *Mci, const double *Mv, const double *b, double *x, double rtol, int maxit,
+int bicgstab_run(int64_t n, int64_t nnzA, const int64_t *Arp, const int32_t *Aci, const double *Av, int64_t nnzM,
+                 const int64_t *Mrp, const int32_t *Mci, const double *Mv, const double *b, double *x, double rtol, int maxit,
                  int *iters, double *relres, cudaStream_t st, double *work) {
     double *buf = work;
     const bool own = work == nullptr;  // else the caller's workspace of bicgstab_workspace_bytes(n)
@@ -336,6 +348,8 @@ int bicgstab_run(int64_t n, const int64_t *Arp, const int32_t *Aci, const double
     S.vblocks = (int)std::min<int64_t>(kDotBlocks, (n + kDotThreads - 1) / kDotThreads);
     S.A = CsrView{Arp, Aci, Av};
     S.M = CsrView{Mrp, Mci, Mv};
+    S.long_A = nnzA / n >= kLongAverage;
+    S.long_M = Mrp && nnzM / n >= kLongAverage;
     S.b = b;
     S.x = x;
     double *q = buf;
@@ -354,7 +368,10 @@ int bicgstab_run(int64_t n, const int64_t *Arp, const int32_t *Aci, const double
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_bicgstab, kThreads, 0) != cudaSuccess || occ < 1)
             return false;
-        const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(S.vblocks, (int64_t)occ * sms));
+        // a block per virtual block or, where M's rows are long, one per 64 rows of it (a pass of its
+        // groups): blocks beyond the virtual ones take part in M's products only
+        const int64_t want = std::max<int64_t>(S.vblocks, S.long_M ? (n + kGroups - 1) / kGroups : 1);
+        const int grid = (int)std::max<int64_t>(1, std::min<int64_t>({want, kDotBlocks, (int64_t)occ * sms}));
         // partial sums of virtual blocks without rows, and the control block
         if (cudaMemsetAsync(S.partials, 0, sizeof(double) * ((size_t)D_COUNT * kDotBlocks + kControlWords), st) !=
             cudaSuccess)

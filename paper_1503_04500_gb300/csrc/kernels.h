@@ -98,14 +98,15 @@ int occupancy_bin_half(bool fp32, int warps, const Caps &cap);
 int occupancy_bin_block(bool fp32, int kind, const Caps &cap);
 
 // apply / solver kernels (apply_kernels.cu)
-cudaError_t launch_spmv(int64_t n, const int64_t *row_ptr, const int32_t *col_idx, const double *val,
+// (nnz: the entries, or about as many; only the split of the rows depends on it)
+cudaError_t launch_spmv(int64_t n, int64_t nnz, const int64_t *row_ptr, const int32_t *col_idx, const double *val,
                         const double *x, double *y, cudaStream_t st);
 // gval[e] = gy[row(e)] * x[col(e)] over the stored entries of a CSR matrix
 cudaError_t launch_spmv_grad_values(int64_t n, const int64_t *row_ptr, const int32_t *col_idx, const double *gy,
                                     const double *x, double *gval, cudaStream_t st);
 // right-preconditioned BiCGStab (bicgstab.cu)
-int bicgstab_run(int64_t n, const int64_t *Arp, const int32_t *Aci, const double *Av, const int64_t *Mrp,
-                 const int32_t *Mci, const double *Mv, const double *b, double *x, double rtol, int maxit,
+int bicgstab_run(int64_t n, int64_t nnzA, const int64_t *Arp, const int32_t *Aci, const double *Av, int64_t nnzM,
+                 const int64_t *Mrp, const int32_t *Mci, const double *Mv, const double *b, double *x, double rtol, int maxit,
                  int *iters, double *relres, cudaStream_t st, double *work = nullptr);
 // device bytes bicgstab_run needs as its workspace for size n
 size_t bicgstab_workspace_bytes(int64_t n);

@@ -92,7 +92,7 @@ extern "C" rsai_status rsai_bicgstab_noalloc(const rsai_csr *A, const rsai_csr *
     if (rc != RSAI_OK) return (rsai_status)rc;
     int it = 0;
     double rr = 0.0;
-    const int status = bicgstab_run(A->n, A->row_ptr, A->col_idx, A->val, M ? M->row_ptr : nullptr,
+    const int status = bicgstab_run(A->n, A->nnz, A->row_ptr, A->col_idx, A->val, M ? M->nnz : 0, M ? M->row_ptr : nullptr,
                                     M ? M->col_idx : nullptr, M ? M->val : nullptr, b, x, rtol, maxit, &it, &rr,
                                     (cudaStream_t)stream, work);
     *iters = it;

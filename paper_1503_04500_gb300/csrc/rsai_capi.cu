@@ -89,6 +89,7 @@ struct rsai_handle {
     double *pool_vals = nullptr;
     int64_t pool_cap = 0;
     unsigned long long *pool_top = nullptr;
+    int64_t entries_M = 0;  // that the first build reserved: about nnz(M), for the split of its products
     int64_t room_cap = 0;  // most entries that the room for the global bin's columns makes it
     // entries that the columns of a first build reserved, once none is left for the
     // global bin (-1: not known yet)
@@ -766,6 +767,7 @@ int build_common(rsai_handle *h, cudaStream_t st) {
                 cudaMemcpyAsync(&top, h->pool_top, sizeof(top), cudaMemcpyDeviceToHost, st);
                 TRY(cuda_status(cudaStreamSynchronize(st)));
             }
+            h->entries_M = top;
             if (top <= h->pool_cap) {
                 settled = true;
                 if (!retry && top > cap) final_cap = doubled(top);
@@ -1105,7 +1107,7 @@ rsai_status rsai_spmv(const rsai_csr *A, const double *x, double *y, void *strea
     if (rc != RSAI_OK) return (rsai_status)rc;
     if (!x || !y) return RSAI_ERR_INVALID_ARG;
     if (!have_device()) return RSAI_ERR_NO_DEVICE;
-    return (rsai_status)cuda_status(launch_spmv(A->n, A->row_ptr, A->col_idx, A->val, x, y, (cudaStream_t)stream));
+    return (rsai_status)cuda_status(launch_spmv(A->n, A->nnz, A->row_ptr, A->col_idx, A->val, x, y, (cudaStream_t)stream));
 }
 
 rsai_status rsai_spmv_grad_values(const rsai_csr *A, const double *gy, const double *x, double *gval, void *stream) {
@@ -1136,7 +1138,7 @@ rsai_status rsai_set_allocator(rsai_alloc_fn alloc, rsai_free_fn release, void *
 rsai_status rsai_apply(rsai_handle *h, const double *x, double *y, void *stream) {
     if (!h || !x || !y) return RSAI_ERR_INVALID_ARG;
     return (rsai_status)cuda_status(
-        launch_spmv(h->n, h->Mrowptr, h->Mcols, h->Mvals, x, y, (cudaStream_t)stream));
+        launch_spmv(h->n, h->entries_M, h->Mrowptr, h->Mcols, h->Mvals, x, y, (cudaStream_t)stream));
 }
 
 rsai_status rsai_bicgstab(const rsai_csr *A, rsai_handle *M, const double *b, double *x, double rtol, int32_t maxit,
@@ -1157,8 +1159,8 @@ rsai_status rsai_bicgstab(const rsai_csr *A, rsai_handle *M, const double *b, do
         work = (double *)raw_alloc(a, wb, st);
         if (!work) return RSAI_ERR_OOM;
     }
-    rc = bicgstab_run(A->n, A->row_ptr, A->col_idx, A->val, M ? M->Mrowptr : nullptr, M ? M->Mcols : nullptr,
-                      M ? M->Mvals : nullptr, b, x, rtol, maxit, &it, &rr, st, work);
+    rc = bicgstab_run(A->n, A->nnz, A->row_ptr, A->col_idx, A->val, M ? M->entries_M : 0, M ? M->Mrowptr : nullptr,
+                      M ? M->Mcols : nullptr, M ? M->Mvals : nullptr, b, x, rtol, maxit, &it, &rr, st, work);
     if (work) raw_free(a, work, wb, st);
     *iters = it;
     *relres = rr;
