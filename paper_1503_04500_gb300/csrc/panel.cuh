@@ -389,8 +389,10 @@ constexpr int kAhead = 6;
 // overlap the arithmetic.  In FP32 the products go two at a time: W pairs
 // two reflectors per column, the update pairs two columns.
 // A panel of fewer columns (all that fit the staging area of a column of thousands of
-// rows) skips the chunks past its last: multiplied as zeros they were three quarters of
-// the FP64 work of a panel of four (|I| up to 5710: global bin 2387 -> 1686 ms).
+// rows) skips in FP64 the chunks past its last: multiplied as zeros they were three quarters
+// of the FP64 work of a panel of four (|I| up to 5710: global bin 2387 -> 1686 ms).  In FP32,
+// where most such panels are the last ones of short factors, the tests cost more than the
+// products (n = 5000 power law, rebuild 132.7 ms without, 135.6 with them).
 template <int KC, int D, bool FULL, typename T>
 __device__ __forceinline__ void wy_apply_cols(const T *V, int qq, int nb, const T *tm, T *const (&tc)[KC],
                                               const bool (&has)[KC], int lane) {
@@ -460,7 +462,6 @@ __device__ __forceinline__ void wy_apply_cols(const T *V, int qq, int nb, const 
                     for (int x = 0; x < KC; ++x) cc[x] = pack2(cur[x], cur[x]);
 #pragma unroll
                     for (int c = 0; c < NC; ++c) {
-                        if (!FULL && c * CW >= nb) break;
                         const Chunk<T> v = panel_chunk<FULL>(V, qq, nb, r, c);
                         const f32x2 v01 = pack2(v.v[0], v.v[1]), v23 = pack2(v.v[2], v.v[3]);
 #pragma unroll
@@ -538,7 +539,6 @@ __device__ __forceinline__ void wy_apply_cols(const T *V, int qq, int nb, const 
                    for (int g = 0; g < KC / 2; ++g) a2[g] = pack2(cur[2 * g], cur[2 * g + 1]);
 #pragma unroll
                    for (int c = 0; c < NC; ++c) {
-                       if (!FULL && c * CW >= nb) break;
                        const Chunk<T> v = panel_chunk<FULL>(V, qq, nb, r, c);
 #pragma unroll
                        for (int k = 0; k < CW; ++k) {
@@ -552,7 +552,7 @@ __device__ __forceinline__ void wy_apply_cols(const T *V, int qq, int nb, const 
                } else {
 #pragma unroll
                    for (int c = 0; c < NC; ++c) {
-                       if (!FULL && c * CW >= nb) break;
+                       if (!FULL && !F32 && c * CW >= nb) break;
                        const Chunk<T> v = panel_chunk<FULL>(V, qq, nb, r, c);
 #pragma unroll
                        for (int k = 0; k < CW; ++k)
