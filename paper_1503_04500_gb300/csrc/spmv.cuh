@@ -70,15 +70,16 @@ __device__ __forceinline__ void spmv_row(const CsrView &A, const double *x, doub
 // of the warp calls.  For every R: lane sub of a row adds entries sub, sub + 8, ... in
 // order and a butterfly over 4, 2, 1 joins the lanes, so all of them give the same bits.
 //
-// R > 1 rows of at most kShortRow entries go side by side: their loads, and those of the next
-// round of 8 entries, are in flight together, and the butterflies are one reduce-scatter (4 additions per lane for four rows instead of
-// 12, the same sums): on this GPU's FP64 unit (2 lanes per cycle and SM) the additions
-// of one butterfly per row took longer than the products of a row of 16 entries.
+// R > 1 rows of at most kShortRow entries go side by side: their loads (AHEAD: and those of
+// the next round of 8 entries) are in flight together, and the butterflies are one
+// reduce-scatter (4 additions per lane for four rows instead of 12, the same sums): on
+// this GPU's FP64 unit (2 lanes per cycle and SM) the additions of one butterfly per
+// row took longer than the products of a row of 16 entries.
 // A longer row would hold the others' lanes up; spmv_short_rows leaves it and sets its bit in
 // the mask that it returns, and spmv_long_rows takes the warp's long rows one per group (with all
 // rows side by side M of a power law, 60000 rows of 69 entries, took 39 us instead of the 28
 // of a row per group, and 100000 rows of 9 entries, a few of 200, 26 instead of 16).
-template <int R>
+template <int R, bool AHEAD = true>
 __device__ __forceinline__ unsigned spmv_short_rows(const CsrView &A, const double *x, double *y, int64_t row0,
                                                     int64_t end, int sub) {
     static_assert(R == 2 || R == 4, "the exchanges below");
@@ -102,28 +103,40 @@ __device__ __forceinline__ unsigned spmv_short_rows(const CsrView &A, const doub
     double acc[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) acc[r] = 0.0;
-    int32_t c[R];
-    double v[R];
-    auto load = [&](int e, int32_t (&cn)[R], double (&vn)[R]) {
+    auto load = [&](int e, int32_t (&c)[R], double (&v)[R]) {
 #pragma unroll
         for (int r = 0; r < R; ++r) {
-            cn[r] = e < len[r] ? A.col_idx[at[r] + e] : -1;
-            vn[r] = e < len[r] ? A.val[at[r] + e] : 0.0;
+            c[r] = e < len[r] ? A.col_idx[at[r] + e] : -1;
+            v[r] = e < len[r] ? A.val[at[r] + e] : 0.0;
         }
     };
-    load(sub, c, v);
-    for (int e = sub; e < most;) {
-        e += 8;
-        int32_t cn[R];
-        double vn[R];
-        load(e, cn, vn);
+    auto add = [&](const int32_t (&c)[R], const double (&v)[R]) {
 #pragma unroll
         for (int r = 0; r < R; ++r)
             if (c[r] >= 0) acc[r] = fma(v[r], x[c[r]], acc[r]);
+    };
+    if constexpr (AHEAD) {
+        int32_t c[R];
+        double v[R];
+        load(sub, c, v);
+        for (int e = sub; e < most;) {
+            e += 8;
+            int32_t cn[R];
+            double vn[R];
+            load(e, cn, vn);
+            add(c, v);
 #pragma unroll
-        for (int r = 0; r < R; ++r) {
-            c[r] = cn[r];
-            v[r] = vn[r];
+            for (int r = 0; r < R; ++r) {
+                c[r] = cn[r];
+                v[r] = vn[r];
+            }
+        }
+    } else {
+        for (int e = sub; e < most; e += 8) {
+            int32_t c[R];
+            double v[R];
+            load(e, c, v);
+            add(c, v);
         }
     }
     const bool hi = sub & 4, mid = sub & 2;
@@ -156,19 +169,6 @@ __device__ __forceinline__ void spmv_long_rows(const CsrView &A, const double *x
         spmv_row<4>(A, x, y, first + R * (bit >> 3) + (bit & 7), w != 0u, sub);
         for (int g = 0; g < 4; ++g) left &= left - 1u;
     }
-}
-
-// Bit r: row0 + r is a long row
-template <int R> __device__ __forceinline__ unsigned long_rows(const CsrView &A, int64_t row0, int64_t end) {
-    unsigned is_long = 0;
-    int64_t a = row0 < end ? A.row_ptr[row0] : 0;
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-        const int64_t b = row0 + r < end ? A.row_ptr[row0 + r + 1] : a;
-        is_long |= (b - a > kShortRow ? 1u : 0u) << r;
-        a = b;
-    }
-    return is_long;
 }
 
 // Rows per group for n rows with nnz entries: one where rows are long on the average (rows
