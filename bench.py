@@ -35,9 +35,9 @@ sys.path.insert(0, ROOT)
 PARAMS = dict(c=3, l_max=10, eps=0.3, tol=1e-3, drop="fixed")
 METRIC = "RSAI M-columns/sec at matched ||AM-I||_F, FP32+refine vs FP64; bwd/fwd ratio"
 WORKLOAD = "convdiff3d_7pt_upwind_64^3_Pe5"
-# norm1, tau, 4 bins (W, W2, C, G), 3 kernels ordering the global bin's queue, 2 column-stats kernels,
-# 2 x 3 scan kernels, pool->CSC, CSC->rows, row sort
-KERNELS_PER_BUILD = 20
+# norm1, tau, the FP32 copy of A's values, 7 bins (H or W0, then W, W2, S0, S, C, G), 3 kernels ordering the
+# global bin's queue, 2 column-stats kernels, 2 x 2 scan kernels, pool->CSC, CSC->rows, row sort
+KERNELS_PER_BUILD = 22
 # GB300's published FP64 rate (a side field; the roofline divides by the measured FMA-chain rate)
 PEAK_FP64_PUBLISHED = 1.25e12
 # copy bandwidth measured on this GPU type, used only when MEASURED_PEAKS.json is absent
@@ -600,9 +600,7 @@ def main():
         "tuning": {"fp32_refine": tuned32["tuning"], "fp64": tuned64["tuning"]},
         "parametric2d_256": c4, "powerlaw_1e6": c3, "batch": c5, "rsai_vs_spai": spai_cmp,
         "cpu_baseline": cpu, "e2e": e2e, "clocks": clocks,
-        # the half-warp bin adds one launch when the tuned shape uses it
-        # (+1: the FP32 copy of A's values that an FP32+refine build makes)
-        "gpu_launches": (KERNELS_PER_BUILD + 1 + int(tuned32["tuning"].get("half_bin", 0))) * args.steps,
+        "gpu_launches": KERNELS_PER_BUILD * args.steps,
         "wall_s_timed_region": t_wall,
     }
     if rank == 0:
