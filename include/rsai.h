@@ -172,6 +172,10 @@ rsai_status rsai_params_check(const rsai_params *p);
  *              frozen pattern, ||r_k|| and the per-column flags.
  * Validates A (shape, sorted, index range, no empty column) on the device
  * before building.  The call returns when M and its statistics are ready.
+ * Columns that reach the global bin (matrices with dense rows) take every SM, in this and
+ * in every later pass over them (rsai_rebuild, rsai_refit, rsai_backward): CTAs without a
+ * column left stay, with their shared memory, to help the others until the last column is
+ * done, so kernels of other streams get no SM before that (rsai_tuning.global_bin_ctas).
  * Errors: INVALID_ARG, SHAPE, UNSORTED, INDEX_RANGE, EMPTY_COLUMN, OOM, CUDA,
  * WORKSPACE (a column outgrew every bin: the handle is still returned with
  * those columns flagged RSAI_COL_FAILED).
@@ -305,8 +309,8 @@ rsai_status rsai_build_phase_times(rsai_handle *h, void *stream, double *ms);
  * It allocates nothing: its work vectors live in one fixed device array inside
  * the library (about 4.7 MB, held by every GPU that loads the library until the
  * process exits) and n must not exceed 65536 (else RSAI_ERR_TOO_LARGE).  Like
- * rsai_bicgstab it waits for the stream at every iteration to read the scalars
- * of its stopping test, so it cannot be captured into a CUDA graph.  The first
+ * rsai_bicgstab it waits for the stream once, when the solve has ended, to read
+ * its status, iterations and residual, so it cannot be captured into a CUDA graph.  The first
  * call on each device looks up the array's device address (and keeps it); make
  * that first call while no stream of the process is being captured.  After a
  * cudaDeviceReset of a device the kept address is stale, so do not call it on

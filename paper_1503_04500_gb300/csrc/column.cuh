@@ -165,9 +165,6 @@ template <typename T> struct Work {
 // COL_OVERFLOW_J: |J| outgrew the bin (a bin with the same |J| limit cannot take the column either)
 enum ColStatus { COL_DONE = 0, COL_OVERFLOW = 1, COL_OVERFLOW_J = 2 };
 
-// Entries of a CSR row loaded together in the row-driven loops
-constexpr int kRowGroup = 4;
-
 // Rows per lane of the register QR: q <= 64 on a warp, q <= 48 on half a warp
 template <class Team> constexpr int kRegRows = Team::SIZE == 16 ? 3 : 2;
 
@@ -570,36 +567,36 @@ template <class Team, typename T, class CapT = Caps> struct Column {
     __device__ __forceinline__ double row_dot(int64_t e0, int len, const double *v, const StageMap &map,
                                               const int32_t *Js, int &cnt) const {
         const int sub = team.rank() & 7;
-                    double acc[4] = {0.0, 0.0, 0.0, 0.0};
-                    int most = len;
-        #pragma unroll
-                    for (int o = 16; o >= 8; o >>= 1) most = max(most, __shfl_xor_sync(0xffffffffu, most, o));
-                    for (int b = 0; b < most; b += 32) {
-        #pragma unroll
-                        for (int h = 0; h < 4; ++h) {
-                            if (b + 8 * h >= most) break;  // the same for the whole warp
-                            const int e = b + 8 * h + sub;
-                            if (e < len) {
-                                const int32_t col = A.col_idx[e0 + e];
-                                int pos;
-                                if (Team::STAGED && map.on()) pos = map.find(col);
-                                else pos = find_i32(Js, p, col);
-                                if (pos >= 0) {
-                                    acc[h] = fma(A.val[e0 + e], v[pos], acc[h]);
-                                    ++cnt;
-                                }
-                            }
-                        }
+        double acc[4] = {0.0, 0.0, 0.0, 0.0};
+        int most = len;
+#pragma unroll
+        for (int o = 16; o >= 8; o >>= 1) most = max(most, __shfl_xor_sync(0xffffffffu, most, o));
+        for (int b = 0; b < most; b += 32) {
+#pragma unroll
+            for (int h = 0; h < 4; ++h) {
+                if (b + 8 * h >= most) break;  // the same for the whole warp
+                const int e = b + 8 * h + sub;
+                if (e < len) {
+                    const int32_t col = A.col_idx[e0 + e];
+                    int pos;
+                    if (Team::STAGED && map.on()) pos = map.find(col);
+                    else pos = find_i32(Js, p, col);
+                    if (pos >= 0) {
+                        acc[h] = fma(A.val[e0 + e], v[pos], acc[h]);
+                        ++cnt;
                     }
-                    double x = acc[0];
-                    if (most > 16) {
-                        x += acc[2];
-                        x += acc[1] + acc[3];
-                    } else if (most > 8) {
-                        x += acc[1];
-                    }
-        #pragma unroll
-                    for (int o = 4; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+                }
+            }
+        }
+        double x = acc[0];
+        if (most > 16) {
+            x += acc[2];
+            x += acc[1] + acc[3];
+        } else if (most > 8) {
+            x += acc[1];
+        }
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
         return x;
     }
 

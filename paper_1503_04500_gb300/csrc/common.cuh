@@ -250,7 +250,9 @@ struct WarpTeam {
 // Every CTA size gives the same bits: in the smaller CTAs (at most 128 rows, at
 // most NT columns) a float reduction is over one element per thread of a CTA of
 // 128, the same per-warp butterflies added over the warps in order; the absent
-// warps would add zeros.
+// warps would add zeros.  (But for ||a_k||^2 of the first solve, J = {k}, where a thread of a
+// CTA of 64 adds its two rows first: it decides the first dominant rows only, since a column
+// that comes to these bins solves again on a wider J.)
 constexpr int kVirtualWarps = 16;
 template <int NT, bool STAGED_ = false> struct BlockTeam {
     static constexpr int SIZE = NT;

@@ -6,13 +6,15 @@
 
 namespace rsai {
 
-// NT threads per column.  STAGED: the workspace is a global-memory slab per CTA
-// (gwork) and shared memory stages the panels; else it is in shared memory.
-// MINB: CTAs per SM that the register budget has to allow.
-// The sizes of bins S0 and S (plan_bins fills the same numbers into Caps when c * l_max <= 64)
+// The sizes of bins S0 and S (plan_bins fills the same numbers into Caps when c * l_max <= 64;
+// above, R is larger and the layout is the runtime one: 200^2 at eps = 0.12, CTA bins in
+// FP32 108.9 ms with c * l_max = 64, 112.8 with 66, in FP64 232 both)
 using CapsS0 = FixedCaps<96, 40, 256, 64, 128, 1>;
 using CapsS = FixedCaps<128, 64, 512, 64, 256, 1>;
 
+// NT threads per column.  STAGED: the workspace is a global-memory slab per CTA
+// (gwork) and shared memory stages the panels; else it is in shared memory.
+// MINB: CTAs per SM that the register budget has to allow.
 template <typename T, int NT, bool STAGED, int MINB, int MODE, class CapT>
 __global__ void __launch_bounds__(NT, MINB)
     k_bin_block(DevA A, DevParams P, CapT cap, ColQueue Q, ColOut O, Frozen F, unsigned long long *gctr,

@@ -52,12 +52,12 @@ struct rsai_handle {
     int32_t *col_idx = nullptr, *row_idx = nullptr;
     double *val = nullptr, *cval = nullptr;
     float *cval32 = nullptr;  // FP32 copy of cval (FP32_REFINE builds), refreshed by every build
-    // 8-byte words: (unused), (unused), frob2, counters, column counts, partial sums
     // One buffer that every build zeroes: the error word, the result pool's top,
     // ||A||_1 per block, the scalar block and the rows' counters (`zeroed_bytes`); the words before
     // the scalar block's statistics are read back together (rsai_get_stats).
     unsigned long long *zeroed = nullptr;
     size_t zeroed_bytes = 0;
+    // 8-byte words: (unused), (unused), frob2, counters, column counts, partial sums
     unsigned long long *dscal = nullptr;
     // blocks (a batch of independent matrices as one block-diagonal matrix)
     int32_t nblocks = 1;
@@ -819,9 +819,11 @@ rsai_handle *new_handle(const rsai_params *params, cudaStream_t st) {
     cudaGetDevice(&h->device);
     cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, h->device);
     h->params = *params;
-    // the shapes the autotuner picks on the 64^3 convection-diffusion problem:
-    // FP64 builds start in the half-warp bin with the register QR up to
-    // |J| = 8, FP32+refine builds in the warp bin with the register QR up to 16
+    // FP64 builds start in the half-warp bin with the register QR up to |J| = 8, FP32+refine
+    // builds in the warp bin (W0) with the register QR up to 16.  On the 64^3 convection-diffusion
+    // problem the autotuner now picks other shapes (half a warp per column in FP32, 2.4 against
+    // 3.3 ms in the first bin; no register QR in FP64); their sums have another order, so
+    // the defaults stay.
     if (params->precision == RSAI_FP64) {
         h->tuning.half_bin = 1;
         h->tuning.small_qr_max_p = 8;

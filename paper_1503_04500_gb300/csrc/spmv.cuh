@@ -174,7 +174,7 @@ __device__ __forceinline__ void spmv_long_rows(const CsrView &A, const double *x
 // Rows per group for n rows with nnz entries: one where rows are long on the average (rows
 // side by side would wait for the longest) or where groups of more would leave SMs idle, four where
 // there are warps enough for the FP64 unit to be what bounds it.  Times in us with 1, 2 and 4 (128
-// threads per CTA): 5 entries per row, n = 20000 7.3, 5.3, 5.3, n = 262144 25.8, 15.5, 13.5; 17
+// threads per CTA, launches back to back with gaps of about 1 us): 5 entries per row, n = 20000 7.3, 5.3, 5.3, n = 262144 25.8, 15.5, 13.5; 17
 // per row, 2000 5.3, 5.3, 7.3, 60000 11.4, 9.4, 9.4, 262144 31.9, 22.2, 21.7; power-law
 // rows of 9 on the average, 5000 9.4, 9.4, 9.4, 20000 9.4, 9.4, 11.4, 262144 32.0, 29.8, 30.2;
 // rows of 79, 2000 11.4, 13.5, 17.6, 20000 15.5, 17.6, 22.8, 262144 109, 107, 111.
